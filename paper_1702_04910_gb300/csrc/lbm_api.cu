@@ -72,7 +72,6 @@ struct lbm_handle {
     Coll<double> kd;
     Coll<float> kf;
     Coll<dfloat> kff;
-    Coll<fx64> kfx;
     // learned force correction
     lbm_mlp* model;
     int model_mode;    // 0 off, 1 correct, 2 features only
@@ -144,7 +143,6 @@ Launch base_launch(lbm_handle* h) {
     L.kd = h->kd;
     L.kf = h->kf;
     L.kff = h->kff;
-    L.kfx = h->kfx;
     L.cp.kind = h->kind;
     L.cp.variant = h->variant;
     L.cp.np = h->np;
@@ -450,19 +448,13 @@ lbm_status lbm_create(const lbm_config* cfg, void* stream, lbm_handle** out) {
     g.bc_z = cfg->bc_z;
     g.n = n;
     set_open_boundaries(g, *cfg);
-    g.tx = cfg->nx >= 128 ? 128 : (cfg->nx >= 64 ? 64 : 32);
-    g.ty = 256 / g.tx;
-    g.ntx = (cfg->nx + g.tx - 1) / g.tx;
-    g.nty = (cfg->ny + g.ty - 1) / g.ty;
-    g.tz = cfg->storage == LBM_STORE_F32 ? 2 : 1;  // two z cells per thread (k_bulk)
-    g.ntz = (cfg->nz + g.tz - 1) / g.tz;
+    set_tiles(g, cfg->storage);
 
     const double lp = -1.0 / cfg->tau;
     const double lm = cfg->collision == LBM_TRT ? 1.0 / (cfg->magic / (0.5 + 1.0 / lp) - 0.5) : lp;
     h->kd = make_coll<double>(lp, lm, cfg->rho0, cfg->force_density);
     h->kf = make_coll<float>(lp, lm, cfg->rho0, cfg->force_density);
     h->kff = make_coll<dfloat>(lp, lm, cfg->rho0, cfg->force_density);
-    h->kfx = make_coll<fx64>(lp, lm, cfg->rho0, cfg->force_density);
 
     size_t bytes = (size_t)NQ * (size_t)n * h->esize;
     cudaError_t e = cudaMalloc(&h->buf[0], bytes);

@@ -54,7 +54,6 @@ struct WorkList {
 
 struct lbm_batch {
     int n;
-    int mode;  // bulk collision arithmetic: 0 FP64, 3 fixed point
     cudaStream_t stream;
     cudaStream_t cap, side;
     cudaEvent_t ev_fork, ev_join, t0, t1;
@@ -209,7 +208,7 @@ cudaError_t enqueue_step(lbm_batch* b, int* kernels) {
             e = launch_stamp(b->dprof, 0, s);
             ++k;
         }
-        if (e == cudaSuccess) e = launch_batch_bulk(b->mode, b->dcases, bl.view(), bl.total, b->grid, b->dstatus, s);
+        if (e == cudaSuccess) e = launch_batch_bulk(b->dcases, bl.view(), bl.total, b->grid, b->dstatus, s);
         if (e == cudaSuccess && b->profiling) {
             e = launch_stamp(b->dprof, 1, s);
             ++k;
@@ -346,7 +345,6 @@ lbm_status make_case(lbm_batch* b, int c, const lbm_config& cfg, const lbm_parti
     k.cp.rho0 = cfg.rho0;
     k.cp.mr_cpc = cfg.coupling == LBM_MEM_MR ? mr_correction_scale(cfg) : 0.0;
     k.kd = make_coll<double>(lp, lm, cfg.rho0, cfg.force_density);
-    k.kfx = make_coll<fx64>(lp, lm, cfg.rho0, cfg.force_density);
     region_extent(g, p.diameter, k.map_ext);
     near_grid(g, p.diameter, k.box);
     k.nblk = near_blocks(k.box);
@@ -395,10 +393,10 @@ void release(lbm_batch* b) {
 // the given grid.  src = buf[cur], dst = buf[1 - cur]: the next sweep
 // overwrites every cell this writes, so the simulation state is unchanged.
 lbm_status time_bulk(lbm_batch* b, const WorkList& w, int grid, int reps, double* ms) {
-    BK(b, launch_batch_bulk(b->mode, b->dcases, w.view(), w.total, grid, b->dstatus, b->stream), "tuning launch");
+    BK(b, launch_batch_bulk(b->dcases, w.view(), w.total, grid, b->dstatus, b->stream), "tuning launch");
     BK(b, cudaEventRecord(b->t0, b->stream), "event record");
     for (int r = 0; r < reps; ++r)
-        BK(b, launch_batch_bulk(b->mode, b->dcases, w.view(), w.total, grid, b->dstatus, b->stream),
+        BK(b, launch_batch_bulk(b->dcases, w.view(), w.total, grid, b->dstatus, b->stream),
            "tuning launch");
     BK(b, cudaEventRecord(b->t1, b->stream), "event record");
     BK(b, cudaEventSynchronize(b->t1), "event sync");
@@ -430,7 +428,6 @@ lbm_status lbm_batch_create(int n_cases, const lbm_config* cfgs, const lbm_parti
     lbm_batch* b = new (std::nothrow) lbm_batch();
     if (!b) return LBM_ERR_OOM;
     b->n = n_cases;
-    b->mode = storage == LBM_STORE_F64_FX ? 3 : 0;
     b->stream = (cudaStream_t)stream;
     b->cfg.assign(cfgs, cfgs + n_cases);
     b->hc.resize(n_cases);
@@ -587,7 +584,7 @@ lbm_status lbm_batch_create(int n_cases, const lbm_config* cfgs, const lbm_parti
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        b->resident = std::max(sms, 1) * batch_bulk_blocks_per_sm(b->mode);
+        b->resident = std::max(sms, 1) * batch_bulk_blocks_per_sm();
         b->grid = 0;
         st = build_graph(b);
     }

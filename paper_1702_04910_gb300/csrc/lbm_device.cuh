@@ -17,6 +17,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "lbm_fixed.cuh"
 
 namespace lbmgpu {
@@ -76,16 +78,18 @@ struct Geom {
     double fhalf[3];    // f_ext / (2 rho0): Eq. (8) velocity = j~/rho0 - fhalf
 };
 
-// Collision constants in the arithmetic type C.
+// Collision constants in the arithmetic type C; FP64 also carries those of the
+// fixed-point form (lbm_fixed.cuh).
+template <typename C> struct CollExtra {};
+template <> struct CollExtra<double> { FixColl fix; };
 template <typename C>
-struct Coll {
+struct Coll : CollExtra<C> {
     C lam_p, lam_m;   // lambda_+ = -1/tau, lambda_- from Eq. (11)
     C rho0, inv_rho0;
     C fx, fy, fz;     // f_ext
     int has_force;
     // folded constants of the pair update (see collide_fluid)
     C alpha, beta;    // 1 + (l+ + l-)/2, (l+ - l-)/2
-    C hs, hd;         // (alpha + beta)/2 = (1 + l+)/2, (alpha - beta)/2 = (1 + l-)/2
     C c0;             // 1 + l+
     C m15r0;          // -3/2 / rho0 (multiplies j.j, j = rho0 U)
     C lpw[3];         // l+ w_k, k = rest, axis, diagonal
@@ -542,11 +546,6 @@ __device__ __forceinline__ void moments_j(const C (&f)[NQ], C& rho, C& jx, C& jy
 //   f_qbar' = alpha f_qbar + beta f_q    - (P - M)
 // with P = l+ f^eq,+ - F^+ and M = l- f^eq,- - F^-, which expands
 // f_q + l+ (f_q^+ - f^eq,+) + l- (f_q^- - f^eq,-) + F_q exactly.
-// Arithmetic whose products cost far more than its sums (the 64-bit fixed
-// point) takes the pair update in sum / difference form,
-//   f_q' = hs (f_q + f_qbar) + hd (f_q - f_qbar) - (P + M),
-//   f_qbar' = hs (f_q + f_qbar) - hd (f_q - f_qbar) - (P - M):
-// two products per pair instead of four (PairSumDiff, lbm_fixed.cuh).
 // C is the arithmetic type, KT the type of the constants (C itself, or float
 // for the packed f2: C(k.x) broadcasts a constant to both lanes).
 template <typename C, int Q, int K, bool FORCE, typename KT>
@@ -556,25 +555,8 @@ __device__ __forceinline__ void trt_pair(C (&f)[NQ], C cu, const C (&bw)[3], con
                 : fma(C(k.k1w[K]), cu * cu, bw[K]);
     C M = FORCE ? fma(C(k.k2w[K]), cu, C(-k.fq[(Q - 1) / 2])) : C(k.k2w[K]) * cu;
     const C a = f[Q], b = f[QB];
-    if constexpr (PairSumDiff<C>::value) {
-        const C sp = k.hs * (a + b), sd = k.hd * (a - b);
-        f[Q] = (sp + sd) - (P + M);
-        f[QB] = (sp - sd) - (P - M);
-    } else {
-        f[Q] = fma(C(k.alpha), a, fma(C(k.beta), b, -(P + M)));
-        f[QB] = fma(C(k.alpha), b, fma(C(k.beta), a, -(P - M)));
-    }
-}
-
-// Sum / difference pair update with P given (see trt_pair).
-template <typename C, int Q, int K>
-__device__ __forceinline__ void trt_pair_sd(C (&f)[NQ], C cu, C P, const Coll<C>& k) {
-    constexpr int QB = Q + 1;
-    const C M = k.k2w[K] * cu;
-    const C a = f[Q], b = f[QB];
-    const C sp = k.hs * (a + b), sd = k.hd * (a - b);
-    f[Q] = (sp + sd) - (P + M);
-    f[QB] = (sp - sd) - (P - M);
+    f[Q] = fma(C(k.alpha), a, fma(C(k.beta), b, -(P + M)));
+    f[QB] = fma(C(k.alpha), b, fma(C(k.beta), a, -(P - M)));
 }
 
 // Two FP32 lanes in one register pair, for the Blackwell packed f32x2
@@ -608,13 +590,6 @@ __device__ __forceinline__ bool density_bad(float r) {
 __device__ __forceinline__ unsigned density_bad(f2 r) {
     return (density_bad(r.v.x) ? 1u : 0u) | (density_bad(r.v.y) ? 2u : 0u);
 }
-// fixed point cannot hold NaN (the conversion from FP64 turns a non-finite
-// value into 0); a saturated conversion or a wrapped sum shows as a density
-// outside (0, 16)
-__device__ __forceinline__ bool density_bad(fx64 r) {
-    return !(r.v > 0 && r.v < (16LL << FX_SHIFT));
-}
-
 // Returns true when the cell's density is not finite and positive.
 // SHIFTED: f holds the shifted populations f_q - w_q, whose sum is rho - 1.
 // Written in j = rho0 U (ux, uy, uz below hold j); the constants k1w, k2w,
@@ -626,29 +601,6 @@ __device__ __forceinline__ auto collide_fluid_t(C (&f)[NQ], const Coll<KT>& k) {
     C rho, ux, uy, uz;
     moments_j(f, rho, ux, uy, uz);
     const auto bad = SHIFTED ? density_bad(rho + C(1)) : density_bad(rho);
-    if constexpr (PairSumDiff<C>::value && !FORCE) {
-        // products shared between pairs: with t_a = k1w_diag u_a^2 and
-        // c_ab = k1w_axis u_a u_b (k1w_axis = 2 k1w_diag), the quadratic term
-        // of P is 2 t_a on an axis pair and t_a + t_b +- c_ab on a diagonal one
-        const C xx = ux * ux, yy = uy * uy, zz = uz * uz;
-        const C base = fma(k.m15r0, (xx + yy) + zz, rho);
-        C bw[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) bw[c] = k.lpw[c] * base;
-        const C tx = k.k1w[2] * xx, ty = k.k1w[2] * yy, tz = k.k1w[2] * zz;
-        const C cxy = k.k1w[1] * (ux * uy), cxz = k.k1w[1] * (ux * uz), cyz = k.k1w[1] * (uy * uz);
-        f[0] = fma(k.c0, f[0], -bw[0]);
-        trt_pair_sd<C, 1, 1>(f, ux, (tx + tx) + bw[1], k);
-        trt_pair_sd<C, 3, 1>(f, uy, (ty + ty) + bw[1], k);
-        trt_pair_sd<C, 5, 1>(f, uz, (tz + tz) + bw[1], k);
-        trt_pair_sd<C, 7, 2>(f, ux + uy, ((tx + ty) + cxy) + bw[2], k);
-        trt_pair_sd<C, 9, 2>(f, ux - uy, ((tx + ty) - cxy) + bw[2], k);
-        trt_pair_sd<C, 11, 2>(f, ux + uz, ((tx + tz) + cxz) + bw[2], k);
-        trt_pair_sd<C, 13, 2>(f, ux - uz, ((tx + tz) - cxz) + bw[2], k);
-        trt_pair_sd<C, 15, 2>(f, uy + uz, ((ty + tz) + cyz) + bw[2], k);
-        trt_pair_sd<C, 17, 2>(f, uy - uz, ((ty + tz) - cyz) + bw[2], k);
-        return bad;
-    }
     const C uu = fma(ux, ux, fma(uy, uy, uz * uz));
     const C base = fma(C(k.m15r0), uu, rho);
     C bw[3];
@@ -681,6 +633,19 @@ template <typename C, bool SHIFTED = false, typename KT>
 __device__ __forceinline__ auto collide_fluid(C (&f)[NQ], const Coll<KT>& k) {
     if (k.has_force) return collide_fluid_t<C, true, SHIFTED>(f, k);
     return collide_fluid_t<C, false, SHIFTED>(f, k);
+}
+
+// The same for a cell of any storage: FP64 populations take the fixed-point
+// form where it holds (lbm_fixed.cuh), the FP64 form elsewhere.
+template <typename C>
+__device__ __forceinline__ bool collide_cell(C (&f)[NQ], const Coll<C>& k) {
+    if constexpr (std::is_same<C, double>::value) {
+        if (k.fix.on) {
+            if (k.has_force ? fixed_collide_t<true>(f, k.fix) : fixed_collide_t<false>(f, k.fix))
+                return false;
+        }
+    }
+    return collide_fluid(f, k);
 }
 
 // Collision operator values C_q (Eq. (5)/(9)) and forcing F_q (Eq. (7)) as

@@ -23,6 +23,7 @@
 #include <cuda_runtime.h>
 
 #include <type_traits>
+#include <utility>
 
 #include "lbm_launch.h"
 
@@ -492,9 +493,17 @@ __device__ inline bool psm_collide(C (&f)[NQ], const Coll<C>& k, const Coupl& cp
 // ---------------------------------------------------------------------------
 // bulk sweep: every cell outside the near-particle regions.  Tiles that no
 // region touches skip the per-cell test (block-uniform branch).
-// Resident 256-thread blocks per SM requested for k_bulk (at most 85
-// registers per thread).
-template <typename C> struct BulkBlocks { static constexpr int value = 3; };
+// Threads per block and resident blocks per SM of k_bulk by stored type and
+// arithmetic (the host's tiles, set_tiles in lbm_launch.h, follow).  FP64:
+// 5 x 128 threads leave the fixed-point collision its 96 registers without
+// spills and 20 warps per SM (128 x 128 x 512 cells, FP64 settling step of 2
+// sweeps: 256 x 3, 80 registers, 1.27 ms; 256 x 2, 128 registers, 1.38;
+// 128 x 4 1.29; 128 x 5 1.09; 128 x 6 1.21; 128 x 7 1.18).  16 bits, one
+// cell per thread: 128 threads balance the last wave better (101 x 101 x 304
+// cells, frame step 296 -> 259 us).  FP32 keeps 256 (0.5 % faster).
+template <typename T, typename C> struct BulkShape { static constexpr int threads = 128, blocks = 6; };
+template <> struct BulkShape<double, double> { static constexpr int threads = 128, blocks = 5; };
+template <> struct BulkShape<float, float> { static constexpr int threads = 256, blocks = 3; };
 
 // One tile (tX, tY, tZ) of the bulk sweep for the calling thread (tx, ty).
 template <typename T, typename C, bool NOSTREAM, int CPT>
@@ -534,14 +543,14 @@ __device__ __forceinline__ void bulk_tile(const T* __restrict__ src, T* __restri
     for (int c = 0; c < CPT; ++c) {
         if (!act[c]) continue;
         const int z = tZ * CPT + c;
-        bad |= collide_fluid(f[c], k);
+        bad |= collide_cell(f[c], k);
         store_own(dst, g, lin(g, x, y, z), f[c]);
     }
     if (bad) atomicOr(status, ST_FLUID);
 }
 
 template <typename T, typename C, bool NOSTREAM, int CPT>
-__global__ void __launch_bounds__(256, BulkBlocks<C>::value)
+__global__ void __launch_bounds__(BulkShape<T, C>::threads, BulkShape<T, C>::blocks)
     k_bulk(const T* __restrict__ src, T* __restrict__ dst, Geom g, Coll<C> k,
            const DevParticle* __restrict__ parts, int np, int all_tiles, int* __restrict__ status) {
     bulk_tile<T, C, NOSTREAM, CPT>(src, dst, g, k, parts, np, all_tiles, blockIdx.x, blockIdx.y,
@@ -1497,17 +1506,6 @@ __device__ __forceinline__ int find_item(const long long* __restrict__ base, int
     return lo;
 }
 
-template <typename C>
-__device__ __forceinline__ const Coll<C>& batch_coll(const BatchCase& B);
-template <>
-__device__ __forceinline__ const Coll<double>& batch_coll<double>(const BatchCase& B) {
-    return B.kd;
-}
-template <>
-__device__ __forceinline__ const Coll<fx64>& batch_coll<fx64>(const BatchCase& B) {
-    return B.kfx;
-}
-
 // cell and tile ranges of each case's particle (after upload or a change of
 // the bulk tiling); the previous state starts equal to the current one
 __global__ void k_batch_regions(BatchCase* __restrict__ cases, int n) {
@@ -1579,60 +1577,71 @@ __global__ void __launch_bounds__(256)
                                              lw);
 }
 
-// One 256-cell segment of an xy plane of the bulk sweep: cells
-// l = seg * 256 + t (x fastest) of plane z.  Domains whose nx is not a
-// multiple of the warp width keep every lane busy (box tiles of tx cells
-// leave tx - nx mod tx lanes of each row idle).
-template <typename C>
-__device__ __forceinline__ void bulk_segment(const double* __restrict__ src,
-                                             double* __restrict__ dst, const Geom& g,
-                                             const Coll<C>& k, const int* reg, int seg, int z,
-                                             int t, int* __restrict__ status) {
-    const int l = seg * 256 + t;
-    if (l >= g.nx * g.ny) return;
-    const int y = l / g.nx, x = l - y * g.nx;
-    if (cell_in_reg(g, reg, x, y, z)) return;  // k_batch_near's cell
-    const long long idx = lin(g, x, y, z);
-    C f[NQ];
-    pull_plain(src, g, x, y, z, idx, f);
-    if (collide_fluid(f, k)) atomicOr(status, ST_FLUID);
-    store_own(dst, g, idx, f);
-}
+// Threads of a k_batch_bulk block and its resident blocks per SM; a work item
+// is 256 cells, so each thread takes BATCH_ITEM / BATCH_THREADS of them.
+constexpr int BATCH_ITEM = 256, BATCH_THREADS = 128, BATCH_BLOCKS = 5;
 
-// One tile of case B in its bulk layout (see k_batch_bulk).
-template <typename C>
-__device__ __forceinline__ void batch_tile(const BatchCase& B, long long local,
-                                           int* __restrict__ status) {
-    const int cur = B.cur;
-    if (B.layout == 1) {
-        const int nseg = (B.g.nx * B.g.ny + 255) / 256;
-        bulk_segment<C>(B.buf[cur], B.buf[1 - cur], B.g, batch_coll<C>(B), B.part->reg,
-                        (int)(local % nseg), (int)(local / nseg), threadIdx.x, status);
-    } else {
-        const int tX = (int)(local % B.g.ntx);
-        const int tY = (int)((local / B.g.ntx) % B.g.nty);
-        const int tZ = (int)(local / ((long long)B.g.ntx * B.g.nty));
-        bulk_tile<double, C, false, 1>(B.buf[cur], B.buf[1 - cur], B.g, batch_coll<C>(B), B.part, 1,
-                                       0, tX, tY, tZ, threadIdx.x % B.g.tx, threadIdx.x / B.g.tx,
-                                       status);
+// Cell (x, y, z) of an item's thread slot t: false beyond the lattice.  Plane
+// segments (layout 1) are 256 consecutive cells of an xy plane, so domains
+// whose nx is not a multiple of the warp width keep every lane busy; box
+// tiles of g.tx cells leave g.tx - nx mod g.tx lanes of each row idle.
+__device__ __forceinline__ bool batch_cell(const Geom& g, int layout, long long local, int t,
+                                           int& x, int& y, int& z) {
+    if (layout == 1) {
+        const int nseg = (g.nx * g.ny + BATCH_ITEM - 1) / BATCH_ITEM;
+        z = (int)(local / nseg);
+        const int l = ((int)local - z * nseg) * BATCH_ITEM + t;
+        y = l / g.nx;
+        x = l - y * g.nx;
+        return l < g.nx * g.ny;
     }
+    const int tX = (int)(local % g.ntx), tY = (int)((local / g.ntx) % g.nty);
+    z = (int)(local / ((long long)g.ntx * g.nty));
+    x = tX * g.tx + t % g.tx;
+    y = tY * g.ty + t / g.tx;
+    return x < g.nx && y < g.ny;
 }
 
-// bulk sweep: persistent 256-thread blocks striding over the tiles of all
+// bulk sweep: persistent blocks striding over the 256-cell items of all
 // listed cases.  Each case has its own tiling (B.layout, chosen by the
-// autotuner): 0 box tiles of g.tx x g.ty cells (thread t -> (t mod g.tx,
-// t / g.tx)); 1 plane segments of 256 cells.  MODE: 0 FP64, 3 fixed-point
-// collision.
-template <int MODE>
-__global__ void __launch_bounds__(256, 3)
+// autotuner): 0 box tiles of g.tx x g.ty cells; 1 plane segments.  The case
+// record is staged in shared memory once per item: its collision constants
+// are read ~60 times per cell, and as global loads they cost the registers
+// that the cell's 19 values need (12 cases of D = 8..16, 6.8 M cells, 3 steps:
+// constants from global memory, 256 threads, 1 KB of spills 4.10 ms; staged,
+// 128 threads, 3.87 ms; the FP64 form 10.08 ms).
+__global__ void __launch_bounds__(BATCH_THREADS, BATCH_BLOCKS)
     k_batch_bulk(BatchCase* __restrict__ cases, BatchList l, long long total,
                  int* __restrict__ status) {
+    __shared__ BatchCase B;
+    __shared__ int reg[12];
+    int held = -1;
     for (long long t = blockIdx.x; t < total; t += gridDim.x) {
         const int i = find_item(l.base, l.n, t);
-        const BatchCase& B = cases[l.list[i]];
-        const long long local = t - l.base[i];
-        if (MODE == 3) batch_tile<fx64>(B, local, status);
-        else batch_tile<double>(B, local, status);
+        const int c = l.list[i];
+        if (c != held) {
+            __syncthreads();
+            const BatchCase* G = cases + c;
+            for (int k = threadIdx.x; k < (int)(sizeof(BatchCase) / 8); k += BATCH_THREADS)
+                reinterpret_cast<long long*>(&B)[k] = reinterpret_cast<const long long*>(G)[k];
+            if (threadIdx.x < 12) reg[threadIdx.x] = G->part->reg[threadIdx.x];
+            __syncthreads();
+            held = c;
+        }
+        const double* src = B.buf[B.cur];
+        double* dst = B.buf[1 - B.cur];
+        bool bad = false;
+        for (int s = threadIdx.x; s < BATCH_ITEM; s += BATCH_THREADS) {
+            int x, y, z;
+            if (!batch_cell(B.g, B.layout, t - l.base[i], s, x, y, z)) continue;
+            if (cell_in_reg(B.g, reg, x, y, z)) continue;  // k_batch_near's cell
+            const long long idx = lin(B.g, x, y, z);
+            double f[NQ];
+            pull_plain(src, B.g, x, y, z, idx, f);
+            bad |= collide_cell(f, B.kd);
+            store_own(dst, B.g, idx, f);
+        }
+        if (bad) atomicOr(status, ST_FLUID);
     }
 }
 
@@ -1701,6 +1710,30 @@ __global__ void k_batch_charge_total(BatchCase* __restrict__ cases, int n) {
 // ---------------------------------------------------------------------------
 // launchers
 namespace {
+// Launch with one common split of the SM's 256 KB between L1 and shared memory.
+// The near sweep needs up to 24 KB of shared memory per block and runs beside
+// the bulk sweep, which needs none.  Left to the default, a bulk block puts its
+// SM in the all-L1 split, and near blocks cannot start there until the SM has
+// drained.  Measured (us per pass, default / 25 / 50 / 100 % of the largest
+// shared-memory size): 24 x 24 x 40 cells FP64, 20 steps 3210 / 2340 / 2330 /
+// 2390; 32^3 FP64, 50 steps 3950 / 3370 / 3370 / 3470; 128 x 128 x 512 FP32, 8
+// steps of 2 sweeps 5090 / 5090 / 4900 / 5690; FP16, 20 steps 3090 / 2980 /
+// 2980 / 3110.
+constexpr int SMEM_CARVEOUT = 50;  // percent of the largest shared-memory size
+template <typename... P, typename... A>
+cudaError_t launch(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t s, A&&... args) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    at[0].val.sharedMemCarveout = SMEM_CARVEOUT;
+    c.attrs = at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, std::forward<A>(args)...);
+}
+
 template <typename T, typename C>
 const Coll<C>& coll_of(const Launch& L);
 template <>
@@ -1715,22 +1748,16 @@ template <>
 const Coll<dfloat>& coll_of<double, dfloat>(const Launch& L) {
     return L.kff;
 }
-template <>
-const Coll<fx64>& coll_of<double, fx64>(const Launch& L) {
-    return L.kfx;
-}
 
 template <typename T, typename C, int CPT>
 cudaError_t bulk_cpt(const void* src, void* dst, const Launch& L) {
     dim3 grid(L.g.ntx, L.g.nty, L.g.ntz);
     const auto& k = coll_of<typename std::conditional<(sizeof(T) < 4), C, T>::type, C>(L);
     if (L.nostream)
-        k_bulk<T, C, true, CPT><<<grid, L.block, 0, L.stream>>>(
-            (const T*)src, (T*)dst, L.g, k, L.parts, L.cp.np, L.all_tiles, L.status);
-    else
-        k_bulk<T, C, false, CPT><<<grid, L.block, 0, L.stream>>>(
-            (const T*)src, (T*)dst, L.g, k, L.parts, L.cp.np, L.all_tiles, L.status);
-    return cudaGetLastError();
+        return launch(k_bulk<T, C, true, CPT>, grid, L.block, L.stream, (const T*)src, (T*)dst, L.g,
+                      k, L.parts, L.cp.np, L.all_tiles, L.status);
+    return launch(k_bulk<T, C, false, CPT>, grid, L.block, L.stream, (const T*)src, (T*)dst, L.g, k,
+                  L.parts, L.cp.np, L.all_tiles, L.status);
 }
 
 // FP64-state sweeps are arithmetic bound and use one cell per thread; the
@@ -1743,9 +1770,8 @@ cudaError_t bulk_t(const void* src, void* dst, const Launch& L) {
         if (!L.nostream && L.g.nx % 2 == 0 && L.g.bc_z != 2) {
             dim3 grid((L.g.nx + 2 * PAIR_TX - 1) / (2 * PAIR_TX), (L.g.ny + PAIR_TY - 1) / PAIR_TY,
                       L.g.nz);
-            k_bulk_pair<T><<<grid, dim3(PAIR_TX, PAIR_TY, 1), 0, L.stream>>>(
-                (const T*)src, (T*)dst, L.g, L.kf, L.parts, L.all_tiles ? 0 : L.cp.np, L.status);
-            return cudaGetLastError();
+            return launch(k_bulk_pair<T>, grid, dim3(PAIR_TX, PAIR_TY, 1), L.stream, (const T*)src,
+                          (T*)dst, L.g, L.kf, L.parts, L.all_tiles ? 0 : L.cp.np, L.status);
         }
     }
     if constexpr (sizeof(T) <= 4) {
@@ -1762,12 +1788,10 @@ cudaError_t near_kind(const void* src, void* dst, const Launch& L) {
     const auto& k = coll_of<C, C>(L);
     const GeoMap gm{L.map, L.map_ext[0], L.map_ext[1], L.map_ext[2]};
     if (L.nostream)
-        k_near<T, C, KIND, true><<<grid, block, 0, L.stream>>>(
-            (const T*)src, (T*)dst, L.g, k, L.cp, L.parts, gm, L.partials, L.status, L.box[2]);
-    else
-        k_near<T, C, KIND, false><<<grid, block, 0, L.stream>>>(
-            (const T*)src, (T*)dst, L.g, k, L.cp, L.parts, gm, L.partials, L.status, L.box[2]);
-    return cudaGetLastError();
+        return launch(k_near<T, C, KIND, true>, grid, block, L.stream, (const T*)src, (T*)dst, L.g, k,
+                      L.cp, L.parts, gm, L.partials, L.status, L.box[2]);
+    return launch(k_near<T, C, KIND, false>, grid, block, L.stream, (const T*)src, (T*)dst, L.g, k,
+                  L.cp, L.parts, gm, L.partials, L.status, L.box[2]);
 }
 
 template <typename T>
@@ -1785,10 +1809,8 @@ cudaError_t refill_t(const void* srcB, void* dst, const Launch& L, const DevPart
     if (L.cp.np <= 0) return cudaSuccess;
     int side = L.box[0];  // set by the caller: cube side in cells
     dim3 grid((unsigned)refill_blocks(side), L.cp.np, 1);
-    k_refill<T, C><<<grid, REFILL_THREADS, 0, L.stream>>>((const T*)srcB, (T*)dst, L.g, coll_of<C, C>(L),
-                                                L.cp, po, pn, extrapolate, side, L.status,
-                                                charge_part);
-    return cudaGetLastError();
+    return launch(k_refill<T, C>, grid, REFILL_THREADS, L.stream, (const T*)srcB, (T*)dst, L.g,
+                  coll_of<C, C>(L), L.cp, po, pn, extrapolate, side, L.status, charge_part);
 }
 
 template <typename T>
@@ -1835,7 +1857,6 @@ cudaError_t from_f64_t(const double* in, void* dst, long long count, long long n
 cudaError_t launch_bulk(int storage, const void* src, void* dst, const Launch& L) {
     switch (storage) {
         case 2: return bulk_t<double, dfloat>(src, dst, L);
-        case 3: return bulk_t<double, fx64>(src, dst, L);
         case 1: return bulk_t<float>(src, dst, L);
         case 4: return bulk_t<__half, float>(src, dst, L);
         case 5: return bulk_t<__nv_bfloat16, float>(src, dst, L);
@@ -1863,9 +1884,8 @@ cudaError_t launch_refill(int storage, const void* srcB, void* dst, const Launch
 }
 cudaError_t launch_charge_total(const Launch& L, const double* charge_part, double* charge) {
     if (L.cp.np <= 0) return cudaSuccess;
-    k_charge_total<<<1, 6 * MAX_PARTICLES, 0, L.stream>>>(L.cp.np, refill_blocks(L.box[0]),
-                                                          charge_part, charge);
-    return cudaGetLastError();
+    return launch(k_charge_total, 1, 6 * MAX_PARTICLES, L.stream, L.cp.np, refill_blocks(L.box[0]),
+                  charge_part, charge);
 }
 cudaError_t launch_macro(int storage, const void* state, const Launch& L, int what, void* out) {
     switch (storage) {
@@ -1908,31 +1928,26 @@ cudaError_t launch_map(const Launch& L) {
     if (L.cp.np <= 0 || L.cp.kind == 0) return cudaSuccess;
     dim3 grid((L.map_ext[0] + 31) / 32, L.map_ext[1], L.map_ext[2] * L.cp.np);
     if (L.cp.kind == 2)
-        k_map<2><<<grid, 32, 0, L.stream>>>(L.g, L.cp, L.parts, L.map, L.map_ext[0], L.map_ext[1],
-                                            L.map_ext[2]);
-    else
-        k_map<1><<<grid, 32, 0, L.stream>>>(L.g, L.cp, L.parts, L.map, L.map_ext[0], L.map_ext[1],
-                                            L.map_ext[2]);
-    return cudaGetLastError();
+        return launch(k_map<2>, grid, 32, L.stream, L.g, L.cp, L.parts, L.map, L.map_ext[0],
+                      L.map_ext[1], L.map_ext[2]);
+    return launch(k_map<1>, grid, 32, L.stream, L.g, L.cp, L.parts, L.map, L.map_ext[0], L.map_ext[1],
+                  L.map_ext[2]);
 }
 
 cudaError_t launch_finalize(const Launch& L, int nsub, double* force_out, const double* charge) {
     if (L.cp.np <= 0) return cudaSuccess;
-    k_finalize<<<L.cp.np, 256, 0, L.stream>>>(L.cp.np, near_blocks(L.box), L.partials, nsub,
-                                               force_out, charge);
-    return cudaGetLastError();
+    return launch(k_finalize, L.cp.np, 256, L.stream, L.cp.np, near_blocks(L.box), L.partials, nsub,
+                  force_out, charge);
 }
 cudaError_t launch_rigid_body(const Launch& L, const double* force, double gx, double gy,
                               double gz, double dt, int wall_contact) {
     if (L.cp.np <= 0) return cudaSuccess;
-    k_rigid<<<1, 32, 0, L.stream>>>(L.g, L.parts, L.parts_prev, L.cp.np, force, L.kd.rho0, gx, gy,
-                                    gz, dt, wall_contact, L.status);
-    return cudaGetLastError();
+    return launch(k_rigid, 1, 32, L.stream, L.g, L.parts, L.parts_prev, L.cp.np, force, L.kd.rho0, gx,
+                  gy, gz, dt, wall_contact, L.status);
 }
 cudaError_t launch_regions(const Launch& L) {
     if (L.cp.np <= 0) return cudaSuccess;
-    k_regions<<<1, 32, 0, L.stream>>>(L.g, L.parts, L.cp.np);
-    return cudaGetLastError();
+    return launch(k_regions, 1, 32, L.stream, L.g, L.parts, L.cp.np);
 }
 
 
@@ -1956,14 +1971,11 @@ cudaError_t launch_batch_near(BatchCase* cases, BatchList l, long long total, in
     k_batch_near<<<(unsigned)total, dim3(NEAR_BX, NEAR_BY, NEAR_BZ), 0, s>>>(cases, l, sub, status);
     return cudaGetLastError();
 }
-cudaError_t launch_batch_bulk(int mode, BatchCase* cases, BatchList l, long long total, int grid,
+cudaError_t launch_batch_bulk(BatchCase* cases, BatchList l, long long total, int grid,
                               int* status, cudaStream_t s) {
     if (l.n == 0 || total == 0) return cudaSuccess;
     const unsigned gsz = (unsigned)(grid <= 0 || total < grid ? total : grid);
-    if (mode == 3)
-        k_batch_bulk<3><<<gsz, 256, 0, s>>>(cases, l, total, status);
-    else
-        k_batch_bulk<0><<<gsz, 256, 0, s>>>(cases, l, total, status);
+    k_batch_bulk<<<gsz, BATCH_THREADS, 0, s>>>(cases, l, total, status);
     return cudaGetLastError();
 }
 cudaError_t launch_batch_swap(BatchCase* cases, BatchList l, cudaStream_t s) {
@@ -2007,12 +2019,9 @@ cudaError_t launch_batch_refill(BatchCase* cases, BatchList l, long long total, 
     k_batch_refill<<<(unsigned)total, REFILL_THREADS, 0, s>>>(cases, l, status);
     return cudaGetLastError();
 }
-int batch_bulk_blocks_per_sm(int mode) {
+int batch_bulk_blocks_per_sm() {
     int nb = 0;
-    if (mode == 3)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch_bulk<3>, 256, 0);
-    else
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch_bulk<0>, 256, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch_bulk, BATCH_THREADS, 0);
     return nb > 0 ? nb : 1;
 }
 

@@ -18,7 +18,6 @@ struct Launch {
     Coll<double> kd;   // FP64 collision constants
     Coll<float> kf;    // FP32 collision constants
     Coll<dfloat> kff;  // float-float collision constants (FP64 storage)
-    Coll<fx64> kfx;    // fixed-point collision constants (FP64 storage)
     Coupl cp;
     DevParticle* parts;       // particle state used by this sweep
     DevParticle* parts_prev;  // state before the last rigid-body update (refill)
@@ -89,7 +88,6 @@ struct BatchCase {
     int wall_contact;
     Coupl cp;          // np = 1
     Coll<double> kd;
-    Coll<fx64> kfx;
     DevParticle* part;
     DevParticle* prev;
     double* force;     // 6 doubles
@@ -104,6 +102,8 @@ struct BatchCase {
     double* charge;       // 6 doubles: pending amounts of the last re-mapping
     double* charge_part;  // refill_blocks(refill_side) x 6 block partials
 };
+
+static_assert(sizeof(BatchCase) % 8 == 0, "staged as 8-byte words");
 
 // Work list of a batched launch: cases list[0..n) with prefix sums base[] of
 // their work items (tiles, blocks or cells).
@@ -134,6 +134,67 @@ inline double mr_correction_scale(const lbm_config& cfg) {
     return -4.0 * Lm / (Lm - 0.5);
 }
 
+// Constants of the fixed-point collision (lbm_fixed.cuh); on = 0 where they
+// do not fit it (forces of a cell's weight, extreme rho0).
+inline FixMul make_fix_mul(double c) {
+    FixMul m{};
+    const unsigned long long K = (unsigned long long)std::llround(std::ldexp(c, 62)) << 2;
+    m.hi = (unsigned)(K >> 32);
+    m.lo = (unsigned)K;
+    m.rnd = 0x80000000ull + m.lo / 2;
+    m.off = (long long)(K >> 2);
+    return m;
+}
+inline void fix_limbs(double x, int& hi, int& lo) {
+    const long long v = std::llround(x);
+    hi = (int)((v + 0x80000000LL) >> 32);
+    lo = (int)(unsigned)(v & 0xFFFFFFFFLL);
+}
+inline FixColl make_fix(double lp, double lm, double rho0, const double fe[3]) {
+    FixColl k{};
+    int sh = 0;
+    double r = std::frexp(rho0, &sh);  // [1/2, 1)
+    if (r > 0.70710678) r *= 0.5;
+    else --sh;
+    r *= 2.0;  // rho0 = r 2^sh, r in [0.707, 1.415)
+    if (sh > 400 || sh < -400 || !(lp > -2.0 && lp < 0.0 && lm > -2.0 && lm < 0.0)) return k;
+    k.unit_rho = r == 1.0;
+    k.e0 = 1017 + sh;
+    const unsigned es = (unsigned)(sh * (1 << 20));
+    k.lim_lo = 0x3F900000u + es;  // 2^-6
+    k.lim0 = 0x3FE80000u + es;    // 3/4
+    k.lima = 0x3FD00000u + es;    // 1/4
+    k.limd = 0x3FC00000u + es;    // 1/8
+    k.out_sub = (FIX_BITS - sh) * (1 << 20);
+    fix_limbs(std::ldexp(1.0 / r, FIX_BITS), k.inv_hi, k.inv_lo);
+    k.p0 = make_fix_mul(-lp / 12.0);
+    k.pa = make_fix_mul(-lp / 36.0);
+    k.pd = make_fix_mul(-lp / 72.0);
+    k.oa = make_fix_mul(-lm / 6.0);
+    k.od = make_fix_mul(-lm / 12.0);
+    double f[3], g[3], gmax = 0.0;
+    for (int a = 0; a < 3; ++a) {
+        f[a] = std::ldexp(fe[a], -sh);
+        g[a] = 2.0 / lp * f[a] / r;
+        gmax = std::fmax(gmax, std::fabs(g[a]));
+        if (!(std::fabs(f[a]) < 0.01)) return k;
+    }
+    if (!(gmax < 0.125)) return k;
+    // g in units 2^-(58 + gs), the largest component in [2^55, 2^57)
+    while (k.gs < 62 && std::ldexp(gmax, k.gs) < 0.125) ++k.gs;
+    for (int a = 0; a < 3; ++a) fix_limbs(std::ldexp(g[a], FIX_BITS + k.gs), k.g_hi[a], k.g_lo[a]);
+    for (int q = 1; q < NQ; q += 2) {
+        // o - F_q^-: the integer part of F_q^- joins off, the fraction rnd
+        const FixMul& m = q <= 6 ? k.oa : k.od;
+        const double F = std::ldexp(3.0 * wq(q) * (cx(q) * f[0] + cy(q) * f[1] + cz(q) * f[2]), FIX_BITS);
+        const double up = std::ceil(F);
+        k.o_off[(q - 1) / 2] = m.off + (long long)up;
+        k.o_rnd[(q - 1) / 2] = m.rnd + (unsigned long long)std::ldexp(up - F, 32);
+    }
+    k.on = 1;
+    return k;
+}
+
 template <typename C>
 inline Coll<C> make_coll(double lp, double lm, double rho0, const double fe[3]) {
     Coll<C> k{};
@@ -147,8 +208,6 @@ inline Coll<C> make_coll(double lp, double lm, double rho0, const double fe[3]) 
     k.has_force = (fe[0] != 0.0 || fe[1] != 0.0 || fe[2] != 0.0);
     k.alpha = (C)(1.0 + 0.5 * (lp + lm));
     k.beta = (C)(0.5 * (lp - lm));
-    k.hs = (C)(0.5 * (1.0 + lp));
-    k.hd = (C)(0.5 * (1.0 + lm));
     k.c0 = (C)(1.0 + lp);
     k.m15r0 = (C)(-1.5 / rho0);
     const double w[3] = {1.0 / 3.0, 1.0 / 18.0, 1.0 / 36.0};
@@ -163,6 +222,7 @@ inline Coll<C> make_coll(double lp, double lm, double rho0, const double fe[3]) 
         k.gq[(q - 1) / 2] = (C)(9.0 * wq(q) * cf / rho0);
         k.fq[(q - 1) / 2] = (C)(3.0 * wq(q) * cf);
     }
+    if constexpr (std::is_same<C, double>::value) k.fix = make_fix(lp, lm, rho0, fe);
     return k;
 }
 
@@ -195,6 +255,19 @@ inline lbm_status check_config(const lbm_config& c) {
     }
     if (c.coupling == LBM_MEM_MR && !mr_supported(c)) return LBM_ERR_UNSUPPORTED;
     return LBM_OK;
+}
+
+// Bulk tiles of a handle's lattice: one tile is one block of k_bulk
+// (BulkShape), a row or more of one z plane; FP32 takes two planes per thread.
+inline void set_tiles(Geom& g, int storage) {
+    const int threads = storage == LBM_STORE_F32 ? 256 : 128;
+    g.tx = g.nx >= 128 ? 128 : (g.nx >= 64 ? 64 : 32);
+    while (g.tx > 8 && (long long)g.ny * g.tx > 65535LL * threads) g.tx /= 2;  // grid y limit
+    g.ty = threads / g.tx;
+    g.ntx = (g.nx + g.tx - 1) / g.tx;
+    g.nty = (g.ny + g.ty - 1) / g.ty;
+    g.tz = storage == LBM_STORE_F32 ? 2 : 1;
+    g.ntz = (g.nz + g.tz - 1) / g.tz;
 }
 
 // Open-boundary data of a configuration (bc_z = 2) into the geometry.
@@ -252,8 +325,8 @@ cudaError_t launch_batch_regions(BatchCase* cases, int n, cudaStream_t s);
 cudaError_t launch_batch_map(BatchCase* cases, BatchList l, long long total, cudaStream_t s);
 cudaError_t launch_batch_near(BatchCase* cases, BatchList l, long long total, int sub,
                               int* status, cudaStream_t s);
-// mode 0 FP64 / 3 fixed-point collision; grid <= 0: one block per tile
-cudaError_t launch_batch_bulk(int mode, BatchCase* cases, BatchList l, long long total, int grid,
+// grid <= 0: one block per tile
+cudaError_t launch_batch_bulk(BatchCase* cases, BatchList l, long long total, int grid,
                               int* status, cudaStream_t s);
 cudaError_t launch_batch_swap(BatchCase* cases, BatchList l, cudaStream_t s);
 cudaError_t launch_batch_finalize(BatchCase* cases, int n, cudaStream_t s);
@@ -266,7 +339,7 @@ cudaError_t launch_batch_charge_total(BatchCase* cases, int n, cudaStream_t s);
 cudaError_t launch_batch_refill(BatchCase* cases, BatchList l, long long total, int* status,
                                 cudaStream_t s);
 cudaError_t launch_batch_init(BatchCase* cases, int n, long long max_cells, cudaStream_t s);
-int batch_bulk_blocks_per_sm(int mode);
+int batch_bulk_blocks_per_sm();
 cudaError_t launch_map(const Launch& L);
 // learned force correction (lbm_learned.cu)
 cudaError_t launch_features(int storage, const void* state, const Launch& L, const double* force,

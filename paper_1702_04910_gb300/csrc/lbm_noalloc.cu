@@ -120,12 +120,7 @@ extern "C" lbm_status lbm_sweep_noalloc(const lbm_config* cfg, const double* src
     g.bc_z = cfg->bc_z;
     g.n = (long long)cfg->nx * cfg->ny * cfg->nz;
     set_open_boundaries(g, *cfg);
-    g.tx = cfg->nx >= 128 ? 128 : (cfg->nx >= 64 ? 64 : 32);
-    g.ty = 256 / g.tx;
-    g.ntx = (cfg->nx + g.tx - 1) / g.tx;
-    g.nty = (cfg->ny + g.ty - 1) / g.ty;
-    g.tz = 1;
-    g.ntz = cfg->nz;
+    set_tiles(g, LBM_STORE_F64);
     double maxd = 0.0;
     ParticleUpload up{};
     for (int i = 0; i < n; ++i) {
