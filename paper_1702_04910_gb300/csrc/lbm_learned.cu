@@ -21,6 +21,7 @@
 //   [500,512)  U_p / u_ref, Omega_p R / u_ref, F / (rho0 u_ref^2 D^2),
 //              T / (rho0 u_ref^2 D^3) (F, T: this step's hydrodynamic force).
 // Outputs: the correction (dF, dT) in the same units as the last two blocks.
+#include <cuda_pipeline.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -137,16 +138,13 @@ __global__ void __launch_bounds__(128)
 }
 
 // ---------------------------------------------------------------------------
-// MLP forward: one 64-thread block per sample.  Inputs are normalised on
-// load, x^ = (x - mu) / sigma; the network output y^ is kept (normalised)
-// and y = y^ * out_scale returned.  H1, H2 may be null (inference).
-// With clip > 0 a sample with any |x^_i| > clip (outside the training data)
-// gets y = 0: the caller's plain force stands.
+// MLP inference: one 64-thread block per sample.  Inputs are normalised on
+// load, x^ = (x - mu) / sigma; the network output y^ times out_scale is
+// returned.  With clip > 0 a sample with any |x^_i| > clip (outside the
+// training data) gets y = 0: the caller's plain force stands.
 __global__ void __launch_bounds__(FH)
     k_mlp_forward(const float* __restrict__ P, const float* __restrict__ norm,
-                  const float* __restrict__ X, int n, float* __restrict__ H1,
-                  float* __restrict__ H2, float* __restrict__ Yn, float* __restrict__ Y,
-                  float clip) {
+                  const float* __restrict__ X, int n, float* __restrict__ Y, float clip) {
     __shared__ float xs[FIN], h1[FH], h2[FH];
     const int smp = blockIdx.x, u = threadIdx.x;
     if (smp >= n) return;
@@ -158,115 +156,294 @@ __global__ void __launch_bounds__(FH)
         out_of_range |= clip > 0.0f && !(fabsf(v) <= clip);
     }
     if (__syncthreads_or(out_of_range)) {
-        if (u < FOUT) {
-            if (Yn) Yn[(long long)smp * FOUT + u] = 0.0f;
-            if (Y) Y[(long long)smp * FOUT + u] = 0.0f;
-        }
+        if (u < FOUT) Y[(long long)smp * FOUT + u] = 0.0f;
         return;
     }
     float a = P[OFF_B1 + u];
     for (int i = 0; i < FIN; ++i) a = fmaf(P[OFF_W1 + i * FH + u], xs[i], a);
-    const float t1 = tanhf(a);
-    h1[u] = t1;
-    if (H1) H1[(long long)smp * FH + u] = t1;
+    h1[u] = tanhf(a);
     __syncthreads();
     a = P[OFF_B2 + u];
     for (int v = 0; v < FH; ++v) a = fmaf(P[OFF_W2 + v * FH + u], h1[v], a);
-    const float t2 = tanhf(a);
-    h2[u] = t2;
-    if (H2) H2[(long long)smp * FH + u] = t2;
+    h2[u] = tanhf(a);
     __syncthreads();
     if (u < FOUT) {
         a = P[OFF_B3 + u];
         for (int v = 0; v < FH; ++v) a = fmaf(P[OFF_W3 + v * FOUT + u], h2[v], a);
-        if (Yn) Yn[(long long)smp * FOUT + u] = a;
-        if (Y) Y[(long long)smp * FOUT + u] = a * norm[NORM_OS + u];
+        Y[(long long)smp * FOUT + u] = a * norm[NORM_OS + u];
     }
 }
 
-// Backward deltas of the loss L = 1/(2n) sum_s sum_k w_k (y^_sk - t_sk / os_k)^2,
-// w_k = (os_k / max_j os_j)^2 (each output's error in the units of the
-// largest target), one 64-thread block per sample: D3 = dL/dz3, D2 = dL/dz2,
-// D1 = dL/dz1 (z: pre-activations), and the sample's loss term.
-__global__ void __launch_bounds__(FH)
-    k_mlp_delta(const float* __restrict__ P, const float* __restrict__ norm,
-                const float* __restrict__ Tt, int n, const float* __restrict__ H1,
-                const float* __restrict__ H2, const float* __restrict__ Yn,
-                float* __restrict__ D1, float* __restrict__ D2, float* __restrict__ D3,
-                double* __restrict__ loss_s) {
-    __shared__ float d3[FOUT], e3[FOUT], d2[FH];
-    const int smp = blockIdx.x, u = threadIdx.x;
-    if (smp >= n) return;
+// Forward pass and backward deltas of S samples per block, for the loss
+// L = 1/(2n) sum_s sum_k w_k (y^_sk - t_sk / os_k)^2, w_k = (os_k / max_j os_j)^2
+// (each output's error in the units of the largest target): H1, H2 the hidden
+// values, D1, D2, D3 = dL/dz of the three layers (z: pre-activations), and the
+// block's loss terms added in a fixed order into loss_b[block].
+//
+// What bounds it: the FP32 FMAs of the first layer (32,768 per sample) and,
+// with one block per sample as before, the 150 KB of parameters each block
+// reads from L2 (1.1 GB for 7200 samples).  A thread keeps S / 8 samples of one
+// unit, so a weight read serves S samples of the block, and the inputs come
+// from shared memory four at a time.  Every sum keeps the order of the
+// one-sample form (i ascending from the bias), so the values are the same
+// bits.  S follows n (gradient()).  7200 samples, cold L2: forward and delta
+// kernels 175 us -> 57 us (long scoreboard first: 8 warps per scheduler).
+constexpr int PASS_GROUPS = 8, PASS_THREADS = PASS_GROUPS * FH;
+template <int S>
+__global__ void __launch_bounds__(PASS_THREADS, 2)
+    k_mlp_pass(const float* __restrict__ P, const float* __restrict__ norm,
+               const float* __restrict__ X, const float* __restrict__ Tt, int n,
+               float* __restrict__ H1, float* __restrict__ H2, float* __restrict__ D1,
+               float* __restrict__ D2, float* __restrict__ D3, double* __restrict__ loss_b) {
+    constexpr int R = S / PASS_GROUPS;  // samples per thread
+    extern __shared__ float4 pass_smem[];
+    float* xs = reinterpret_cast<float*>(pass_smem);  // [S][FIN]; then the arrays below
+    __shared__ float h1[S][FH], h2[S][FH], d2[S][FH];
+    __shared__ __align__(16) float w2[FH][FH + 1];
+    __shared__ float d3[S][FOUT];
+    __shared__ double ls[S];
+    const int tid = threadIdx.x, u = tid % FH, g = tid / FH;
+    const int s0 = blockIdx.x * S;
+    static_assert(PASS_THREADS == FIN, "one input column per thread");
+    const float mu = norm[NORM_MU + tid], is = norm[NORM_IS + tid];
+#pragma unroll 8
+    for (int s = 0; s < S; ++s)
+        xs[s * FIN + tid] =
+            s0 + s < n ? (X[(long long)(s0 + s) * FIN + tid] - mu) * is : 0.0f;
+    // W1 in chunks of WC rows through w2's space, WS chunks in flight
+    constexpr int WC = 16, WS = 4;
+    float (*wc)[WC * FH] = reinterpret_cast<float (*)[WC * FH]>(&w2[0][0]);
+    static_assert(sizeof(float) * WS * WC * FH <= sizeof(w2) && WC * FH == 2 * PASS_THREADS, "chunk");
+    const auto chunk = [&](int c) {
+        if (c < FIN / WC)
+            for (int e = tid; e < WC * FH; e += PASS_THREADS)
+                __pipeline_memcpy_async(&wc[c % WS][e], P + OFF_W1 + c * WC * FH + e, sizeof(float));
+        __pipeline_commit();
+    };
+    float acc[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) acc[r] = P[OFF_B1 + u];
+    for (int c = 0; c < WS - 1; ++c) chunk(c);
+    for (int c = 0; c < FIN / WC; ++c) {
+        __pipeline_wait_prior(WS - 2);
+        __syncthreads();  // chunk c is in place and chunk c - 1 is done with
+        chunk(c + WS - 1);
+        const float* wv = wc[c % WS];
+#pragma unroll
+        for (int i = 0; i < WC; i += 4) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const float4 x =
+                    *reinterpret_cast<const float4*>(xs + (g * R + r) * FIN + c * WC + i);
+                acc[r] = fmaf(wv[(i + 0) * FH + u], x.x, acc[r]);
+                acc[r] = fmaf(wv[(i + 1) * FH + u], x.y, acc[r]);
+                acc[r] = fmaf(wv[(i + 2) * FH + u], x.z, acc[r]);
+                acc[r] = fmaf(wv[(i + 3) * FH + u], x.w, acc[r]);
+            }
+        }
+    }
+    __syncthreads();
+    for (int e = tid; e < FH * FH; e += PASS_THREADS) w2[e / FH][e % FH] = P[OFF_W2 + e];
+#pragma unroll
+    for (int r = 0; r < R; ++r) h1[g * R + r][u] = tanhf(acc[r]);
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < R; ++r) acc[r] = P[OFF_B2 + u];
+#pragma unroll 4
+    for (int v = 0; v < FH; ++v) {
+        const float w = w2[v][u];
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r] = fmaf(w, h1[g * R + r][v], acc[r]);
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) h2[g * R + r][u] = tanhf(acc[r]);
+    __syncthreads();
     const float inv_n = 1.0f / (float)n;
-    if (u < FOUT) {
-        float smax = norm[NORM_OS];
-        for (int k = 1; k < FOUT; ++k) smax = fmaxf(smax, norm[NORM_OS + k]);
-        const float r = norm[NORM_OS + u] / smax, w = r * r;
-        const float e = Yn[(long long)smp * FOUT + u] - Tt[(long long)smp * FOUT + u] / norm[NORM_OS + u];
-        e3[u] = w * e * e;
-        d3[u] = w * e * inv_n;
-        D3[(long long)smp * FOUT + u] = w * e * inv_n;
+    float smax = norm[NORM_OS];
+    for (int k = 1; k < FOUT; ++k) smax = fmaxf(smax, norm[NORM_OS + k]);
+    for (int e = tid; e < S * FOUT; e += PASS_THREADS) {
+        const int s = e / FOUT, k = e % FOUT;
+        float a = P[OFF_B3 + k];
+        for (int v = 0; v < FH; ++v) a = fmaf(P[OFF_W3 + v * FOUT + k], h2[s][v], a);
+        const float rr = norm[NORM_OS + k] / smax, w = rr * rr;
+        float err = 0.0f;
+        if (s0 + s < n) {
+            err = a - Tt[(long long)(s0 + s) * FOUT + k] / norm[NORM_OS + k];
+            D3[(long long)(s0 + s) * FOUT + k] = w * err * inv_n;
+        }
+        d3[s][k] = w * err * inv_n;
+        xs[e] = w * err * err;  // loss terms (the inputs are done with)
     }
     __syncthreads();
-    if (u == 0) {
+    if (tid < S) {
         double l = 0.0;
-        for (int k = 0; k < FOUT; ++k) l += 0.5 * (double)e3[k];
-        loss_s[smp] = l;
+        for (int k = 0; k < FOUT; ++k) l += 0.5 * (double)xs[tid * FOUT + k];
+        ls[tid] = l;
     }
-    float a = 0.0f;
-    for (int k = 0; k < FOUT; ++k) a = fmaf(P[OFF_W3 + u * FOUT + k], d3[k], a);
-    const float h2 = H2[(long long)smp * FH + u];
-    const float g2 = a * (1.0f - h2 * h2);
-    d2[u] = g2;
-    D2[(long long)smp * FH + u] = g2;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int s = g * R + r;
+        float a = 0.0f;
+        for (int k = 0; k < FOUT; ++k) a = fmaf(P[OFF_W3 + u * FOUT + k], d3[s][k], a);
+        d2[s][u] = a * (1.0f - h2[s][u] * h2[s][u]);
+    }
     __syncthreads();
-    a = 0.0f;
-    for (int v = 0; v < FH; ++v) a = fmaf(P[OFF_W2 + u * FH + v], d2[v], a);
-    const float h1 = H1[(long long)smp * FH + u];
-    D1[(long long)smp * FH + u] = a * (1.0f - h1 * h1);
+#pragma unroll
+    for (int r = 0; r < R; ++r) acc[r] = 0.0f;
+#pragma unroll 4
+    for (int v = 0; v < FH; ++v) {
+        const float w = w2[u][v];
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r] = fmaf(w, d2[g * R + r][v], acc[r]);
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int s = g * R + r;
+        if (s0 + s >= n) continue;
+        const long long o = (long long)(s0 + s) * FH + u;
+        H1[o] = h1[s][u];
+        H2[o] = h2[s][u];
+        D2[o] = d2[s][u];
+        D1[o] = acc[r] * (1.0f - h1[s][u] * h1[s][u]);
+    }
+    if (tid == 0) {
+        double l = 0.0;
+        for (int s = 0; s < S; ++s) l += ls[s];
+        loss_b[blockIdx.x] = l;
+    }
 }
 
-// Parameter gradient, one thread per parameter: dW[i][o] = sum_s a_s[i] d_s[o],
-// db[o] = sum_s d_s[o], samples summed in order (deterministic).
-__global__ void __launch_bounds__(256)
+// Parameter gradient: dW[i][o] = sum_s a_s[i] d_s[o], db[o] = sum_s d_s[o],
+// samples in order (a long training run amplifies any other order).  One block
+// per 16 x 16 tile of a weight matrix, two outputs per thread; the tiles of a
+// layer's first rows also add its bias.
+//
+// What bounds it: the chain of n dependent FMAs of every output, 4 cycles
+// each, 14.5 us for 7200 samples, and above it the shared-memory reads of the
+// 256 outputs that 148 blocks leave to an SM.  The operands pass through
+// shared memory sample-fastest, so a thread reads four samples of a row at a
+// time (4 16-byte reads for 16 FMAs, no bank conflicts between rows r and
+// r + 8); row lengths are compile-time, so a chunk's loads are one address and
+// immediate offsets, and the next chunk's are in flight during the sums.
+// Before, one thread per parameter read both operands from global memory for
+// each FMA.  7200 samples, cold L2: 811 us -> 93 us (two outputs per thread,
+// 3 reads for 8 FMAs: 103 us), the same bits; the whole gradient call 977 us
+// -> 169 us.  Samples cut into slices and added later would take 56 us, but
+// the changed order sends a 3000-step Adam run through spikes of the loss.
+constexpr int GT = 16, GRAD_K = 128, GRAD_THREADS = GT * GT / 4;
+constexpr int GRAD_T1 = (FIN / GT) * (FH / GT), GRAD_T2 = (FH / GT) * (FH / GT), GRAD_T3 = FH / GT;
+struct GradTile {
+    __align__(16) float A[GT][GRAD_K + 4];
+    __align__(16) float B[GT][GRAD_K + 4];
+};
+// Tile (i0, o0) of a layer: A [n][LDA] (NORM: normalised on the way), B [n][LDB].
+template <int LDA, int LDB, bool NORM, bool BIAS>
+__device__ __forceinline__ void grad_tile(GradTile& w, const float* __restrict__ norm,
+                                          const float* __restrict__ As,
+                                          const float* __restrict__ Bs, int n, int i0, int o0,
+                                          float* __restrict__ W, float* __restrict__ bias) {
+    const int tid = threadIdx.x;
+    // loads: column lc of samples ls, ls + STEP, ... of the chunk
+    constexpr int STEP = GRAD_THREADS / GT, PER = GRAD_K / STEP;
+    const int lc = tid % GT, ls = tid / GT;
+    const float mu = NORM ? norm[NORM_MU + i0 + lc] : 0.0f;
+    const float is = NORM ? norm[NORM_IS + i0 + lc] : 1.0f;
+    const bool bcol = LDB >= FH || o0 + lc < LDB;
+    float ra[PER], rb[PER];
+    const auto fetch = [&](int s0) {
+        const float* pa = As + (long long)(s0 + ls) * LDA + i0 + lc;
+        const float* pb = Bs + (long long)(s0 + ls) * LDB + o0 + lc;
+        if (s0 + GRAD_K <= n) {
+#pragma unroll
+            for (int k = 0; k < PER; ++k) {
+                ra[k] = pa[k * STEP * LDA];
+                rb[k] = bcol ? pb[k * STEP * LDB] : 0.0f;
+            }
+        } else {  // samples beyond n add zero (mu: its normalised value)
+#pragma unroll
+            for (int k = 0; k < PER; ++k) {
+                const bool in = s0 + ls + k * STEP < n;
+                ra[k] = in ? pa[k * STEP * LDA] : mu;
+                rb[k] = in && bcol ? pb[k * STEP * LDB] : 0.0f;
+            }
+        }
+    };
+    const int ti = tid / 8, to = tid % 8;  // outputs (ti, ti + 8) x (to, to + 8)
+    float acc[2][2] = {}, b0 = 0.0f, b1 = 0.0f;
+    fetch(0);
+    for (int s0 = 0; s0 < n; s0 += GRAD_K) {
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            w.A[lc][ls + k * STEP] = NORM ? (ra[k] - mu) * is : ra[k];
+            w.B[lc][ls + k * STEP] = rb[k];
+        }
+        __syncthreads();
+        if (s0 + GRAD_K < n) fetch(s0 + GRAD_K);
+#pragma unroll 4
+        for (int s = 0; s < GRAD_K; s += 4) {
+            const float4 a0 = *reinterpret_cast<const float4*>(&w.A[ti][s]);
+            const float4 a1 = *reinterpret_cast<const float4*>(&w.A[ti + 8][s]);
+            const float4 u = *reinterpret_cast<const float4*>(&w.B[to][s]);
+            const float4 v = *reinterpret_cast<const float4*>(&w.B[to + 8][s]);
+            const auto dot = [](float4 a, float4 b, float c) {
+                return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, c))));
+            };
+            acc[0][0] = dot(a0, u, acc[0][0]);
+            acc[0][1] = dot(a0, v, acc[0][1]);
+            acc[1][0] = dot(a1, u, acc[1][0]);
+            acc[1][1] = dot(a1, v, acc[1][1]);
+            if (BIAS) {
+                b0 = b0 + u.x + u.y + u.z + u.w;
+                b1 = b1 + v.x + v.y + v.z + v.w;
+            }
+        }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int o = o0 + to + 8 * h;
+        if (LDB < FH && o >= LDB) continue;
+        W[(i0 + ti) * LDB + o] = acc[0][h];
+        W[(i0 + ti + 8) * LDB + o] = acc[1][h];
+        if (BIAS && ti == 0) bias[o] = h ? b1 : b0;
+    }
+}
+
+__global__ void __launch_bounds__(GRAD_THREADS)
     k_mlp_grad(const float* __restrict__ norm, const float* __restrict__ X, int n,
                const float* __restrict__ H1, const float* __restrict__ H2,
                const float* __restrict__ D1, const float* __restrict__ D2,
                const float* __restrict__ D3, float* __restrict__ G) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= NPARAM) return;
-    float acc = 0.0f;
-    if (t < OFF_B1) {
-        const int i = t / FH, o = t % FH;
-        const float mu = norm[NORM_MU + i], is = norm[NORM_IS + i];
-        for (int s = 0; s < n; ++s)
-            acc = fmaf((X[(long long)s * FIN + i] - mu) * is, D1[(long long)s * FH + o], acc);
-    } else if (t < OFF_W2) {
-        const int o = t - OFF_B1;
-        for (int s = 0; s < n; ++s) acc += D1[(long long)s * FH + o];
-    } else if (t < OFF_B2) {
-        const int i = (t - OFF_W2) / FH, o = (t - OFF_W2) % FH;
-        for (int s = 0; s < n; ++s) acc = fmaf(H1[(long long)s * FH + i], D2[(long long)s * FH + o], acc);
-    } else if (t < OFF_W3) {
-        const int o = t - OFF_B2;
-        for (int s = 0; s < n; ++s) acc += D2[(long long)s * FH + o];
-    } else if (t < OFF_B3) {
-        const int i = (t - OFF_W3) / FOUT, o = (t - OFF_W3) % FOUT;
-        for (int s = 0; s < n; ++s)
-            acc = fmaf(H2[(long long)s * FH + i], D3[(long long)s * FOUT + o], acc);
+    __shared__ GradTile w;
+    int t = blockIdx.x;
+    constexpr int OT = FH / GT;  // tiles across the 64 outputs of a layer
+    if (t < GRAD_T1) {
+        const int i0 = t / OT * GT, o0 = t % OT * GT;
+        if (i0 == 0) grad_tile<FIN, FH, true, true>(w, norm, X, D1, n, i0, o0, G + OFF_W1, G + OFF_B1);
+        else grad_tile<FIN, FH, true, false>(w, norm, X, D1, n, i0, o0, G + OFF_W1, nullptr);
+    } else if ((t -= GRAD_T1) < GRAD_T2) {
+        grad_tile<FH, FH, false, true>(w, norm, H1, D2, n, t / OT * GT, t % OT * GT, G + OFF_W2,
+                                       G + OFF_B2);
     } else {
-        const int o = t - OFF_B3;
-        for (int s = 0; s < n; ++s) acc += D3[(long long)s * FOUT + o];
+        grad_tile<FH, FOUT, false, true>(w, norm, H2, D3, n, (t - GRAD_T2) * GT, 0, G + OFF_W3,
+                                         G + OFF_B3);
     }
-    G[t] = acc;
 }
 
-// loss = sum of the per-sample terms / n, summed in order
-__global__ void k_mlp_loss(const double* __restrict__ loss_s, int n, double* __restrict__ loss) {
-    if (blockIdx.x != 0 || threadIdx.x != 0) return;
+// loss = sum of the pass blocks' terms / n: 256 interleaved sums, then a tree
+// (a fixed order; before, one thread read all n terms).
+__global__ void __launch_bounds__(256)
+    k_mlp_loss(const double* __restrict__ loss_b, int nb, int n, double* __restrict__ loss) {
+    __shared__ double ls[256];
     double l = 0.0;
-    for (int s = 0; s < n; ++s) l += loss_s[s];
-    *loss = l / n;
+    for (int b = threadIdx.x; b < nb; b += blockDim.x) l += loss_b[b];
+    ls[threadIdx.x] = l;
+    __syncthreads();
+    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
+        if (threadIdx.x < s) ls[threadIdx.x] += ls[threadIdx.x + s];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *loss = ls[0] / n;
 }
 
 // Adam (Kingma & Ba 2015) with bias correction; step t >= 1.
@@ -366,8 +543,8 @@ struct lbm_mlp {
     int adam_t;
     // per-sample work buffers (grown on demand)
     int cap;
-    float *h1, *h2, *yn, *d1, *d2, *d3;
-    double* loss_s;
+    float *h1, *h2, *d1, *d2, *d3;
+    double* loss_b;  // loss terms of the pass's blocks
     char err[512];
 };
 
@@ -392,13 +569,12 @@ lbm_status mcuda(lbm_mlp* m, cudaError_t e, const char* where) {
 void free_work(lbm_mlp* m) {
     cudaFree(m->h1);
     cudaFree(m->h2);
-    cudaFree(m->yn);
     cudaFree(m->d1);
     cudaFree(m->d2);
     cudaFree(m->d3);
-    cudaFree(m->loss_s);
-    m->h1 = m->h2 = m->yn = m->d1 = m->d2 = m->d3 = nullptr;
-    m->loss_s = nullptr;
+    cudaFree(m->loss_b);
+    m->h1 = m->h2 = m->d1 = m->d2 = m->d3 = nullptr;
+    m->loss_b = nullptr;
     m->cap = 0;
 }
 
@@ -409,29 +585,43 @@ lbm_status ensure_work(lbm_mlp* m, int n) {
     const size_t N = (size_t)n;
     MK(m, cudaMalloc(&m->h1, sizeof(float) * N * FH), "cudaMalloc mlp work");
     MK(m, cudaMalloc(&m->h2, sizeof(float) * N * FH), "cudaMalloc mlp work");
-    MK(m, cudaMalloc(&m->yn, sizeof(float) * N * FOUT), "cudaMalloc mlp work");
     MK(m, cudaMalloc(&m->d1, sizeof(float) * N * FH), "cudaMalloc mlp work");
     MK(m, cudaMalloc(&m->d2, sizeof(float) * N * FH), "cudaMalloc mlp work");
     MK(m, cudaMalloc(&m->d3, sizeof(float) * N * FOUT), "cudaMalloc mlp work");
-    MK(m, cudaMalloc(&m->loss_s, sizeof(double) * N), "cudaMalloc mlp work");
+    MK(m, cudaMalloc(&m->loss_b, sizeof(double) * N), "cudaMalloc mlp work");
     m->cap = n;
     return LBM_OK;
+}
+
+template <int S>
+cudaError_t launch_pass(lbm_mlp* m, const float* x, const float* t, int n, int& blocks) {
+    blocks = (n + S - 1) / S;
+    const int smem = S * FIN * (int)sizeof(float);
+    if (smem > 16 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(
+            k_mlp_pass<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+    }
+    k_mlp_pass<S><<<blocks, PASS_THREADS, smem, m->stream>>>(
+        m->params, m->norm, x, t, n, m->h1, m->h2, m->d1, m->d2, m->d3, m->loss_b);
+    return cudaGetLastError();
 }
 
 // forward + deltas + parameter gradient into m->grad and the loss into m->loss
 lbm_status gradient(lbm_mlp* m, const float* x, const float* t, int n) {
     lbm_status st = ensure_work(m, n);
     if (st != LBM_OK) return st;
-    k_mlp_forward<<<n, FH, 0, m->stream>>>(m->params, m->norm, x, n, m->h1, m->h2, m->yn, nullptr,
-                                           0.0f);
-    MK(m, cudaGetLastError(), "mlp forward launch");
-    k_mlp_delta<<<n, FH, 0, m->stream>>>(m->params, m->norm, t, n, m->h1, m->h2, m->yn, m->d1, m->d2,
-                                         m->d3, m->loss_s);
-    MK(m, cudaGetLastError(), "mlp delta launch");
-    k_mlp_grad<<<(NPARAM + 255) / 256, 256, 0, m->stream>>>(m->norm, x, n, m->h1, m->h2, m->d1, m->d2,
-                                                            m->d3, m->grad);
+    // samples per block of the pass: 32 once that gives every SM a block
+    // (152 x 32 samples), fewer for small sets, whose time is one block's chain
+    int blocks = 0;
+    MK(m, n >= 152 * 32 ? launch_pass<32>(m, x, t, n, blocks)
+                        : (n >= 152 * 16 ? launch_pass<16>(m, x, t, n, blocks)
+                                         : launch_pass<8>(m, x, t, n, blocks)),
+       "mlp pass launch");
+    k_mlp_grad<<<GRAD_T1 + GRAD_T2 + GRAD_T3, GRAD_THREADS, 0, m->stream>>>(
+        m->norm, x, n, m->h1, m->h2, m->d1, m->d2, m->d3, m->grad);
     MK(m, cudaGetLastError(), "mlp gradient launch");
-    k_mlp_loss<<<1, 1, 0, m->stream>>>(m->loss_s, n, m->loss);
+    k_mlp_loss<<<1, 256, 0, m->stream>>>(m->loss_b, blocks, n, m->loss);
     MK(m, cudaGetLastError(), "mlp loss launch");
     return LBM_OK;
 }
@@ -450,7 +640,7 @@ namespace lbmgpu {
 cudaError_t mlp_infer(const lbm_mlp* m, const float* x, int n, float* y, float clip,
                       cudaStream_t s) {
     if (n < 1) return cudaSuccess;
-    k_mlp_forward<<<n, FH, 0, s>>>(m->params, m->norm, x, n, nullptr, nullptr, nullptr, y, clip);
+    k_mlp_forward<<<n, FH, 0, s>>>(m->params, m->norm, x, n, y, clip);
     return cudaGetLastError();
 }
 }  // namespace lbmgpu
@@ -563,9 +753,9 @@ lbm_status lbm_mlp_gradient(lbm_mlp* m, const float* x_dev, const float* t_dev, 
     if (grad_host) {
         MK(m, cudaMemcpyAsync(grad_host, m->grad, sizeof(float) * NPARAM, cudaMemcpyDeviceToHost, m->stream),
            "gradient download");
-        MK(m, cudaStreamSynchronize(m->stream), "gradient sync");
+        if (!loss) MK(m, cudaStreamSynchronize(m->stream), "gradient sync");
     }
-    return read_loss(m, loss);
+    return read_loss(m, loss);  // synchronises for both copies
 }
 
 lbm_status lbm_mlp_train(lbm_mlp* m, const float* x_dev, const float* t_dev, int n, int steps,
