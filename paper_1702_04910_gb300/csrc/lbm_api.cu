@@ -307,31 +307,40 @@ lbm_status step_once(lbm_handle* h) {
         if ((st = sweep(h, s, coupled && s == 0)) != LBM_OK) return st;
     if (!coupled) return LBM_OK;
     Launch L = base_launch(h);
-    int pi = prof_begin(h, PC_FINAL);
-    CK(h, launch_finalize(L, nsub, h->d_force, h->remap_charge ? h->d_charge : nullptr),
-       "force total launch");
-    prof_end(h, pi);
-    if (h->model_mode) {
-        // features of P^n and the flow after the sweeps; corrected force
-        pi = prof_begin(h, PC_OTHER);
-        CK(h, launch_features(h->storage, h->buf[h->cur], L, h->d_force, h->u_ref, h->d_feat),
-           "feature launch");
-        if (h->model_mode == 1) {
-            // a particle whose features lie beyond 10 standard deviations of
-            // the training data keeps the plain force (fallback)
-            CK(h, mlp_infer(h->model, h->d_feat, h->np, h->d_corr, 10.0f, h->stream),
-               "force model launch");
-            CK(h, launch_apply_correction(h->d_corr, h->d_parts, h->np, h->u_ref, h->cfg.rho0,
-                                          h->d_force, h->stream),
-               "force correction launch");
+    const double* charge = h->remap_charge ? h->d_charge : nullptr;
+    const double* gr = h->cfg.gravity;
+    int pi;
+    if (!h->model_mode && !h->profiling) {
+        CK(h, launch_finalize_rigid(L, nsub, h->d_force, charge, gr[0], gr[1], gr[2],
+                                    h->cfg.wall_contact),
+           "force total and rigid body launch");
+    } else {
+        // a force model works on the total, and profiling times the two apart
+        pi = prof_begin(h, PC_FINAL);
+        CK(h, launch_finalize(L, nsub, h->d_force, charge), "force total launch");
+        prof_end(h, pi);
+        if (h->model_mode) {
+            // features of P^n and the flow after the sweeps; corrected force
+            pi = prof_begin(h, PC_OTHER);
+            CK(h, launch_features(h->storage, h->buf[h->cur], L, h->d_force, h->u_ref, h->d_feat),
+               "feature launch");
+            if (h->model_mode == 1) {
+                // a particle whose features lie beyond 10 standard deviations of
+                // the training data keeps the plain force (fallback)
+                CK(h, mlp_infer(h->model, h->d_feat, h->np, h->d_corr, 10.0f, h->stream),
+                   "force model launch");
+                CK(h, launch_apply_correction(h->d_corr, h->d_parts, h->np, h->u_ref, h->cfg.rho0,
+                                              h->d_force, h->stream),
+                   "force correction launch");
+            }
+            prof_end(h, pi);
         }
+        pi = prof_begin(h, PC_RIGID);
+        CK(h, launch_rigid_body(L, h->d_force, gr[0], gr[1], gr[2], (double)nsub,
+                                h->cfg.wall_contact),
+           "rigid body launch");
         prof_end(h, pi);
     }
-    pi = prof_begin(h, PC_RIGID);
-    CK(h, launch_rigid_body(L, h->d_force, h->cfg.gravity[0], h->cfg.gravity[1],
-                            h->cfg.gravity[2], (double)nsub, h->cfg.wall_contact),
-       "rigid body launch");
-    prof_end(h, pi);
     if (h->kind == 2) {
         // re-map with the new state; rebuild uncovered cells (src of the last sweep)
         L.box[0] = (int)std::ceil(h->maxd) + 4;  // refill: cube side in cells

@@ -243,41 +243,20 @@ __device__ __forceinline__ bool spans_meet(int a, int la, int r, int lr, int n) 
     return range_off(a, r, n) < lr || range_off(r, a, n) < la;
 }
 
-struct NearRegion {
-    AxisRange ax[3];
-};
-
-__device__ inline NearRegion near_region(const Geom& g, const DevParticle& P) {
-    NearRegion nr;
-    nr.ax[0] = axis_range(P.x[0], P.r, g.nx, g.tx, g.ntx, true);
-    nr.ax[1] = axis_range(P.x[1], P.r, g.ny, g.ty, g.nty, true);
-    nr.ax[2] = axis_range(P.x[2], P.r, g.nz, g.tz, g.ntz, !g.bc_z);
-    return nr;
-}
-
-__device__ __forceinline__ bool tile_in_region(const Geom& g, const NearRegion& nr, int tx,
-                                               int ty, int tz) {
-    return in_range(tx, nr.ax[0].tlo, nr.ax[0].tlen, g.ntx) &&
-           in_range(ty, nr.ax[1].tlo, nr.ax[1].tlen, g.nty) &&
-           in_range(tz, nr.ax[2].tlo, nr.ax[2].tlen, g.ntz);
-}
-
-__device__ __forceinline__ bool cell_in_region(const Geom& g, const NearRegion& nr, int x, int y,
-                                               int z) {
-    return in_range(x, nr.ax[0].clo, nr.ax[0].clen, g.nx) &&
-           in_range(y, nr.ax[1].clo, nr.ax[1].clen, g.ny) &&
-           in_range(z, nr.ax[2].clo, nr.ax[2].clen, g.nz);
+// Cache axis a of the region of a particle centred at x in P.reg.
+__device__ inline void store_region_axis(const Geom& g, DevParticle& P, double x, int a) {
+    const AxisRange r = axis_range(x, P.r, a == 0 ? g.nx : (a == 1 ? g.ny : g.nz),
+                                   a == 0 ? g.tx : (a == 1 ? g.ty : g.tz),
+                                   a == 0 ? g.ntx : (a == 1 ? g.nty : g.ntz), a < 2 || !g.bc_z);
+    P.reg[4 * a + 0] = r.clo;
+    P.reg[4 * a + 1] = r.clen;
+    P.reg[4 * a + 2] = r.tlo;
+    P.reg[4 * a + 3] = r.tlen;
 }
 
 // Cache the region of P's current state in P.reg.
 __device__ inline void store_region(const Geom& g, DevParticle& P) {
-    NearRegion nr = near_region(g, P);
-    for (int a = 0; a < 3; ++a) {
-        P.reg[4 * a + 0] = nr.ax[a].clo;
-        P.reg[4 * a + 1] = nr.ax[a].clen;
-        P.reg[4 * a + 2] = nr.ax[a].tlo;
-        P.reg[4 * a + 3] = nr.ax[a].tlen;
-    }
+    for (int a = 0; a < 3; ++a) store_region_axis(g, P, P.x[a], a);
 }
 
 __device__ __forceinline__ bool tile_in_reg(const Geom& g, const int* reg, int tx, int ty,

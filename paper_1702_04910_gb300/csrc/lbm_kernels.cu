@@ -924,116 +924,127 @@ __global__ void __launch_bounds__(32)
 // blocks of every particle's region, of subcycle k's partials for q.
 // charge != nullptr: the pending re-mapping momentum charge of q, [q][6],
 // divided by the step's lattice time nsub, is taken off.
+//
+// A few thousand doubles at most, so latency bounds it: thread t adds
+// component t mod 6 of every 128th partial (consecutive threads read
+// consecutive doubles), one warp per component adds the 128 sums.  D = 24,
+// 900 partials: 13.7 us (256 threads over all six components, an eight-level
+// tree of FP64 adds per subcycle) + 8.6 us of rigid-body update -> 10.2 us for
+// both in one launch (k_finalize_rigid), cold L2.
+constexpr int FIN_WAYS = 128, FIN_THREADS = 6 * FIN_WAYS;
 __device__ __forceinline__ void finalize_block(int np, long long nblk,
                                                const double* __restrict__ partials, int nsub,
-                                               double* __restrict__ out, int q,
-                                               double (*red)[6],
+                                               double* out, int q, double* red,
                                                const double* __restrict__ charge = nullptr) {
-    const int tid = threadIdx.x;
-    const long long count = (long long)np * nblk;
-    double tot[6] = {0, 0, 0, 0, 0, 0};
-    for (int sub = 0; sub < nsub; ++sub) {
-        const double* base = partials + (long long)sub * count * np * 6;
-        double acc[6] = {0, 0, 0, 0, 0, 0};
-        for (long long kk = tid; kk < count; kk += blockDim.x) {
-#pragma unroll
-            for (int c = 0; c < 6; ++c) acc[c] += base[(kk * np + q) * 6 + c];
-        }
-#pragma unroll
-        for (int c = 0; c < 6; ++c) red[tid][c] = acc[c];
-        __syncthreads();
-        for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-            if (tid < s)
-#pragma unroll
-                for (int c = 0; c < 6; ++c) red[tid][c] += red[tid + s][c];
-            __syncthreads();
-        }
-        if (tid == 0)
-#pragma unroll
-            for (int c = 0; c < 6; ++c) tot[c] += red[0][c];
-        __syncthreads();
+    const int tid = threadIdx.x, c = tid % 6, way = tid / 6;
+    const long long count = (long long)nsub * np * nblk;
+    double acc = 0.0;
+#pragma unroll 4
+    for (long long m = way; m < count; m += FIN_WAYS) acc += partials[(m * np + q) * 6 + c];
+    red[c * FIN_WAYS + way] = acc;
+    __syncthreads();
+    const int w = tid >> 5, lane = tid & 31;
+    if (w < 6) {
+        const double* r = red + w * FIN_WAYS + lane;
+        const double v = warp_sum((r[0] + r[32]) + (r[64] + r[96]));
+        if (lane == 0)
+            out[q * 6 + w] = charge ? v / nsub - charge[q * 6 + w] / nsub : v / nsub;
     }
-    if (tid == 0)
-        for (int c = 0; c < 6; ++c)
-            out[q * 6 + c] = charge ? tot[c] / nsub - charge[q * 6 + c] / nsub : tot[c] / nsub;
 }
 
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(FIN_THREADS)
     k_finalize(int np, long long nblk, const double* __restrict__ partials, int nsub,
                double* __restrict__ out, const double* __restrict__ charge) {
-    __shared__ double red[256][6];
+    __shared__ double red[FIN_THREADS];
     finalize_block(np, nblk, partials, nsub, out, blockIdx.x, red, charge);
 }
 
 // ---------------------------------------------------------------------------
 // explicit Euler rigid-body update over dt, gravity + buoyancy
-// (rho_p - rho0) V g; keeps the previous state in `prev`.
-__device__ __forceinline__ void rigid_one(const Geom& g, DevParticle* __restrict__ part,
-                                          DevParticle* __restrict__ prev,
-                                          const double* __restrict__ force, double rho0, double gx,
-                                          double gy, double gz, double dt, int wall_contact,
-                                          int* __restrict__ status) {
-    DevParticle P = *part;
-    *prev = P;
-    if (P.fixed == 0.0) {
+// (rho_p - rho0) V g; keeps the previous state in `prev`.  Called by one warp
+// per particle: lane a (< 3) updates axis a, so the chain of FP64 divisions
+// that bounds it is one axis long.
+// (`force` may have been written by the same kernel: not __restrict__.)
+__device__ __forceinline__ void rigid_one(const Geom& g, DevParticle* part, DevParticle* prev,
+                                          const double* force, double rho0, double gx, double gy,
+                                          double gz, double dt, int wall_contact, int* status) {
+    const int a = threadIdx.x & 31;
+    constexpr int WORDS = (int)(sizeof(DevParticle) / sizeof(double));
+    for (int i = a; i < WORDS; i += 32)
+        reinterpret_cast<double*>(prev)[i] = reinterpret_cast<const double*>(part)[i];
+    __syncwarp();
+    if (a >= 3) return;
+    const unsigned lanes = 7u;
+    const double D = part->d, R = 0.5 * D, rho = part->rho;
+    double x = part->x[a], u = part->u[a], w = part->w[a];
+    const double x_old = x, u_old = u, w_old = w;
+    if (part->fixed == 0.0) {
         const double PI = 3.14159265358979323846;
-        const double D = P.d, R = 0.5 * D;
         const double V = PI * D * D * D / 6.0;
-        const double m = P.rho * V, I = m * D * D / 10.0;
-        const double grav[3] = {gx, gy, gz};
-        double Ft[3];
-        for (int a = 0; a < 3; ++a) Ft[a] = force[a] + (P.rho - rho0) * V * grav[a];
-        for (int a = 0; a < 3; ++a) P.x[a] += dt * P.u[a];
-        for (int a = 0; a < 3; ++a) P.u[a] += dt * Ft[a] / m;
-        for (int a = 0; a < 3; ++a) P.w[a] += dt * force[3 + a] / I;
+        const double m = rho * V, I = m * D * D / 10.0;
+        const double grav = a == 0 ? gx : (a == 1 ? gy : gz);
+        const double Ft = force[a] + (rho - rho0) * V * grav;
+        x += dt * u;
+        u += dt * Ft / m;
+        w += dt * force[3 + a] / I;
         // a non-finite state, or a surface moving a cell or more per step,
         // is outside what the lattice can represent: report it and keep the
         // previous state so that the cell geometry stays well defined
-        bool sane = true;
-        for (int a = 0; a < 3; ++a)
-            sane = sane && isfinite(P.x[a]) && fabs(P.u[a]) < 1.0 && fabs(P.w[a]) * R < 1.0;
-        if (!sane) {
-            atomicOr(status, ST_UNSTABLE);
-            P = *prev;
+        const bool sane = isfinite(x) && fabs(u) < 1.0 && fabs(w) * R < 1.0;
+        if (!__all_sync(lanes, sane)) {
+            if (a == 0) atomicOr(status, ST_UNSTABLE);
+            x = x_old;
+            u = u_old;
+            w = w_old;
         }
-        const double L[3] = {(double)g.nx, (double)g.ny, (double)g.nz};
-        for (int a = 0; a < 3; ++a) {
-            if (a == 2 && g.bc_z) continue;
-            if (P.x[a] < 0.0) P.x[a] += L[a];
-            else if (P.x[a] >= L[a]) P.x[a] -= L[a];
-        }
-        if (g.bc_z == 2) {
+        const double L = a == 0 ? g.nx : (a == 1 ? g.ny : g.nz);
+        if (!(a == 2 && g.bc_z)) {
+            if (x < 0.0) x += L;
+            else if (x >= L) x -= L;
+        } else if (g.bc_z == 2) {
             // open boundaries: the near region must stay clear of them
-            if (P.x[2] - R - OPEN_MARGIN < 0.0 || P.x[2] + R + OPEN_MARGIN > L[2])
-                atomicOr(status, ST_DOMAIN);
-        } else if (g.bc_z) {
-            if (wall_contact) {
-                if (P.x[2] - R < 1.0) {
-                    P.x[2] = R + 1.0;
-                    if (P.u[2] < 0.0) P.u[2] = 0.0;
-                }
-                if (P.x[2] + R > L[2] - 1.0) {
-                    P.x[2] = L[2] - 1.0 - R;
-                    if (P.u[2] > 0.0) P.u[2] = 0.0;
-                }
-            } else if (P.x[2] - R < 0.0 || P.x[2] + R > L[2]) {
-                atomicOr(status, ST_DOMAIN);
+            if (x - R - OPEN_MARGIN < 0.0 || x + R + OPEN_MARGIN > L) atomicOr(status, ST_DOMAIN);
+        } else if (wall_contact) {
+            if (x - R < 1.0) {
+                x = R + 1.0;
+                if (u < 0.0) u = 0.0;
             }
+            if (x + R > L - 1.0) {
+                x = L - 1.0 - R;
+                if (u > 0.0) u = 0.0;
+            }
+        } else if (x - R < 0.0 || x + R > L) {
+            atomicOr(status, ST_DOMAIN);
         }
     }
-    store_region(g, P);
-    *part = P;
+    part->x[a] = x;
+    part->u[a] = u;
+    part->w[a] = w;
+    store_region_axis(g, *part, x, a);
 }
 
-// explicit Euler rigid-body update over dt, gravity + buoyancy
-// (rho_p - rho0) V g; keeps the previous state in `prev`.
-__global__ void k_rigid(Geom g, DevParticle* __restrict__ parts, DevParticle* __restrict__ prev,
-                        int np, const double* __restrict__ force, double rho0, double gx,
-                        double gy, double gz, double dt, int wall_contact,
-                        int* __restrict__ status) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= np) return;
+// one warp per particle
+__global__ void __launch_bounds__(32)
+    k_rigid(Geom g, DevParticle* __restrict__ parts, DevParticle* __restrict__ prev,
+            const double* __restrict__ force, double rho0, double gx, double gy, double gz,
+            double dt, int wall_contact, int* __restrict__ status) {
+    const int p = blockIdx.x;
     rigid_one(g, parts + p, prev + p, force + 6 * p, rho0, gx, gy, gz, dt, wall_contact, status);
+}
+
+// Force total and rigid-body update of particle blockIdx.x in one launch
+// (nothing else reads the force in between: no force model attached).
+__global__ void __launch_bounds__(FIN_THREADS)
+    k_finalize_rigid(Geom g, int np, long long nblk, const double* __restrict__ partials, int nsub,
+                     double* force, const double* __restrict__ charge, DevParticle* parts,
+                     DevParticle* prev, double rho0, double gx, double gy, double gz, double dt,
+                     int wall_contact, int* status) {
+    __shared__ double red[FIN_THREADS];
+    const int p = blockIdx.x;
+    finalize_block(np, nblk, partials, nsub, force, p, red, charge);
+    __syncthreads();
+    if (threadIdx.x < 32)
+        rigid_one(g, parts + p, prev + p, force + 6 * p, rho0, gx, gy, gz, dt, wall_contact, status);
 }
 
 __global__ void k_regions(Geom g, DevParticle* parts, int np) {
@@ -1242,8 +1253,16 @@ __device__ __forceinline__ void add_cell_moment(double (&acc)[6], const Geom& g,
     acc[5] += sign * (r[0] * j[1] - r[1] * j[0]);
 }
 
-// Candidate test of thread lid of particle p's box, then the warp's
+// Candidate test of one cell of particle p's box per lane, then the warp's
 // candidates one after another.  Every lane of the warp must call this.
+//
+// Warp `warp` of `warps` tests cells warp, warp + warps, ... of the box: the
+// cells a sphere uncovers lie side by side in the rows of its cap, and a warp
+// that tested a run of a row rebuilt up to a dozen of them in turn while most
+// warps had none.  A candidate is a long chain of FP64 latency, so the launch
+// takes about as long as the fullest warp (D = 24 settling, ~45 cells per
+// step: 92 us -> 61 us).
+//
 // acc != nullptr: re-mapping momentum charge of particle p (uncovered cells
 // plus, covered cells minus; moments about the new centre) added to this
 // thread's six sums.  The box holds every cell of the new sphere while the
@@ -1252,9 +1271,10 @@ template <typename T, typename C>
 __device__ __forceinline__ void refill_cells(const T* __restrict__ srcB, T* __restrict__ dst,
                                              const Geom& g, const Coll<C>& k, const Coupl& cp,
                                              const DevParticle* so, const DevParticle* sn,
-                                             int extrapolate, int side, int p, long long lid,
-                                             int* __restrict__ status, RefillWarp& w, int lane,
-                                             double (*acc)[6] = nullptr) {
+                                             int extrapolate, int side, int p, long long warp,
+                                             long long warps, int* __restrict__ status,
+                                             RefillWarp& w, int lane, double (*acc)[6] = nullptr) {
+    const long long lid = warp + lane * warps;
     bool cand = lid < (long long)side * side * side;
     int x = 0, y = 0, z = 0;
     if (cand) {
@@ -1276,21 +1296,31 @@ __device__ __forceinline__ void refill_cells(const T* __restrict__ srcB, T* __re
     const bool test_new = own_old == p + 1 || (acc && own_old == 0);
     const int own_new = test_new ? cell_owner(g, sn, cp.np, x, y, z) : -1;
     cand = own_old == p + 1 && own_new == 0;
-    if (acc && own_old == 0 && own_new == p + 1) {
-        // covered: the fluid momentum of its pre-collision populations leaves the fluid
-        C f[NQ];
-        mem_pull(srcB, g, cp, so, cp.np, (const GeoMap*)nullptr, x, y, z, lin(g, x, y, z), f,
-                 (Slots*)nullptr, status);
-        double j[3] = {0.0, 0.0, 0.0};
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            j[0] += (double)f[q] * cx(q);
-            j[1] += (double)f[q] * cy(q);
-            j[2] += (double)f[q] * cz(q);
-        }
-        add_cell_moment(*acc, g, sn[p], x, y, z, j, -1.0);
-    }
     const unsigned full = 0xffffffffu;
+    if (acc) {
+        // covered: the fluid momentum of the cell's pre-collision populations
+        // leaves the fluid; lane q pulls direction q
+        for (unsigned m = __ballot_sync(full, own_old == 0 && own_new == p + 1); m; m &= m - 1) {
+            const int src_lane = __ffs(m) - 1;
+            const int xc = __shfl_sync(full, x, src_lane), yc = __shfl_sync(full, y, src_lane),
+                      zc = __shfl_sync(full, z, src_lane);
+            if (lane < NQ)
+                w.f[0][lane] =
+                    (double)mem_pull_dir<T, C>(srcB, g, cp, so, xc, yc, zc, lane, status);
+            __syncwarp();
+            if (lane == src_lane) {
+                double j[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) {
+                    j[0] += w.f[0][q] * cx(q);
+                    j[1] += w.f[0][q] * cy(q);
+                    j[2] += w.f[0][q] * cz(q);
+                }
+                add_cell_moment(*acc, g, sn[p], x, y, z, j, -1.0);
+            }
+            __syncwarp();
+        }
+    }
     for (unsigned m = __ballot_sync(full, cand); m; m &= m - 1) {
         const int src_lane = __ffs(m) - 1;
         const int cxl = __shfl_sync(full, x, src_lane), cyl = __shfl_sync(full, y, src_lane),
@@ -1353,22 +1383,31 @@ __global__ void __launch_bounds__(REFILL_THREADS)
     const int p = blockIdx.y, lane = tid & 31;
     double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     refill_cells<T, C>(srcB, dst, g, k, cp, so, sn, extrapolate, side, p,
-                       (long long)blockIdx.x * blockDim.x + tid, status, rw[tid >> 5], lane,
+                       (long long)blockIdx.x * (REFILL_THREADS / 32) + (tid >> 5),
+                       (long long)gridDim.x * (REFILL_THREADS / 32), status, rw[tid >> 5], lane,
                        charge_part ? &acc : nullptr);
     if (!charge_part) return;
     if (tid == 0) charge_step_check(g, sn[p], so[p], status);
     charge_block_sum(acc, charge_part + ((long long)p * gridDim.x + blockIdx.x) * 6);
 }
 
-// out[p * 6 + c] = sum over the nblk refill blocks of particle p, in order.
-__global__ void k_charge_total(int np, long long nblk, const double* __restrict__ part,
-                               double* __restrict__ out) {
-    const int t = threadIdx.x;
-    if (t >= 6 * np) return;
-    const int p = t / 6, c = t - 6 * (t / 6);
+// out[c] = sum over nblk refill-block partials [blk][6]; warp c of the block's
+// six adds component c (one thread per component over 172 partials: 16 us;
+// this form 3.9 us).
+__device__ __forceinline__ void charge_total(long long nblk, const double* __restrict__ part,
+                                             double* __restrict__ out) {
+    const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double s = 0.0;
-    for (long long b = 0; b < nblk; ++b) s += part[((long long)p * nblk + b) * 6 + c];
-    out[t] = s;
+#pragma unroll 4
+    for (long long b = lane; b < nblk; b += 32) s += part[b * 6 + c];
+    s = warp_sum(s);
+    if (lane == 0) out[c] = s;
+}
+
+// one block of six warps per particle
+__global__ void __launch_bounds__(192)
+    k_charge_total(long long nblk, const double* __restrict__ part, double* __restrict__ out) {
+    charge_total(nblk, part + (long long)blockIdx.x * nblk * 6, out + blockIdx.x * 6);
 }
 
 // ---------------------------------------------------------------------------
@@ -1650,18 +1689,18 @@ __global__ void k_batch_swap(BatchCase* __restrict__ cases, BatchList l) {
     if (i < l.n) cases[l.list[i]].cur ^= 1;
 }
 
-__global__ void __launch_bounds__(256) k_batch_finalize(BatchCase* __restrict__ cases) {
-    __shared__ double red[256][6];
+__global__ void __launch_bounds__(FIN_THREADS) k_batch_finalize(BatchCase* __restrict__ cases) {
+    __shared__ double red[FIN_THREADS];
     const BatchCase& B = cases[blockIdx.x];
     const int nsub = B.kind != 0 ? B.subcycles : 1;
     finalize_block(1, B.nblk, B.partials, nsub, B.force, 0, red,
                    B.remap_charge ? B.charge : nullptr);
 }
 
-__global__ void k_batch_rigid(BatchCase* __restrict__ cases, int n, int* __restrict__ status) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n) return;
-    const BatchCase& B = cases[c];
+// one warp per case
+__global__ void __launch_bounds__(32) k_batch_rigid(BatchCase* __restrict__ cases,
+                                                    int* __restrict__ status) {
+    const BatchCase& B = cases[blockIdx.x];
     const double dt = B.kind != 0 ? (double)B.subcycles : 1.0;
     rigid_one(B.g, B.part, B.prev, B.force, B.kd.rho0, B.gravity[0], B.gravity[1], B.gravity[2],
               dt, B.wall_contact, status);
@@ -1684,7 +1723,8 @@ __global__ void __launch_bounds__(REFILL_THREADS)
     __shared__ RefillWarp rw[REFILL_THREADS / 32];
     double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     refill_cells<double, double>(B.buf[1 - cur], B.buf[cur], B.g, B.kd, B.cp, so, sn, 1,
-                                 B.refill_side, 0, local * blockDim.x + threadIdx.x, status,
+                                 B.refill_side, 0, local * (REFILL_THREADS / 32) + (threadIdx.x >> 5),
+                                 refill_blocks(B.refill_side) * (REFILL_THREADS / 32), status,
                                  rw[threadIdx.x >> 5], threadIdx.x & 31,
                                  B.remap_charge ? &acc : nullptr);
     // re-mapping charge: block partial `local` of this case (see k_refill)
@@ -1694,17 +1734,10 @@ __global__ void __launch_bounds__(REFILL_THREADS)
 }
 
 // Per case with the charge on: charge[c] = the fixed-order total of its
-// refill-block partials.  One thread per (case, component).
-__global__ void k_batch_charge_total(BatchCase* __restrict__ cases, int n) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= 6 * n) return;
-    const BatchCase& B = cases[t / 6];
-    if (!B.remap_charge) return;
-    const int c = t % 6;
-    const long long nb = refill_blocks(B.refill_side);
-    double s = 0.0;
-    for (long long k = 0; k < nb; ++k) s += B.charge_part[k * 6 + c];
-    B.charge[c] = s;
+// refill-block partials.  One block of six warps per case.
+__global__ void __launch_bounds__(192) k_batch_charge_total(BatchCase* __restrict__ cases) {
+    const BatchCase& B = cases[blockIdx.x];
+    if (B.remap_charge) charge_total(refill_blocks(B.refill_side), B.charge_part, B.charge);
 }
 
 // ---------------------------------------------------------------------------
@@ -1884,8 +1917,8 @@ cudaError_t launch_refill(int storage, const void* srcB, void* dst, const Launch
 }
 cudaError_t launch_charge_total(const Launch& L, const double* charge_part, double* charge) {
     if (L.cp.np <= 0) return cudaSuccess;
-    return launch(k_charge_total, 1, 6 * MAX_PARTICLES, L.stream, L.cp.np, refill_blocks(L.box[0]),
-                  charge_part, charge);
+    return launch(k_charge_total, L.cp.np, 192, L.stream, refill_blocks(L.box[0]), charge_part,
+                  charge);
 }
 cudaError_t launch_macro(int storage, const void* state, const Launch& L, int what, void* out) {
     switch (storage) {
@@ -1936,14 +1969,21 @@ cudaError_t launch_map(const Launch& L) {
 
 cudaError_t launch_finalize(const Launch& L, int nsub, double* force_out, const double* charge) {
     if (L.cp.np <= 0) return cudaSuccess;
-    return launch(k_finalize, L.cp.np, 256, L.stream, L.cp.np, near_blocks(L.box), L.partials, nsub,
+    return launch(k_finalize, L.cp.np, FIN_THREADS, L.stream, L.cp.np, near_blocks(L.box), L.partials, nsub,
                   force_out, charge);
 }
 cudaError_t launch_rigid_body(const Launch& L, const double* force, double gx, double gy,
                               double gz, double dt, int wall_contact) {
     if (L.cp.np <= 0) return cudaSuccess;
-    return launch(k_rigid, 1, 32, L.stream, L.g, L.parts, L.parts_prev, L.cp.np, force, L.kd.rho0, gx,
+    return launch(k_rigid, L.cp.np, 32, L.stream, L.g, L.parts, L.parts_prev, force, L.kd.rho0, gx,
                   gy, gz, dt, wall_contact, L.status);
+}
+cudaError_t launch_finalize_rigid(const Launch& L, int nsub, double* force, const double* charge,
+                                  double gx, double gy, double gz, int wall_contact) {
+    if (L.cp.np <= 0) return cudaSuccess;
+    return launch(k_finalize_rigid, L.cp.np, FIN_THREADS, L.stream, L.g, L.cp.np,
+                  near_blocks(L.box), L.partials, nsub, force, charge, L.parts, L.parts_prev,
+                  L.kd.rho0, gx, gy, gz, (double)nsub, wall_contact, L.status);
 }
 cudaError_t launch_regions(const Launch& L) {
     if (L.cp.np <= 0) return cudaSuccess;
@@ -1984,15 +2024,15 @@ cudaError_t launch_batch_swap(BatchCase* cases, BatchList l, cudaStream_t s) {
     return cudaGetLastError();
 }
 cudaError_t launch_batch_finalize(BatchCase* cases, int n, cudaStream_t s) {
-    k_batch_finalize<<<n, 256, 0, s>>>(cases);
+    k_batch_finalize<<<n, FIN_THREADS, 0, s>>>(cases);
     return cudaGetLastError();
 }
 cudaError_t launch_batch_charge_total(BatchCase* cases, int n, cudaStream_t s) {
-    k_batch_charge_total<<<(6 * n + 255) / 256, 256, 0, s>>>(cases, n);
+    k_batch_charge_total<<<n, 192, 0, s>>>(cases);
     return cudaGetLastError();
 }
 cudaError_t launch_batch_rigid(BatchCase* cases, int n, int* status, cudaStream_t s) {
-    k_batch_rigid<<<(n + 63) / 64, 64, 0, s>>>(cases, n, status);
+    k_batch_rigid<<<n, 32, 0, s>>>(cases, status);
     return cudaGetLastError();
 }
 // Device time stamp (the GPU's nanosecond global timer): end = 0 keeps it in

@@ -319,6 +319,9 @@ cudaError_t launch_to_f64(int storage, const void* in, double* out, long long co
 // is taken off the totals
 cudaError_t launch_finalize(const Launch& L, int nsub, double* force_out,
                             const double* charge = nullptr);
+// the force total and the rigid-body update (dt = nsub) in one launch
+cudaError_t launch_finalize_rigid(const Launch& L, int nsub, double* force, const double* charge,
+                                  double gx, double gy, double gz, int wall_contact);
 cudaError_t launch_regions(const Launch& L);
 // batched ensemble (all cases on one stream; see lbm_batch.cu)
 cudaError_t launch_batch_regions(BatchCase* cases, int n, cudaStream_t s);
