@@ -50,16 +50,18 @@ __host__ __device__ constexpr double wq(int q) {
     return q == 0 ? 1.0 / 3.0 : (q <= 6 ? 1.0 / 18.0 : 1.0 / 36.0);
 }
 
-// Particle record in device memory (160 B).  `reg` caches the near-particle
-// region of the current state (see axis_range): per axis {cell start, cell
-// count, tile start, tile count}, recomputed whenever the state changes.
+// Particle record in device memory (176 B).  Recomputed whenever the state
+// changes (store_region): `reg`, the near-particle region (see axis_range),
+// per axis {cell start, cell count, tile start, tile count}; xi + xf, the
+// centre as a cell index and an FP32 remainder (see inside_f).
 struct DevParticle {
     double x[3], u[3], w[3];
     double d, r, rho, fixed;
-    double pad;
     int reg[12];
-    int pad2[2];
+    int xi[3];
+    float xf[3];
 };
+static_assert(sizeof(DevParticle) % sizeof(double) == 0, "copied as doubles");
 
 // Lattice geometry and tiling.  A tile is one thread block: tx * ty cells in
 // one z plane.
@@ -147,9 +149,48 @@ __device__ __forceinline__ bool point_inside(const Geom& g, const DevParticle& P
     return norm2_rn(dx, dy, dz) <= mul_rn(P.r, P.r);
 }
 
+// ---- FP32 filter of the geometric predicates ----------------------------------
+// The FP64 predicates cost ~25 operations on a pipe of 2 lanes per SM.  Offsets
+// from a centre are known to ~1e-7 of their size in FP32 (cell indices minus
+// xi are exact, xf is a rounded remainder), so the squared distance is off by
+// less than 3e-7 d^2 + 2.2e-7 d; a point whose squared distance differs from
+// r^2 by more than 4e-6 (r^2 + r + 1) is decided in FP32, the few others by
+// the FP64 form: the same decisions everywhere.
+
+// Minimum-image offset along axis a of the point i + add from P's centre.
+// (A wrapped offset that the FP64 form would leave, or the reverse, has a
+// length of half the domain, beyond any sphere.)
+__device__ __forceinline__ float offset_f(const DevParticle& P, int a, int i, float add, int n,
+                                          bool periodic) {
+    float d = (float)(i - P.xi[a]) + (add - P.xf[a]);
+    if (periodic) {
+        const float L = (float)n, h = 0.5f * L;
+        if (d > h) d -= L;
+        else if (d < -h) d += L;
+    }
+    return d;
+}
+__device__ __forceinline__ float margin_f(float r) { return 4e-6f * (r * r + r + 1.0f); }
+// 1: inside or on the sphere of radius r, 0: outside, -1: too close to tell
+__device__ __forceinline__ int inside_f(float d2, float r) {
+    const float r2 = r * r, m = margin_f(r);
+    return d2 > r2 + m ? 0 : (d2 < r2 - m ? 1 : -1);
+}
+// Offsets of cell (x, y, z)'s centre and its squared distance from P's centre.
+struct CellOffset {
+    float dx, dy, dz;
+    __device__ __forceinline__ float d2() const { return dx * dx + dy * dy + dz * dz; }
+};
+__device__ __forceinline__ CellOffset cell_offset(const Geom& g, const DevParticle& P, int x, int y,
+                                                  int z) {
+    return CellOffset{offset_f(P, 0, x, 0.5f, g.nx, true), offset_f(P, 1, y, 0.5f, g.ny, true),
+                      offset_f(P, 2, z, 0.5f, g.nz, !g.bc_z)};
+}
+
 __device__ __forceinline__ bool cell_inside(const Geom& g, const DevParticle& P, int x, int y,
                                             int z) {
-    return point_inside(g, P, x + 0.5, y + 0.5, z + 0.5);
+    const int in = inside_f(cell_offset(g, P, x, y, z).d2(), (float)P.r);
+    return in >= 0 ? in != 0 : point_inside(g, P, x + 0.5, y + 0.5, z + 0.5);
 }
 
 // Owner of a cell under a particle set: 0 fluid, s+1 inside particle s.
@@ -243,7 +284,7 @@ __device__ __forceinline__ bool spans_meet(int a, int la, int r, int lr, int n) 
     return range_off(a, r, n) < lr || range_off(r, a, n) < la;
 }
 
-// Cache axis a of the region of a particle centred at x in P.reg.
+// Cache axis a of the region, and of the split centre, of a particle centred at x.
 __device__ inline void store_region_axis(const Geom& g, DevParticle& P, double x, int a) {
     const AxisRange r = axis_range(x, P.r, a == 0 ? g.nx : (a == 1 ? g.ny : g.nz),
                                    a == 0 ? g.tx : (a == 1 ? g.ty : g.tz),
@@ -252,9 +293,12 @@ __device__ inline void store_region_axis(const Geom& g, DevParticle& P, double x
     P.reg[4 * a + 1] = r.clen;
     P.reg[4 * a + 2] = r.tlo;
     P.reg[4 * a + 3] = r.tlen;
+    const double fl = floor(x);
+    P.xi[a] = (int)fl;
+    P.xf[a] = (float)(x - fl);
 }
 
-// Cache the region of P's current state in P.reg.
+// Cache the region and the split centre of P's current state.
 __device__ inline void store_region(const Geom& g, DevParticle& P) {
     for (int a = 0; a < 3; ++a) store_region_axis(g, P, P.x[a], a);
 }
@@ -708,36 +752,45 @@ __device__ inline int solid_count(const Geom& g, const DevParticle& P, int x, in
 }
 
 // solid_count with the n^3 samples spread over the 32 lanes of a warp: every
-// lane passes the same cell; all lanes must call it (warp-synchronous).  Same
-// predicate and the same integer count as solid_count.
-__device__ inline int solid_count_warp(const Geom& g, const DevParticle& P, int x, int y, int z,
-                                       int n, int lane) {
+// lane passes the same cell, whose centre offset is c; all lanes must call it
+// (warp-synchronous).  Same predicate (FP32 filter, FP64 where it cannot tell)
+// and the same integer count as solid_count.
+__device__ inline int solid_count_warp(const Geom& g, const DevParticle& P, const CellOffset& c,
+                                       int x, int y, int z, int n, int lane) {
     const bool pow2 = (n & (n - 1)) == 0;
+    const int sh = 31 - __clz(n);
     const double h = 0.5 / n;
-    const double X = x, Y = y, Z = z;
+    const float r = (float)P.r, hf = 1.0f / (float)n;
     int inside = 0;
     for (int s = lane; s < n * n * n; s += 32) {
-        const int i = s % n, j = (s / n) % n, k = s / (n * n);
-        const double pz = Z + (pow2 ? (2 * k + 1) * h : (k + 0.5) / n);
-        const double py = Y + (pow2 ? (2 * j + 1) * h : (j + 0.5) / n);
-        const double px = X + (pow2 ? (2 * i + 1) * h : (i + 0.5) / n);
-        inside += point_inside(g, P, px, py, pz) ? 1 : 0;
+        const int i = pow2 ? s & (n - 1) : s % n, j = pow2 ? (s >> sh) & (n - 1) : (s / n) % n,
+                  k = pow2 ? s >> (2 * sh) : s / (n * n);
+        const float dx = c.dx + (((float)i + 0.5f) * hf - 0.5f),
+                    dy = c.dy + (((float)j + 0.5f) * hf - 0.5f),
+                    dz = c.dz + (((float)k + 0.5f) * hf - 0.5f);
+        int in = inside_f(dx * dx + dy * dy + dz * dz, r);
+        if (in < 0) {
+            const double pz = z + (pow2 ? (2 * k + 1) * h : (k + 0.5) / n);
+            const double py = y + (pow2 ? (2 * j + 1) * h : (j + 0.5) / n);
+            const double px = x + (pow2 ? (2 * i + 1) * h : (i + 0.5) / n);
+            in = point_inside(g, P, px, py, pz) ? 1 : 0;
+        }
+        inside += in;
     }
     return __reduce_add_sync(0xffffffffu, inside);
 }
 
-// The quick part of solid_count: 0 or n^3 for cells wholly outside / inside
-// the sphere, -1 for cells that need the samples.
-__device__ inline int solid_count_quick(const Geom& g, const DevParticle& P, int x, int y, int z,
-                                        int n) {
-    double dx, dy, dz;
-    separation(g, x + 0.5, y + 0.5, z + 0.5, P, dx, dy, dz);
-    double ax = fabs(dx), ay = fabs(dy), az = fabs(dz);
-    double nxd = fmax(ax - 0.5, 0.0), nyd = fmax(ay - 0.5, 0.0), nzd = fmax(az - 0.5, 0.0);
-    double R2 = mul_rn(P.r, P.r);
-    if (norm2_rn(nxd, nyd, nzd) > R2 * (1.0 + 1e-12) + 1e-9) return 0;
-    double fxd = ax + 0.5, fyd = ay + 0.5, fzd = az + 0.5;
-    if (norm2_rn(fxd, fyd, fzd) < R2 * (1.0 - 1e-12) - 1e-9) return n * n * n;
+// The quick part of solid_count for the cell with centre offset c: 0 or n^3
+// for cells wholly outside / inside the sphere by more than the FP32 margin,
+// -1 for cells that need the samples.
+__device__ inline int solid_count_quick(const DevParticle& P, const CellOffset& c, int n) {
+    const float r = (float)P.r, m = margin_f(r + 2.0f);
+    const float ax = fabsf(c.dx), ay = fabsf(c.dy), az = fabsf(c.dz);
+    const float ux = fmaxf(ax - 0.5f, 0.0f), uy = fmaxf(ay - 0.5f, 0.0f),
+                uz = fmaxf(az - 0.5f, 0.0f);
+    if (ux * ux + uy * uy + uz * uz > r * r + m) return 0;
+    const float fx = ax + 0.5f, fy = ay + 0.5f, fz = az + 0.5f;
+    if (fx * fx + fy * fy + fz * fz < r * r - m) return n * n * n;
     return -1;
 }
 
@@ -782,17 +835,30 @@ __device__ __forceinline__ int mapped_owner(const Geom& g, const DevParticle* pa
 }
 
 // ---- MEM link geometry ---------------------------------------------------------
-// delta: smallest root t of |x + t c - X| = R, clamped to [0, 1].
-__device__ inline double link_delta(const Geom& g, const DevParticle& P, double px, double py,
-                                    double pz, int ccx, int ccy, int ccz) {
-    double dx, dy, dz;
-    separation(g, px, py, pz, P, dx, dy, dz);
-    double a = (double)(ccx * ccx + ccy * ccy + ccz * ccz);
-    double b = dx * ccx + dy * ccy + dz * ccz;
-    double c = (dx * dx + dy * dy + dz * dz) - P.r * P.r;
+// FP64 offset of cell (x, y, z)'s centre from P's centre (minimum image; the
+// FP32 offsets tell which image, so no FP64 comparisons are needed).
+__device__ __forceinline__ void centre_offset(const Geom& g, const DevParticle& P, int x, int y,
+                                              int z, double (&r)[3]) {
+    const int c[3] = {x, y, z}, n[3] = {g.nx, g.ny, g.nz};
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const float d = (float)(c[a] - P.xi[a]) + (0.5f - P.xf[a]), h = 0.5f * (float)n[a];
+        int i = c[a];
+        if (a < 2 || !g.bc_z) i += d > h ? -n[a] : (d < -h ? n[a] : 0);
+        r[a] = ((double)i + 0.5) - P.x[a];
+    }
+}
+
+// delta: smallest root t of |r + t c| = R, clamped to [0, 1]; r the offset of
+// the fluid cell's centre, c the link's direction (|c|^2 = 1 or 2).
+__device__ __forceinline__ double link_delta(const DevParticle& P, const double (&r)[3], double ccx,
+                                             double ccy, double ccz, bool axis) {
+    const double a = axis ? 1.0 : 2.0;
+    const double b = r[0] * ccx + r[1] * ccy + r[2] * ccz;
+    const double c = (r[0] * r[0] + r[1] * r[1] + r[2] * r[2]) - P.r * P.r;
     double disc = b * b - a * c;
     if (disc < 0.0) disc = 0.0;
-    double t = (-b - sqrt(disc)) / a;
+    const double t = (-b - sqrt(disc)) * (axis ? 1.0 : 0.5);
     return t < 0.0 ? 0.0 : (t > 1.0 ? 1.0 : t);
 }
 

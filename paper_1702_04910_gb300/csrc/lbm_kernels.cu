@@ -215,12 +215,17 @@ __device__ __forceinline__ double mem_link(const T* __restrict__ src, const Geom
         return 0.0;
     }
     const DevParticle& P = parts[owner - 1];
-    const double xc = x + 0.5, yc = y + 0.5, zc = z + 0.5;
-    const double delta =
-        cp.variant == 0 ? 0.5 : link_delta(g, P, xc, yc, zc, rcx(qp), rcy(qp), rcz(qp));
-    const double xb[3] = {xc + delta * cqx, yc + delta * cqy, zc + delta * cqz};
+    // every offset from the centre follows from the cell's: x_b - X_p = r + delta c
+    double arm[3];
+    centre_offset(g, P, x, y, z, arm);
+    const double delta = cp.variant == 0 ? 0.5 : link_delta(P, arm, cqx, cqy, cqz, qp <= 6);
+    arm[0] += delta * cqx;
+    arm[1] += delta * cqy;
+    arm[2] += delta * cqz;
     double v[3];
-    body_velocity(g, P, xb[0], xb[1], xb[2], v[0], v[1], v[2]);
+    v[0] = P.u[0] + (P.w[1] * arm[2] - P.w[2] * arm[1]);
+    v[1] = P.u[1] + (P.w[2] * arm[0] - P.w[0] * arm[2]);
+    v[2] = P.u[2] + (P.w[0] * arm[1] - P.w[1] * arm[0]);
     const double vc = v[0] * cqx + v[1] * cqy + v[2] * cqz;
     const double ftqp = ld_pdf(src + (long long)qp * g.n + idx, qp);  // f~_qp(x)
     const double wr = 3.0 * wq(qp) * cp.rho0;                 // w_q / c_s^2 * rho0
@@ -257,21 +262,22 @@ __device__ __forceinline__ double mem_link(const T* __restrict__ src, const Geom
                     const double f3 = ld_pdf(src + (long long)qp * g.n + lin(g, x3, y3, z3), qp);
                     const double fq2 = ld_pdf(src + (long long)q * g.n + lin(g, x2, y2, z2), q);
                     own_momentum(src, g, idx, mc);
-                    const double d1 = (1.0 + delta) * (1.0 + delta);
-                    const double k0 = (1.0 - 2.0 * delta - 2.0 * delta * delta) / d1;
-                    const double km1 = delta * delta / d1;
-                    const double alpha = 4.0 / d1;
+                    const double d1 = 1.0 / ((1.0 + delta) * (1.0 + delta));
+                    const double k0 = (1.0 - 2.0 * delta - 2.0 * delta * delta) * d1;
+                    const double km1 = delta * delta * d1;
+                    const double alpha = 4.0 * d1;
                     // (1 - |lambda_-|) n^-_qp(x, t), rebuilt from the stored values
                     const double odd = 0.5 * (ftqp - fq) -
                                        3.0 * wq(qp) * (cqx * mc.j[0] + cqy * mc.j[1] + cqz * mc.j[2]);
                     val = ftqp + k0 * (f2 - fq) + km1 * (f3 - fq2) - alpha * wr * vc +
-                          cp.mr_cpc / d1 * odd;
+                          cp.mr_cpc * d1 * odd;
                     mr_done = true;
                 }
             }
             if (!mr_done) {
-                const double k0 = (1.0 - 2.0 * delta) / (1.0 + 2.0 * delta);
-                const double alpha = 4.0 / (1.0 + 2.0 * delta);
+                const double d1 = 1.0 / (1.0 + 2.0 * delta);
+                const double k0 = (1.0 - 2.0 * delta) * d1;
+                const double alpha = 4.0 * d1;
                 val = ftqp + k0 * f2 - k0 * fq - alpha * wr * vc;
             }
             cli_done = true;
@@ -279,11 +285,10 @@ __device__ __forceinline__ double mem_link(const T* __restrict__ src, const Geom
     }
     if (!cli_done) val = ftqp - 2.0 * wr * vc;
     if (ft) {
-        double F[3], arm[3], Tq[3];
+        double F[3], Tq[3];
         F[0] = (cqx - v[0]) * ftqp - (-cqx - v[0]) * val;
         F[1] = (cqy - v[1]) * ftqp - (-cqy - v[1]) * val;
         F[2] = (cqz - v[2]) * ftqp - (-cqz - v[2]) * val;
-        separation(g, xb[0], xb[1], xb[2], P, arm[0], arm[1], arm[2]);
         cross3(arm, F, Tq);
         ft[0] = F[0];
         ft[1] = F[1];
@@ -716,14 +721,93 @@ __global__ void __launch_bounds__(PAIR_TX * PAIR_TY, 768 / (PAIR_TX * PAIR_TY))
 // cell is solid iff its centre is within R, R6), so its pull is the plain one.
 __device__ __forceinline__ bool clear_of_particles(const Geom& g, const DevParticle* sp, int np,
                                                    int x, int y, int z) {
-    const double xc = x + 0.5, yc = y + 0.5, zc = z + 0.5;
     for (int s = 0; s < np; ++s) {
-        double dx, dy, dz;
-        separation(g, xc, yc, zc, sp[s], dx, dy, dz);
-        const double r = sp[s].r + 1.5;
-        if (dx * dx + dy * dy + dz * dz <= r * r) return false;
+        const float r = (float)sp[s].r + 1.5f;
+        if (!(cell_offset(g, sp[s], x, y, z).d2() > r * r + margin_f(r))) return false;
     }
     return true;
+}
+
+// Phase 1 of the MEM pull for a cell at offsets (kx, ky, kz) of particle p's
+// region box, owners from the box's map: `own` collects the directions whose
+// upstream cell is solid, `wall` those that cross a closed wall.  All 18 map
+// entries are loaded before the first is used, then all PDFs: the pull is two
+// memory latencies long instead of one per direction (with the link terms from
+// one centre offset: k_near MEM CLI, D = 8 FP64 32.7 us -> 23.7 us, D = 24
+// FP32 37.7 -> 31.9).  A neighbour outside the
+// box is fluid for one particle (the box holds every cell within two of the
+// sphere's surface); with more it is looked up in the other boxes.
+template <int Q>
+struct NearOwners {
+    __device__ __forceinline__ static void run(const Geom& g, const DevParticle* sp, int np,
+                                               const GeoMap& gm, const unsigned short* m0,
+                                               const NbrOff& o, unsigned in, int x, int y, int z,
+                                               unsigned short (&e)[NQ], unsigned& wall) {
+        // bits of `in`: x - 1, x + 1, y - 1, y + 1, z - 1, z + 1 lie in the box
+        constexpr int dx = -cx(Q), dy = -cy(Q), dz = -cz(Q);
+        constexpr unsigned need = (dx < 0 ? 1u : dx > 0 ? 2u : 0u) | (dy < 0 ? 4u : dy > 0 ? 8u : 0u) |
+                                  (dz < 0 ? 16u : dz > 0 ? 32u : 0u);
+        e[Q] = 0;
+        if ((dz < 0 && o.zlo) || (dz > 0 && o.zhi)) {
+            wall |= 1u << Q;
+        } else if ((in & need) == need) {
+            e[Q] = __ldg(m0 + (dx + gm.ex * (dy + (long long)gm.ey * dz)));
+        } else if (np > 1) {
+            const Nbr b = make_nbr(g, x, y, z);
+            int xs, ys, zs;
+            shifted<Q>(b, x, y, z, -1, xs, ys, zs);
+            e[Q] = (unsigned short)mapped_owner(g, sp, np, gm, xs, ys, zs);
+        }
+        NearOwners<Q + 1>::run(g, sp, np, gm, m0, o, in, x, y, z, e, wall);
+    }
+};
+template <>
+struct NearOwners<NQ> {
+    __device__ __forceinline__ static void run(const Geom&, const DevParticle*, int, const GeoMap&,
+                                               const unsigned short*, const NbrOff&, unsigned, int,
+                                               int, int, unsigned short (&)[NQ], unsigned&) {}
+};
+template <typename T, typename C, int Q>
+struct NearPull {
+    __device__ __forceinline__ static void run(const T* __restrict__ src, const Geom& g,
+                                               const NbrOff& o, long long idx, unsigned solid,
+                                               unsigned wall, C (&f)[NQ]) {
+        if ((wall >> Q) & 1u)
+            f[Q] = PdfStore<T>::template load<C>(src + (long long)opp(Q) * g.n + idx, opp(Q));
+        else if (!((solid >> Q) & 1u))
+            f[Q] = PdfStore<T>::template load<C>(src + (long long)Q * g.n + idx + upstream_off<Q>(o), Q);
+        NearPull<T, C, Q + 1>::run(src, g, o, idx, solid, wall, f);
+    }
+};
+template <typename T, typename C>
+struct NearPull<T, C, NQ> {
+    __device__ __forceinline__ static void run(const T* __restrict__, const Geom&, const NbrOff&,
+                                               long long, unsigned, unsigned, C (&)[NQ]) {}
+};
+template <typename T, typename C>
+__device__ __forceinline__ void near_pull(const T* __restrict__ src, const Geom& g,
+                                          const DevParticle* sp, int np, const GeoMap& gm, int p,
+                                          int kx, int ky, int kz, int x, int y, int z,
+                                          long long idx, C (&f)[NQ], unsigned& cut, int* status) {
+    f[0] = PdfStore<T>::template load<C>(src + idx, 0);
+    if (kx >= gm.ex || ky >= gm.ey || kz >= gm.ez) {  // a box larger than its map: report, no access
+        atomicOr(status, ST_BOUNDS);
+        return;
+    }
+    const int* R = sp[p].reg;
+    const unsigned in = (kx > 0 ? 1u : 0u) | (kx + 1 < min(R[1], gm.ex) ? 2u : 0u) |
+                        (ky > 0 ? 4u : 0u) | (ky + 1 < min(R[5], gm.ey) ? 8u : 0u) |
+                        (kz > 0 ? 16u : 0u) | (kz + 1 < min(R[9], gm.ez) ? 32u : 0u);
+    const NbrOff o = make_off(g, x, y, z);
+    const unsigned short* m0 = gm.map + (((long long)p * gm.ez + kz) * gm.ey + ky) * gm.ex + kx;
+    unsigned short e[NQ];
+    unsigned wall = 0;
+    NearOwners<1>::run(g, sp, np, gm, m0, o, in, x, y, z, e, wall);
+    unsigned solid = 0;
+#pragma unroll
+    for (int q = 1; q < NQ; ++q) solid |= e[q] ? 1u << q : 0u;
+    NearPull<T, C, 1>::run(src, g, o, idx, solid, wall, f);
+    cut = solid;
 }
 
 template <typename T, typename C, int KIND, bool NOSTREAM>
@@ -807,15 +891,13 @@ __device__ __forceinline__ void near_block(const T* __restrict__ src, T* __restr
             if (clear_of_particles(g, sp, cp.np, x, y, z)) {
                 pull_plain(src, g, x, y, z, idx, f);  // no solid neighbour, no link
             } else {
-                const Nbr b = make_nbr(g, x, y, z);
-                f[0] = PdfStore<T>::template load<C>(src + idx, 0);
-                MemPull<T, C, 1>::run(src, g, sp, cp.np, &gm, b, x, y, z, idx, f, cut, status);
+                near_pull(src, g, sp, cp.np, gm, p, kx, ky, kz, x, y, z, idx, f, cut, status);
             }
         }
         mem_links_warp(src, g, cp, sp, &gm, x, y, z, idx, cut, f, slots, status, lw[tid >> 5],
                        tid & 31);
         if (fluid) {
-            if (collide_fluid(f, k)) atomicOr(status, ST_FLUID);
+            if (collide_cell(f, k)) atomicOr(status, ST_FLUID);
             store_own(dst, g, idx, f);
         }
     }
@@ -876,7 +958,9 @@ __global__ void __launch_bounds__(256)
 // (ky, kz the same on every lane).  PSM: cells wholly outside or inside the
 // sphere take the quick count; the warp then samples each remaining cell of
 // the row together (two of the 64 samples per lane for n = 4), so a row costs
-// a few cooperative sample sets instead of one 64-sample loop per lane.
+// a few cooperative sample sets instead of one 64-sample loop per lane.  The
+// samples are decided in FP32 wherever that can tell (inside_f): D = 8, n = 4
+// 18.1 us -> 5.7 us.
 template <int KIND>
 __device__ __forceinline__ void map_cell(const Geom& g, const Coupl& cp, const DevParticle* sp,
                                          unsigned short* __restrict__ map, int ex, int ey, int ez,
@@ -893,14 +977,16 @@ __device__ __forceinline__ void map_cell(const Geom& g, const Coupl& cp, const D
         return;
     }
     const int lane = threadIdx.x & 31;
-    const int quick = valid ? solid_count_quick(g, sp[p], x, y, z, cp.subsample) : 0;
+    const CellOffset co = cell_offset(g, sp[p], x, y, z);
+    const int quick = valid ? solid_count_quick(sp[p], co, cp.subsample) : 0;
     if (valid && quick >= 0) *out = (unsigned short)quick;
     unsigned todo = __ballot_sync(0xffffffffu, valid && quick < 0);
     while (todo) {
         const int c = __ffs(todo) - 1;
         todo &= todo - 1;
         const int xc = __shfl_sync(0xffffffffu, x, c);
-        const int cnt = solid_count_warp(g, sp[p], xc, y, z, cp.subsample, lane);
+        const CellOffset cc{__shfl_sync(0xffffffffu, co.dx, c), co.dy, co.dz};
+        const int cnt = solid_count_warp(g, sp[p], cc, xc, y, z, cp.subsample, lane);
         if (lane == c) *out = (unsigned short)cnt;
     }
 }
@@ -1100,47 +1186,82 @@ __device__ __forceinline__ C mem_pull_dir(const T* __restrict__ src, const Geom&
 
 // Per-warp scratch of the refill.
 struct RefillWarp {
-    double f[3][NQ];  // pre-collision values of the extrapolation cells
+    double f[3][NQ];  // pre-collision values of the extrapolation cells; f[0]: the rebuilt ones
     double r[NQ];     // densities of the usable neighbours (no extrapolation cell)
     int ok[NQ];
 };
 
+// Sum over the warp, the same bits on every lane.
+__device__ __forceinline__ double warp_sum_all(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// q_n = argmax_q n . c_q, lowest q on ties, n the unit vector along r.  Lane q
+// weighs direction q, in FP32 on r itself;
+// where two directions come within the FP32 error (exact ties on a lattice
+// symmetry plane do) the unit vector and the comparison are FP64, as defined.
+// All lanes call it with the same r and get the same answer.
+__device__ __forceinline__ int normal_direction(const double (&r)[3], int lane) {
+    const unsigned full = 0xffffffffu;
+    const bool dir = lane >= 1 && lane < NQ;
+    const float rx = (float)r[0], ry = (float)r[1], rz = (float)r[2];
+    const float d = dir ? rx * rcx(lane) + ry * rcy(lane) + rz * rcz(lane) : 0.0f;
+    const float best = __uint_as_float(__reduce_max_sync(full, __float_as_uint(fmaxf(d, 0.0f))));
+    const unsigned near = __ballot_sync(
+        full, dir && d >= best - 1e-5f * (fabsf(rx) + fabsf(ry) + fabsf(rz)));
+    if (__popc(near) == 1) return __ffs(near) - 1;
+    const double len = sqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]);
+    double nrm[3] = {r[0], r[1], r[2]};
+    if (len > 0.0)
+        for (int a = 0; a < 3; ++a) nrm[a] /= len;
+    double bd = dir ? nrm[0] * rcx(lane) + nrm[1] * rcy(lane) + nrm[2] * rcz(lane) : -1e300;
+    int bq = dir ? lane : NQ;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double od = __shfl_xor_sync(full, bd, o);
+        const int oq = __shfl_xor_sync(full, bq, o);
+        if (od > bd || (od == bd && oq < bq)) {
+            bd = od;
+            bq = oq;
+        }
+    }
+    return bq;
+}
+
 // Rebuilds candidate cell (x, y, z) of particle p; all 32 lanes call it with
-// the same cell.  The pulls are spread over the lanes, the rest is computed
-// by every lane alike and lane 0 stores.  jm receives the momentum
-// sum_q c_q f_q of the rebuilt pre-collision populations (every lane).
+// the same cell.  The pulls are spread over the lanes, and lane q combines and
+// corrects population q; the collision is computed by every lane alike and
+// lane 0 stores.  jm receives the momentum sum_q c_q f_q of the rebuilt
+// pre-collision populations (every lane; only with `momentum`).
+//
+// One cell is one chain of FP64 and memory latency on an otherwise idle GPU,
+// so the chain's length is what counts: predicates filtered in FP32, the
+// normal direction and the 19 corrections across the lanes (every lane doing
+// all of it in FP64: 47 us for one cell, 61 us for the 45 of a D = 24 step;
+// this form 30 us and 36 us).
 template <typename T, typename C>
 __device__ __forceinline__ void refill_warp(const T* __restrict__ srcB, T* __restrict__ dst,
                                             const Geom& g, const Coll<C>& k, const Coupl& cp,
                                             const DevParticle* so, const DevParticle* sn,
                                             int extrapolate, int p, int x, int y, int z,
                                             int* __restrict__ status, RefillWarp& w, int lane,
-                                            double (&jm)[3]) {
+                                            bool momentum, double (&jm)[3]) {
     const DevParticle& Pn = sn[p];
-    const double xc = x + 0.5, yc = y + 0.5, zc = z + 0.5;
-    double v[3];
-    body_velocity(g, Pn, xc, yc, zc, v[0], v[1], v[2]);
+    double r[3], v[3];
+    centre_offset(g, Pn, x, y, z, r);
+    v[0] = Pn.u[0] + (Pn.w[1] * r[2] - Pn.w[2] * r[1]);
+    v[1] = Pn.u[1] + (Pn.w[2] * r[0] - Pn.w[0] * r[2]);
+    v[2] = Pn.u[2] + (Pn.w[0] * r[1] - Pn.w[1] * r[0]);
     C fn[NQ];
     int m = 0;
-    int qn = 1;
     int nbx[3], nby[3], nbz[3];
     if (extrapolate) {
-        double nrm[3];
-        separation(g, xc, yc, zc, Pn, nrm[0], nrm[1], nrm[2]);
-        double len = sqrt(nrm[0] * nrm[0] + nrm[1] * nrm[1] + nrm[2] * nrm[2]);
-        if (len > 0.0)
-            for (int a = 0; a < 3; ++a) nrm[a] /= len;
-        double best = -1e300;
-        for (int q = 1; q < NQ; ++q) {
-            double d = nrm[0] * cx(q) + nrm[1] * cy(q) + nrm[2] * cz(q);
-            if (d > best) {
-                best = d;
-                qn = q;
-            }
-        }
+        const int qn = normal_direction(r, lane);
         for (int kk = 1; kk <= 3; ++kk) {
-            int xx = wrap_i(x + kk * cx(qn), g.nx), yy = wrap_i(y + kk * cy(qn), g.ny),
-                zz = z + kk * cz(qn);
+            int xx = wrap_i(x + kk * rcx(qn), g.nx), yy = wrap_i(y + kk * rcy(qn), g.ny),
+                zz = z + kk * rcz(qn);
             if (g.bc_z) {
                 if (zz < 0 || zz >= g.nz) break;
             } else {
@@ -1154,6 +1275,8 @@ __device__ __forceinline__ void refill_warp(const T* __restrict__ srcB, T* __res
             ++m;
         }
     }
+    const bool dir = lane < NQ;
+    const double cxl = dir ? rcx(lane) : 0, cyl = dir ? rcy(lane) : 0, czl = dir ? rcz(lane) : 0;
     if (m > 0) {
         // the m x 19 pulls, lane by lane
         for (int i = lane; i < m * NQ; i += 32) {
@@ -1162,30 +1285,21 @@ __device__ __forceinline__ void refill_warp(const T* __restrict__ srcB, T* __res
                 (double)mem_pull_dir<T, C>(srcB, g, cp, so, nbx[jn], nby[jn], nbz[jn], q, status);
         }
         __syncwarp();
-        if (m == 1) {
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) fn[q] = (C)w.f[0][q];
-        } else if (m == 2) {
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) fn[q] = (C)2 * (C)w.f[0][q] - (C)w.f[1][q];
-        } else {
-#pragma unroll
-            for (int q = 0; q < NQ; ++q)
-                fn[q] = (C)3 * (C)w.f[0][q] - (C)3 * (C)w.f[1][q] + (C)w.f[2][q];
+        C fl = (C)0;
+        if (dir) {
+            if (m == 1) fl = (C)w.f[0][lane];
+            else if (m == 2) fl = (C)2 * (C)w.f[0][lane] - (C)w.f[1][lane];
+            else fl = (C)3 * (C)w.f[0][lane] - (C)3 * (C)w.f[1][lane] + (C)w.f[2][lane];
         }
         // velocity constraint: only the momentum moment changes (sum_q c_qa^2 = 10)
-        double j[3] = {0.0, 0.0, 0.0};
+        const double dj0 = cp.rho0 * v[0] - warp_sum_all((double)fl * cxl);
+        const double dj1 = cp.rho0 * v[1] - warp_sum_all((double)fl * cyl);
+        const double dj2 = cp.rho0 * v[2] - warp_sum_all((double)fl * czl);
+        fl = (C)((double)fl + (cxl * dj0 + cyl * dj1 + czl * dj2) / 10.0);
+        if (dir) w.f[0][lane] = (double)fl;
+        __syncwarp();
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            j[0] += (double)fn[q] * cx(q);
-            j[1] += (double)fn[q] * cy(q);
-            j[2] += (double)fn[q] * cz(q);
-        }
-        double dj[3];
-        for (int a = 0; a < 3; ++a) dj[a] = cp.rho0 * v[a] - j[a];
-#pragma unroll
-        for (int q = 0; q < NQ; ++q)
-            fn[q] = (C)((double)fn[q] + (cx(q) * dj[0] + cy(q) * dj[1] + cz(q) * dj[2]) / 10.0);
+        for (int q = 0; q < NQ; ++q) fn[q] = (C)w.f[0][q];
     } else {
         double rbar = cp.rho0;
         if (extrapolate) {
@@ -1198,15 +1312,15 @@ __device__ __forceinline__ void refill_warp(const T* __restrict__ srcB, T* __res
                 else zz = wrap_i(zz, g.nz);
                 if (ok)
                     ok = !cell_owner(g, so, cp.np, xx, yy, zz) && !cell_owner(g, sn, cp.np, xx, yy, zz);
-                double r = 0.0;
+                double rho = 0.0;
                 if (ok) {
                     C fq[NQ];
                     mem_pull(srcB, g, cp, so, cp.np, (const GeoMap*)nullptr, xx, yy, zz,
                              lin(g, xx, yy, zz), fq, (Slots*)nullptr, status);
 #pragma unroll
-                    for (int qq = 0; qq < NQ; ++qq) r += (double)fq[qq];
+                    for (int qq = 0; qq < NQ; ++qq) rho += (double)fq[qq];
                 }
-                w.r[q] = r;
+                w.r[q] = rho;
                 w.ok[q] = ok ? 1 : 0;
             }
             __syncwarp();
@@ -1220,15 +1334,18 @@ __device__ __forceinline__ void refill_warp(const T* __restrict__ srcB, T* __res
             if (cnt > 0) rbar = sum / cnt;
         }
         equilibrium((C)rbar, (C)v[0], (C)v[1], (C)v[2], k.rho0, fn);
-    }
-    jm[0] = jm[1] = jm[2] = 0.0;
+        if (lane == 0)
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        jm[0] += (double)fn[q] * cx(q);
-        jm[1] += (double)fn[q] * cy(q);
-        jm[2] += (double)fn[q] * cz(q);
+            for (int q = 0; q < NQ; ++q) w.f[0][q] = (double)fn[q];
+        __syncwarp();
     }
-    collide_fluid(fn, k);
+    if (momentum) {
+        const double fl = dir ? w.f[0][lane] : 0.0;
+        jm[0] = warp_sum_all(fl * cxl);
+        jm[1] = warp_sum_all(fl * cyl);
+        jm[2] = warp_sum_all(fl * czl);
+    }
+    collide_cell(fn, k);
     if (lane == 0) {
         if (x < 0 || x >= g.nx || y < 0 || y >= g.ny || z < 0 || z >= g.nz)
             atomicOr(status, ST_BOUNDS);
@@ -1244,7 +1361,7 @@ __device__ __forceinline__ void add_cell_moment(double (&acc)[6], const Geom& g,
                                                 const DevParticle& P, int x, int y, int z,
                                                 const double (&j)[3], double sign) {
     double r[3];
-    separation(g, x + 0.5, y + 0.5, z + 0.5, P, r[0], r[1], r[2]);
+    centre_offset(g, P, x, y, z, r);
     acc[0] += sign * j[0];
     acc[1] += sign * j[1];
     acc[2] += sign * j[2];
@@ -1261,7 +1378,7 @@ __device__ __forceinline__ void add_cell_moment(double (&acc)[6], const Geom& g,
 // that tested a run of a row rebuilt up to a dozen of them in turn while most
 // warps had none.  A candidate is a long chain of FP64 latency, so the launch
 // takes about as long as the fullest warp (D = 24 settling, ~45 cells per
-// step: 92 us -> 61 us).
+// step: 92 us for runs of a row, 61 us dealt out).
 //
 // acc != nullptr: re-mapping momentum charge of particle p (uncovered cells
 // plus, covered cells minus; moments about the new centre) added to this
@@ -1327,7 +1444,7 @@ __device__ __forceinline__ void refill_cells(const T* __restrict__ srcB, T* __re
                   czl = __shfl_sync(full, z, src_lane);
         double jm[3];
         refill_warp<T, C>(srcB, dst, g, k, cp, so, sn, extrapolate, p, cxl, cyl, czl, status, w,
-                          lane, jm);
+                          lane, acc != nullptr, jm);
         if (acc && lane == src_lane) add_cell_moment(*acc, g, sn[p], cxl, cyl, czl, jm, 1.0);
     }
 }
