@@ -495,6 +495,118 @@ __device__ inline bool psm_collide(C (&f)[NQ], const Coll<C>& k, const Coupl& cp
     return density_bad(rho);
 }
 
+// The FP64 form of psm_collide, written per opposite pair with s = (f_q +
+// f_qbar)/2, d = (f_q - f_qbar)/2 and e+-, v+- the even / odd parts of
+// f_eq(rho, U) and f_eq(rho, v):
+//   fluid  (1 - B) (l+ (s - e+) + F+),  (1 - B) (l- (d - e-) + F-)
+//   M1     v+ - e+,                     e- + v- - 2 d
+//   M2     v+ - s + om (s - e+),        v- - d + om (d - e-),  om = 1 - 1/tau
+//   M3     0,                           2 (v- - d)
+// are the even and odd parts of the change (the solid ones times B_s), and
+// sum_q C_q c_qbar of Eq. (28) is rho0 (U - v) for M1 and M2, twice that for
+// M3.  It is bound by the FP64 pipe: ~300 operations and no arrays over q
+// beside f, 123 registers, against ~700 and 254 of the general form (k_near
+// PSM M1B1 D = 8: 35.1 us -> 25.4 us).  FP32 keeps the general form: its time
+// hides under the bulk sweep, and its results stay the same bits.
+__device__ inline bool psm_collide64(double (&f)[NQ], const Coll<double>& k, const Coupl& cp,
+                                     const Geom& g, const DevParticle* parts, int nobj,
+                                     const int (&pid)[CELL_SLOTS], const double (&eps)[CELL_SLOTS],
+                                     int x, int y, int z, Slots& slots) {
+    using C = double;
+    C rho, jx, jy, jz;
+    moments_j(f, rho, jx, jy, jz);
+    const C ux = jx * k.inv_rho0, uy = jy * k.inv_rho0, uz = jz * k.inv_rho0;
+    C vx[CELL_SLOTS], vy[CELL_SLOTS], vz[CELL_SLOTS], bv[CELL_SLOTS], Bs[CELL_SLOTS];
+    double B = 0.0;
+    const int variant = cp.variant;
+    const double fscale = variant == 2 ? 2.0 : 1.0;
+#pragma unroll
+    for (int o = 0; o < CELL_SLOTS; ++o) {
+        vx[o] = vy[o] = vz[o] = bv[o] = Bs[o] = (C)0;
+        if (o >= nobj) continue;
+        const DevParticle& P = parts[pid[o]];
+        const double e = eps[o];
+        const double b = variant == 0 ? e : e * (cp.tau - 0.5) / ((1.0 - e) + (cp.tau - 0.5));
+        B += b;
+        double r[3], v[3];
+        centre_offset(g, P, x, y, z, r);
+        v[0] = P.u[0] + (P.w[1] * r[2] - P.w[2] * r[1]);
+        v[1] = P.u[1] + (P.w[2] * r[0] - P.w[0] * r[2]);
+        v[2] = P.u[2] + (P.w[0] * r[1] - P.w[1] * r[0]);
+        const double s = b * fscale;
+        const double F[3] = {s * ((double)jx - cp.rho0 * v[0]), s * ((double)jy - cp.rho0 * v[1]),
+                             s * ((double)jz - cp.rho0 * v[2])};
+        double Tq[3];
+        cross3(r, F, Tq);
+        slots.add(pid[o], F, Tq);
+        Bs[o] = (C)b;
+        vx[o] = (C)v[0];
+        vy[o] = (C)v[1];
+        vz[o] = (C)v[2];
+        bv[o] = rho - (C)1.5 * k.rho0 * (vx[o] * vx[o] + vy[o] * vy[o] + vz[o] * vz[o]);
+    }
+    const C oneB = (C)(1.0 - B), om = (C)(1.0 - 1.0 / cp.tau);
+    const C olp = oneB * k.lam_p, olm = oneB * k.lam_m;
+    const C bu = rho - (C)1.5 * k.rho0 * (ux * ux + uy * uy + uz * uz);
+    const C uf = k.has_force ? ux * k.fx + uy * k.fy + uz * k.fz : (C)0;
+    // rest direction
+    {
+        const C w = (C)(1.0 / 3.0), e = w * bu;
+        C dp = olp * (f[0] - e);
+        if (k.has_force) dp -= oneB * uf;
+#pragma unroll
+        for (int o = 0; o < CELL_SLOTS; ++o) {
+            if (o >= nobj) continue;
+            const C v = w * bv[o];
+            if (variant == 0) dp += Bs[o] * (v - e);
+            else if (variant == 1) dp += Bs[o] * ((v - f[0]) + om * (f[0] - e));
+        }
+        f[0] += dp;
+    }
+#pragma unroll
+    for (int q = 1; q < NQ; q += 2) {
+        const C w = (C)wq(q);
+        const C k1 = (C)(4.5 * wq(q)) * k.rho0, k2 = (C)(3.0 * wq(q)) * k.rho0;
+        const auto dot = [&](C ax, C ay, C az) {
+            C d = (C)0;
+            if (cx(q)) d = cx(q) > 0 ? ax : -ax;
+            if (cy(q)) d = cx(q) ? (cy(q) > 0 ? d + ay : d - ay) : ay;
+            if (cz(q)) d = cx(q) || cy(q) ? (cz(q) > 0 ? d + az : d - az) : az;
+            return d;
+        };
+        const C s = (C)0.5 * (f[q] + f[q + 1]), d = (C)0.5 * (f[q] - f[q + 1]);
+        const C cu = dot(ux, uy, uz);
+        const C ep = w * bu + (k1 * cu) * cu, em = k2 * cu;
+        C dp = olp * (s - ep), dm = olm * (d - em);
+        if (k.has_force) {
+            const C cf = dot(k.fx, k.fy, k.fz);
+            dp += oneB * (w * ((C)9 * cu * cf - (C)3 * uf));
+            dm += oneB * ((C)3 * w * cf);
+        }
+#pragma unroll
+        for (int o = 0; o < CELL_SLOTS; ++o) {
+            if (o >= nobj) continue;
+            const C cv = dot(vx[o], vy[o], vz[o]);
+            const C vm = k2 * cv;
+            if (variant == 2) {
+                dm += Bs[o] * ((C)2 * (vm - d));
+                continue;
+            }
+            const C vp = w * bv[o] + (k1 * cv) * cv;
+            if (variant == 0) {
+                dp += Bs[o] * (vp - ep);
+                dm += Bs[o] * ((em + vm) - (C)2 * d);
+            } else {
+                dp += Bs[o] * ((vp - s) + om * (s - ep));
+                dm += Bs[o] * ((vm - d) + om * (d - em));
+            }
+        }
+        f[q] += dp + dm;
+        f[q + 1] += dp - dm;
+    }
+    return density_bad(rho);
+}
+
 // ---------------------------------------------------------------------------
 // bulk sweep: every cell outside the near-particle regions.  Tiles that no
 // region touches skip the per-cell test (block-uniform branch).
@@ -836,24 +948,27 @@ __device__ __forceinline__ void near_block(const T* __restrict__ src, T* __restr
         atomicOr(status, ST_BOUNDS);
         active = false;
     }
-    if (active) {
-        const long long idx = lin(g, x, y, z);
+    if (KIND == 2 && NOSTREAM && active) {
+        // MEM with no stream (first sweep after set-up): fluid cells collide
+        if (!map_at(gm, p, kx, ky, kz)) {
+            const long long idx = lin(g, x, y, z);
+            C f[NQ];
+            load_own(src, g, idx, f);
+            if (collide_cell(f, k)) atomicOr(status, ST_FLUID);
+            store_own(dst, g, idx, f);
+        }
+    }
+    if (KIND != 2) {
         C f[NQ];
-        if (KIND == 2) {
-            // MEM with no stream (first sweep after set-up): fluid cells collide
-            if (NOSTREAM && !map_at(gm, p, kx, ky, kz)) {
-                load_own(src, g, idx, f);
-                if (collide_fluid(f, k)) atomicOr(status, ST_FLUID);
-                store_own(dst, g, idx, f);
-            }
-        } else {
+        int nobj = 0;
+        int pid[CELL_SLOTS];
+        double eps[CELL_SLOTS];
+        const long long idx = active ? lin(g, x, y, z) : 0;
+        if (active) {
             if (NOSTREAM)
                 load_own(src, g, idx, f);
             else
                 pull_plain(src, g, x, y, z, idx, f);
-            int nobj = 0;
-            int pid[CELL_SLOTS];
-            double eps[CELL_SLOTS];
             if (KIND == 1) {
                 const double n3 = (double)cp.subsample * cp.subsample * cp.subsample;
                 for (int s = 0; s < cp.np; ++s) {
@@ -871,12 +986,23 @@ __device__ __forceinline__ void near_block(const T* __restrict__ src, T* __restr
                     }
                 }
             }
+        }
+        if constexpr (std::is_same<C, double>::value) {
+            // a warp with any covered cell takes the PSM form for all of them
+            // (B = 0 is the fluid collision), so that it runs one form, not two
+            const bool coupled = KIND == 1 && __any_sync(0xffffffffu, nobj > 0);
+            if (active) {
+                const bool bad = coupled ? psm_collide64(f, k, cp, g, sp, nobj, pid, eps, x, y, z, slots)
+                                         : collide_cell(f, k);
+                if (bad) atomicOr(status, ST_FLUID);
+            }
+        } else if (active) {
             const bool bad = nobj == 0
                                  ? collide_fluid(f, k)
                                  : psm_collide(f, k, cp, g, sp, nobj, pid, eps, x, y, z, slots);
             if (bad) atomicOr(status, ST_FLUID);
-            store_own(dst, g, idx, f);
         }
+        if (active) store_own(dst, g, idx, f);
     }
     if (KIND == 2 && !NOSTREAM) {
         // MEM (Sec. 2.2): solid cells are not updated; every lane of the warp
@@ -904,11 +1030,16 @@ __device__ __forceinline__ void near_block(const T* __restrict__ src, T* __restr
     if (KIND == 0 || (NOSTREAM && KIND == 2)) return;
     // fixed-order reduction of this block's contribution for each particle
     const int lane = tid & 31, warp = tid >> 5, nwarp = nthr / 32;
+    const bool any = __any_sync(0xffffffffu, slots.id[0] >= 0);
     for (int q = 0; q < cp.np; ++q) {
+        if (any) {
 #pragma unroll
-        for (int c = 0; c < 6; ++c) {
-            double v = warp_sum(slots.get(q, c));
-            if (lane == 0) red[warp][c] = v;
+            for (int c = 0; c < 6; ++c) {
+                double v = warp_sum(slots.get(q, c));
+                if (lane == 0) red[warp][c] = v;
+            }
+        } else if (lane < 6) {
+            red[warp][lane] = 0.0;  // no cell of this warp feels a force
         }
         __syncthreads();
         if (tid < 6) {
