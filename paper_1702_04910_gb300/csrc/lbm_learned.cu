@@ -53,9 +53,17 @@ static_assert(NPARAM == LBM_MLP_PARAMS, "parameter count");
 constexpr int NORM_MU = 0, NORM_IS = FIN, NORM_OS = 2 * FIN, NNORM = 2 * FIN + FOUT;
 
 // ---------------------------------------------------------------------------
-// feature stencil: one block per particle, one thread per grid point
+// feature stencil: 8 threads per grid point, one per corner of its trilinear
+// cell, FEAT_POINTS points per block, blocks (chunk, particle).
+//
+// Bound by latency: 8 corners x (19 loads, ~60 FP64 operations) per point.
+// With a thread per point on one SM they came one after another (53 us for one
+// particle); across 8 lanes and 8 SMs each thread has one corner, and the
+// corners are added by a butterfly (12 us, cold L2).
+constexpr int FEAT_POINTS = 16, FEAT_THREADS = 8 * FEAT_POINTS;
+constexpr int FEAT_CHUNKS = (NPTS + FEAT_POINTS - 1) / FEAT_POINTS;
 template <typename T>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(FEAT_THREADS)
     k_features(const T* __restrict__ state, Geom g, Coupl cp, const DevParticle* __restrict__ parts,
                GeoMap gm, const double* __restrict__ force, double u_ref, float* __restrict__ feat) {
     __shared__ DevParticle sp[MAX_PARTICLES];
@@ -63,44 +71,38 @@ __global__ void __launch_bounds__(128)
     for (int i = threadIdx.x; i < nd; i += blockDim.x)
         reinterpret_cast<double*>(sp)[i] = reinterpret_cast<const double*>(parts)[i];
     __syncthreads();
-    const int p = blockIdx.x;
+    const int p = blockIdx.y;
     const DevParticle& P = sp[p];
     float* out = feat + (long long)p * FIN;
-    const int s = threadIdx.x;
+    const int s = blockIdx.x * FEAT_POINTS + threadIdx.x / 8, corner = threadIdx.x % 8;
+    double eps = 0.0, u[3] = {0.0, 0.0, 0.0};
     if (s < NPTS) {
-        const int i = s % NSTEN, j = (s / NSTEN) % NSTEN, k = s / (NSTEN * NSTEN);
+        const int ijk[3] = {s % NSTEN, (s / NSTEN) % NSTEN, s / (NSTEN * NSTEN)};
         const double h = 0.5 * (P.r + NEAR_HALO);
-        const double pos[3] = {P.x[0] + (i - 2) * h, P.x[1] + (j - 2) * h, P.x[2] + (k - 2) * h};
-        int base[3];
-        double fr[3];
+        int at[3];
+        double w = 1.0;
         for (int a = 0; a < 3; ++a) {
-            const double c = pos[a] - 0.5;  // cell-centre coordinate
-            const double fl = floor(c);
-            base[a] = (int)fl;
-            fr[a] = c - fl;
+            const double c = (P.x[a] + (ijk[a] - 2) * h) - 0.5;  // cell-centre coordinate
+            const double fl = floor(c), fr = c - fl;
+            const int d = (corner >> a) & 1;
+            at[a] = (int)fl + d;
+            w *= d ? fr : 1.0 - fr;
         }
-        const double n3 = (double)cp.subsample * cp.subsample * cp.subsample;
-        double eps = 0.0, u[3] = {0.0, 0.0, 0.0};
-        for (int corner = 0; corner < 8; ++corner) {
-            const int d[3] = {corner & 1, (corner >> 1) & 1, (corner >> 2) & 1};
-            double w = 1.0;
-            for (int a = 0; a < 3; ++a) w *= d[a] ? fr[a] : 1.0 - fr[a];
-            const int X = wrap_i(base[0] + d[0], g.nx), Y = wrap_i(base[1] + d[1], g.ny);
-            int Z = base[2] + d[2];
-            if (g.bc_z) {
-                if (Z < 0 || Z >= g.nz) continue;  // beyond a resting wall: eps 0, u 0
-            } else {
-                Z = wrap_i(Z, g.nz);
-            }
-            const double xc = X + 0.5, yc = Y + 0.5, zc = Z + 0.5;
-            double e = 0.0, v[3] = {0.0, 0.0, 0.0};
-            int own = 0;
+        const int X = wrap_i(at[0], g.nx), Y = wrap_i(at[1], g.ny);
+        int Z = at[2];
+        bool in = true;  // beyond a resting wall: eps 0, u 0
+        if (g.bc_z) in = Z >= 0 && Z < g.nz;
+        else Z = wrap_i(Z, g.nz);
+        if (in) {
             // the step's geometry map (cells outside every region box are
             // fluid / uncovered)
+            double e = 0.0, v[3] = {0.0, 0.0, 0.0};
+            int own = 0;
             if (cp.kind == 2) {
                 own = mapped_owner(g, sp, cp.np, gm, X, Y, Z);
                 e = own ? 1.0 : 0.0;
             } else if (cp.kind == 1) {
+                const double n3 = (double)cp.subsample * cp.subsample * cp.subsample;
                 for (int q = 0; q < cp.np; ++q) {
                     int ox, oy, oz;
                     if (region_offsets(g, sp[q].reg, X, Y, Z, ox, oy, oz)) e += map_at(gm, q, ox, oy, oz) / n3;
@@ -108,32 +110,41 @@ __global__ void __launch_bounds__(128)
                 e = e < 1.0 ? e : 1.0;
             }
             if (own) {
-                body_velocity(g, sp[own - 1], xc, yc, zc, v[0], v[1], v[2]);
+                body_velocity(g, sp[own - 1], X + 0.5, Y + 0.5, Z + 0.5, v[0], v[1], v[2]);
             } else {
                 const long long idx = lin(g, X, Y, Z);
-                for (int q = 0; q < NQ; ++q) {
+#pragma unroll
+                for (int q = 1; q < NQ; ++q) {
                     const double f = ld_pdf(state + (long long)q * g.n + idx, q);
-                    v[0] += f * cx(q);
-                    v[1] += f * cy(q);
-                    v[2] += f * cz(q);
+                    if (cx(q)) v[0] += cx(q) > 0 ? f : -f;
+                    if (cy(q)) v[1] += cy(q) > 0 ? f : -f;
+                    if (cz(q)) v[2] += cz(q) > 0 ? f : -f;
                 }
                 for (int a = 0; a < 3; ++a) v[a] /= cp.rho0;
             }
-            eps += w * e;
-            for (int a = 0; a < 3; ++a) u[a] += w * v[a];
+            eps = w * e;
+            for (int a = 0; a < 3; ++a) u[a] = w * v[a];
         }
-        out[s] = (float)eps;
-        for (int a = 0; a < 3; ++a) out[NPTS * (1 + a) + s] = (float)((u[a] - P.u[a]) / u_ref);
     }
-    if (s == 0) {
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+        eps += __shfl_xor_sync(0xffffffffu, eps, o);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) u[a] += __shfl_xor_sync(0xffffffffu, u[a], o);
+    }
+    if (s < NPTS && corner < 4) {
+        const int a = corner - 1;
+        const double ua = corner < 2 ? u[0] : (corner == 2 ? u[1] : u[2]);
+        out[NPTS * corner + s] = corner == 0 ? (float)eps : (float)((ua - P.u[a < 0 ? 0 : a]) / u_ref);
+    }
+    if (blockIdx.x == 0 && threadIdx.x < 3) {
+        const int a = threadIdx.x;
         const double D = P.d, fs = cp.rho0 * u_ref * u_ref * D * D, ts = fs * D;
         const double* F = force + 6 * p;
-        for (int a = 0; a < 3; ++a) {
-            out[4 * NPTS + a] = (float)(P.u[a] / u_ref);
-            out[4 * NPTS + 3 + a] = (float)(P.w[a] * P.r / u_ref);
-            out[4 * NPTS + 6 + a] = (float)(F[a] / fs);
-            out[4 * NPTS + 9 + a] = (float)(F[3 + a] / ts);
-        }
+        out[4 * NPTS + a] = (float)(P.u[a] / u_ref);
+        out[4 * NPTS + 3 + a] = (float)(P.w[a] * P.r / u_ref);
+        out[4 * NPTS + 6 + a] = (float)(F[a] / fs);
+        out[4 * NPTS + 9 + a] = (float)(F[3 + a] / ts);
     }
 }
 
@@ -505,8 +516,8 @@ template <typename T>
 cudaError_t features_t(const void* state, const Launch& L, const double* force, double u_ref,
                        float* feat) {
     const GeoMap gm{L.map, L.map_ext[0], L.map_ext[1], L.map_ext[2]};
-    k_features<T><<<L.cp.np, 128, 0, L.stream>>>((const T*)state, L.g, L.cp, L.parts, gm, force,
-                                                  u_ref, feat);
+    k_features<T><<<dim3(FEAT_CHUNKS, L.cp.np), FEAT_THREADS, 0, L.stream>>>(
+        (const T*)state, L.g, L.cp, L.parts, gm, force, u_ref, feat);
     return cudaGetLastError();
 }
 
