@@ -764,31 +764,40 @@ struct PullPair<T, NQ> {
                                                long long, int, int, int, f2 (&)[NQ]) {}
 };
 
-// Grid (ceil(nx / (2 PAIR_TX)), ceil(ny / PAIR_TY), nz), block (PAIR_TX, PAIR_TY).
-// One row of 128 cells per 64-thread block: the near-particle sweep runs
+// Grid (ceil(nx / (2 W)), ny, nz), one row segment per block of W = 64, 96 or 32
+// threads, whichever leaves the fewest beyond the row's end (pair_width: 192
+// cells per row are 96 threads; as two blocks of 64, a quarter of them idle,
+// the BF16 sweep of 192 x 192 x 768 cells took 473 us, 0.67 of HBM, and takes
+// 376 us, 0.85).  One row of 128 cells per 64-thread block: the near-particle sweep runs
 // beside this kernel and each of its blocks holds 7.7k (MEM) to 11.5k (PSM)
 // registers; with small bulk blocks an SM that hosts near blocks gives up
 // only as many bulk warps as their registers need (measured in the 128 x 128
 // x 512 step, FP16: 0.70 of HBM with 64 x 4, 0.745 with 64 x 2, 0.76 with
 // 64 x 1; 32 x 1 and 128 x 1 are slower).
-constexpr int PAIR_TX = 64, PAIR_TY = 1;
+inline int pair_width(int nx) {
+    const int pairs = nx / 2;
+    int best = 64;
+    const auto waste = [&](int w) { return (pairs + w - 1) / w * w; };
+    if (waste(96) < waste(best)) best = 96;
+    if (waste(32) < waste(best)) best = 32;
+    return best;
+}
 
-template <typename T>
-__global__ void __launch_bounds__(PAIR_TX * PAIR_TY, 768 / (PAIR_TX * PAIR_TY))
+template <typename T, int W>
+__global__ void __launch_bounds__(W, 768 / W)
     k_bulk_pair(const T* __restrict__ src, T* __restrict__ dst, Geom g, Coll<float> k,
                 const DevParticle* __restrict__ parts, int np, int* __restrict__ status) {
-    const int bx0 = 2 * blockIdx.x * PAIR_TX, by0 = blockIdx.y * PAIR_TY;
+    const int bx0 = 2 * blockIdx.x * W, y = blockIdx.y, z = blockIdx.z;
     const int x0 = bx0 + 2 * threadIdx.x;
-    const int y = by0 + threadIdx.y, z = blockIdx.z;
-    if (x0 >= g.nx || y >= g.ny) return;
+    if (x0 >= g.nx) return;
     // k_near's cells are left alone; a block whose cells no region reaches
     // (block-uniform test) skips the per-cell one
     bool near_a = false, near_b = false;
     for (int s = 0; s < np; ++s) {
         const int* r = parts[s].reg;
         if (!in_range(z, r[8], r[9], g.nz) ||
-            !spans_meet(by0, min(PAIR_TY, g.ny - by0), r[4], r[5], g.ny) ||
-            !spans_meet(bx0, min(2 * PAIR_TX, g.nx - bx0), r[0], r[1], g.nx))
+            !in_range(y, r[4], r[5], g.ny) ||
+            !spans_meet(bx0, min(2 * W, g.nx - bx0), r[0], r[1], g.nx))
             continue;
         near_a = near_a || cell_in_reg(g, r, x0, y, z);
         near_b = near_b || cell_in_reg(g, r, x0 + 1, y, z);
@@ -814,6 +823,90 @@ __global__ void __launch_bounds__(PAIR_TX * PAIR_TY, 768 / (PAIR_TX * PAIR_TY))
         for (int q = 0; q < NQ; ++q)
             dst[(long long)q * g.n + idx] = Pair16<T>::one(near_a ? f[q].v.y : f[q].v.x);
     }
+}
+
+// 16-bit shifted storage where rows cannot be taken as aligned words (odd nx)
+// or the boundary planes have their own rules (open boundaries): each thread
+// takes the cells z and z + 1 of one column, with 2-byte accesses, and collides
+// them in the two lanes of the packed arithmetic on the shifted values, as
+// k_bulk_pair does.  One cell per thread in scalar FP32 was bound by issue
+// (565 instructions per cell, 0.34 of HBM); this form halves the arithmetic
+// and the addresses: 101 x 101 x 304 cells FP16 85 us -> 73 us (k_near beside
+// it), 440 instructions per 64 cells, issue 57 %.
+template <typename T>
+__device__ __forceinline__ float raw16(const T* p);
+template <>
+__device__ __forceinline__ float raw16<__half>(const __half* p) {
+    return __half2float(__ldg(p));
+}
+template <>
+__device__ __forceinline__ float raw16<__nv_bfloat16>(const __nv_bfloat16* p) {
+    return __bfloat162float(__ldg(p));
+}
+template <typename T, int Q>
+struct PullRaw {
+    __device__ __forceinline__ static void run(const T* __restrict__ src, const Geom& g,
+                                               const NbrOff& o, long long idx, float (&f)[NQ]) {
+        if ((cz(Q) > 0 && o.zlo) || (cz(Q) < 0 && o.zhi))
+            f[Q] = raw16(src + (long long)opp(Q) * g.n + idx);
+        else
+            f[Q] = raw16(src + (long long)Q * g.n + idx + upstream_off<Q>(o));
+        PullRaw<T, Q + 1>::run(src, g, o, idx, f);
+    }
+};
+template <typename T>
+struct PullRaw<T, NQ> {
+    __device__ __forceinline__ static void run(const T* __restrict__, const Geom&, const NbrOff&,
+                                               long long, float (&)[NQ]) {}
+};
+// Shifted values pulled to cell (x, y, z).  The open boundaries work on f:
+// the cells of those planes take the plain pull and are shifted after it.
+template <typename T>
+__device__ __forceinline__ void pull_raw(const T* __restrict__ src, const Geom& g, int x, int y,
+                                         int z, long long idx, float (&f)[NQ]) {
+    const NbrOff o = make_off(g, x, y, z);
+    if (g.bc_z == 2 && (o.zlo || o.zhi)) {
+        pull_plain(src, g, x, y, z, idx, f);
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) f[q] -= (float)wq(q);
+    } else {
+        PullRaw<T, 0>::run(src, g, o, idx, f);
+    }
+}
+
+// Blocks are runs of 128 cells of a plane, x fastest (row tiles of 64 left a
+// fifth of the lanes of a 101-cell row idle).
+constexpr int ZPAIR_THREADS = 128, ZPAIR_BLOCKS = 5;
+template <typename T>
+__global__ void __launch_bounds__(ZPAIR_THREADS, ZPAIR_BLOCKS)
+    k_bulk_zpair(const T* __restrict__ src, T* __restrict__ dst, Geom g, Coll<float> k,
+                 const DevParticle* __restrict__ parts, int np, int* __restrict__ status) {
+    const unsigned l = blockIdx.x * ZPAIR_THREADS + threadIdx.x;
+    if (l >= (unsigned)g.nx * (unsigned)g.ny) return;
+    const int y = l / (unsigned)g.nx, x = l - (unsigned)y * g.nx, z = 2 * blockIdx.z;
+    bool act0 = true, act1 = z + 1 < g.nz;
+    for (int s = 0; s < np; ++s) {  // k_near's cells
+        const int* r = parts[s].reg;
+        if (!in_range(x, r[0], r[1], g.nx) || !in_range(y, r[4], r[5], g.ny)) continue;
+        act0 = act0 && !in_range(z, r[8], r[9], g.nz);
+        act1 = act1 && !in_range(z + 1, r[8], r[9], g.nz);
+    }
+    if (!act0 && !act1) return;
+    const long long idx = lin(g, x, y, z), plane = (long long)g.nx * g.ny;
+    float a[NQ], b[NQ];
+    if (act0) pull_raw(src, g, x, y, z, idx, a);
+    if (act1) pull_raw(src, g, x, y, z + 1, idx + plane, b);
+    f2 f[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) f[q] = f2(make_float2(act0 ? a[q] : 0.0f, act1 ? b[q] : 0.0f));
+    const unsigned bad = collide_fluid<f2, true>(f, k);
+    if (((bad & 1u) && act0) || ((bad & 2u) && act1)) atomicOr(status, ST_FLUID);
+    if (act0)
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) dst[(long long)q * g.n + idx] = Pair16<T>::one(f[q].v.x);
+    if (act1)
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) dst[(long long)q * g.n + idx + plane] = Pair16<T>::one(f[q].v.y);
 }
 
 // ---------------------------------------------------------------------------
@@ -2046,14 +2139,27 @@ cudaError_t bulk_cpt(const void* src, void* dst, const Launch& L) {
 template <typename T, typename C = T>
 cudaError_t bulk_t(const void* src, void* dst, const Launch& L) {
     if constexpr (sizeof(T) == 2) {
-        // 16-bit sweep with two x-neighbours per thread: even nx, streaming,
-        // no open boundaries (those planes take the per-cell kernel)
+        // 16-bit sweep, two cells per thread: x-neighbours as words for even nx
+        // without open boundaries, z-neighbours otherwise; the first sweep
+        // after set-up (no stream) takes the per-cell kernel
+        const int np = L.all_tiles ? 0 : L.cp.np;
         if (!L.nostream && L.g.nx % 2 == 0 && L.g.bc_z != 2) {
-            dim3 grid((L.g.nx + 2 * PAIR_TX - 1) / (2 * PAIR_TX), (L.g.ny + PAIR_TY - 1) / PAIR_TY,
-                      L.g.nz);
-            return launch(k_bulk_pair<T>, grid, dim3(PAIR_TX, PAIR_TY, 1), L.stream, (const T*)src,
-                          (T*)dst, L.g, L.kf, L.parts, L.all_tiles ? 0 : L.cp.np, L.status);
+            const int w = pair_width(L.g.nx);
+            const dim3 grid((L.g.nx / 2 + w - 1) / w, L.g.ny, L.g.nz);
+            const auto go = [&](auto kernel) {
+                return launch(kernel, grid, w, L.stream, (const T*)src, (T*)dst, L.g, L.kf, L.parts,
+                              np, L.status);
+            };
+            return w == 96 ? go(k_bulk_pair<T, 96>)
+                           : (w == 32 ? go(k_bulk_pair<T, 32>) : go(k_bulk_pair<T, 64>));
         }
+        const long long plane = (long long)L.g.nx * L.g.ny;
+        if (!L.nostream && plane < (1LL << 31))
+            return launch(k_bulk_zpair<T>,
+                          dim3((unsigned)((plane + ZPAIR_THREADS - 1) / ZPAIR_THREADS), 1,
+                               (L.g.nz + 1) / 2),
+                          ZPAIR_THREADS, L.stream, (const T*)src, (T*)dst, L.g, L.kf, L.parts, np,
+                          L.status);
     }
     if constexpr (sizeof(T) <= 4) {
         if (L.g.tz == 2) return bulk_cpt<T, C, 2>(src, dst, L);
