@@ -158,7 +158,8 @@ Launch base_launch(lbm_handle* h) {
     L.all_tiles = 0;
     L.block = dim3(h->g.tx, h->g.ty, 1);
     L.stream = h->stream;
-    near_grid(h->g, h->maxd, L.box);
+    L.near_nblk = near_blocks(h->g, h->maxd);
+    L.refill_side = (int)std::ceil(h->maxd) + 4;
     L.map = h->d_map;
     region_extent(h->g, h->maxd, L.map_ext);
     return L;
@@ -203,9 +204,8 @@ lbm_status alloc_particles(lbm_handle* h, int n) {
 // Force partials for `subcycles` sweeps of the near kernel at the current
 // particle count and largest diameter.
 lbm_status ensure_partials(lbm_handle* h) {
-    int box[3];
-    near_grid(h->g, h->maxd, box);
-    const size_t need = (size_t)h->subcycles * (size_t)near_partial_doubles(box, h->np);
+    const size_t need =
+        (size_t)h->subcycles * (size_t)near_partial_doubles(near_blocks(h->g, h->maxd), h->np);
     const size_t mneed0 = (size_t)map_entries(h->g, h->maxd, h->np);
     if (h->remap_charge) {
         // refill-block partials of the re-mapping charge (box side as in step_once)
@@ -268,7 +268,7 @@ lbm_status after_pre_state(lbm_handle* h) {
 lbm_status sweep(lbm_handle* h, int sub, bool with_map) {
     Launch L = base_launch(h);
     L.nostream = h->pending_pre;
-    L.partials = h->d_partials + (size_t)sub * (size_t)near_partial_doubles(L.box, h->np);
+    L.partials = h->d_partials + (size_t)sub * (size_t)near_partial_doubles(L.near_nblk, h->np);
     const void* src = h->buf[h->cur];
     void* dst = h->buf[1 - h->cur];
     // The near-particle cells and the bulk cells are disjoint: the (small,
@@ -343,7 +343,6 @@ lbm_status step_once(lbm_handle* h) {
     }
     if (h->kind == 2) {
         // re-map with the new state; rebuild uncovered cells (src of the last sweep)
-        L.box[0] = (int)std::ceil(h->maxd) + 4;  // refill: cube side in cells
         pi = prof_begin(h, PC_REFILL);
         CK(h, launch_refill(h->storage, h->buf[1 - h->cur], h->buf[h->cur], L, h->d_prev,
                             h->d_parts, 1, h->remap_charge ? h->d_charge_part : nullptr),
@@ -592,7 +591,6 @@ lbm_status lbm_set_particles(lbm_handle* h, int n, const lbm_particle* host_in) 
     CK(h, launch_regions(L), "region launch");
     if (remap) {
         L = base_launch(h);
-        L.box[0] = (int)std::ceil(h->maxd) + 4;
         CK(h, launch_refill(h->storage, h->buf[1 - h->cur], h->buf[h->cur], L, h->d_tmp, h->d_parts, 0),
            "refill launch");
     }

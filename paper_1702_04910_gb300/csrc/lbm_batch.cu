@@ -346,8 +346,7 @@ lbm_status make_case(lbm_batch* b, int c, const lbm_config& cfg, const lbm_parti
     k.cp.mr_cpc = cfg.coupling == LBM_MEM_MR ? mr_correction_scale(cfg) : 0.0;
     k.kd = make_coll<double>(lp, lm, cfg.rho0, cfg.force_density);
     region_extent(g, p.diameter, k.map_ext);
-    near_grid(g, p.diameter, k.box);
-    k.nblk = near_blocks(k.box);
+    k.nblk = near_blocks(g, p.diameter);
     k.refill_side = (int)std::ceil(p.diameter) + 4;
     for (int a = 0; a < 3; ++a) k.gravity[a] = cfg.gravity[a];
     k.cur = 0;

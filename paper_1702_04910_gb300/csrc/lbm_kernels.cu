@@ -403,9 +403,12 @@ __device__ __forceinline__ void mem_links_warp(const T* __restrict__ src, const 
         w.jt[lane][2] = mc.j[2];
     }
     __syncwarp();
+    // with no more particles than slots a lane keeps the forces of the links it
+    // evaluates; the warp's sum is the same, and no cell can run out of slots
+    const bool direct = cp.np <= CELL_SLOTS;
     for (int base = 0; base < total; base += 32) {
         const int e = base + lane;
-        w.own[lane] = 0;
+        if (!direct) w.own[lane] = 0;
         if (e < total) {
             const int ol = w.list[e] >> 5, q = w.list[e] & 31;
             const int lx = w.x[ol], ly = w.y[ol], lz = w.z[ol];
@@ -417,9 +420,22 @@ __device__ __forceinline__ void mem_links_warp(const T* __restrict__ src, const 
                 mc.j[1] = w.jt[ol][1];
                 mc.j[2] = w.jt[ol][2];
             }
-            w.lv[e] = mem_link(src, g, cp, parts, cp.np, gm, b, lx, ly, lz, w.idx[ol], q,
-                               &w.ft[lane][0], &w.own[lane], status, mc);
+            double ft[6];
+            int own;
+            w.lv[e] = mem_link(src, g, cp, parts, cp.np, gm, b, lx, ly, lz, w.idx[ol], q, ft, &own,
+                               status, mc);
+            if (direct) {
+                if (own) {
+                    const double F[3] = {ft[0], ft[1], ft[2]}, Tq[3] = {ft[3], ft[4], ft[5]};
+                    slots.add(own - 1, F, Tq);
+                }
+            } else {
+#pragma unroll
+                for (int c = 0; c < 6; ++c) w.ft[lane][c] = ft[c];
+                w.own[lane] = own;
+            }
         }
+        if (direct) continue;
         __syncwarp();
         // this round's links of this lane's cell: entries [lo, hi)
         const int lo = first > base ? first : base;
@@ -434,8 +450,34 @@ __device__ __forceinline__ void mem_links_warp(const T* __restrict__ src, const 
         }
         __syncwarp();
     }
+    __syncwarp();
     WarpMerge<C, 1>::run(cut, w.lv, first, f);
     __syncwarp();
+}
+
+// Sums of six values over the warp: halves of the lanes take halves of the
+// components first, so that 9 FP64 adds per lane do instead of 30.  Lane 4 c
+// (c < 6) returns the sum of component c.
+__device__ __forceinline__ double warp_sum6(const double (&v)[6], int lane) {
+    const unsigned full = 0xffffffffu;
+    double a[4], b[2], s;
+    const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const double hi = i < 2 ? v[4 + i] : 0.0;  // components 6 and 7 do not exist
+        const double o = __shfl_xor_sync(full, h4 ? v[i] : hi, 16);
+        a[i] = (h4 ? hi : v[i]) + o;
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const double o = __shfl_xor_sync(full, h3 ? a[i] : a[2 + i], 8);
+        b[i] = (h3 ? a[2 + i] : a[i]) + o;
+    }
+    const double o = __shfl_xor_sync(full, h2 ? b[0] : b[1], 4);
+    s = (h2 ? b[1] : b[0]) + o;
+    s += __shfl_xor_sync(full, s, 2);
+    s += __shfl_xor_sync(full, s, 1);
+    return s;
 }
 
 // ---------------------------------------------------------------------------
@@ -910,17 +952,6 @@ __global__ void __launch_bounds__(ZPAIR_THREADS, ZPAIR_BLOCKS)
 }
 
 // ---------------------------------------------------------------------------
-// near-particle sweep over the cell region of each particle (cells within
-// R + NEAR_HALO of the centre per axis).  Grid (bx, by, bz * np) of
-// NEAR_BX x NEAR_BY x NEAR_BZ blocks: block (bx, by, bz) of particle p covers
-// region offsets [bx*NEAR_BX, ...) etc.; a cell that also lies in the region
-// of a lower-index particle is left to that particle's blocks.  Each block
-// writes, for every particle q, its fixed-order force/torque sum to
-// partials[((p * nblk + blk) * np + q) * 6 + c].
-// One near-kernel block: region offsets (bx, by, bzz) of particle p, whose
-// force/torque sums land in partials[((p * nblk + blk) * np + q) * 6 + c].
-// `sp` holds the particle records in shared memory; every thread of the
-// block must call this (it synchronises for the reduction).
 // MEM: a cell whose centre lies farther than R + 3/2 from every sphere centre
 // has no solid neighbour (neighbour centres are at most sqrt(2) away and a
 // cell is solid iff its centre is within R, R6), so its pull is the plain one.
@@ -1015,19 +1046,42 @@ __device__ __forceinline__ void near_pull(const T* __restrict__ src, const Geom&
     cut = solid;
 }
 
-template <typename T, typename C, int KIND, bool NOSTREAM>
+// Cell of a lane of near block blk, as offsets in the region R; false beyond it.
+// PSM: 32 consecutive cells of the region.  MEM: four runs of 8 cells, a
+// quarter of the region apart: the cut links lie in a thin shell and are taken
+// 32 at a time, so a warp should not hold many more than the others.  Region cells
+// number less than 2^32: the two buffers of a larger lattice fit no memory.
+template <int KIND>
+__device__ __forceinline__ bool near_cell(const int* R, long long blk, int lane, int& kx, int& ky,
+                                          int& kz) {
+    const unsigned ex = R[1], ey = R[5], total = ex * ey * (unsigned)R[9];
+    const unsigned runs = (total + 7) / 8, used = KIND == 2 ? (runs + 3) / 4 : (total + 31) / 32;
+    const unsigned b = (unsigned)blk;
+    const unsigned l = KIND == 2 ? (b + (lane >> 3) * used) * 8 + (lane & 7) : b * 32 + lane;
+    const bool in = b < used && l < total;
+    const unsigned row = in ? l / ex : 0u, plane = in ? row / ey : 0u;
+    kx = in ? (int)(l - row * ex) : 0;
+    ky = (int)(row - plane * ey);
+    kz = (int)plane;
+    return in;
+}
+
+// One near-kernel block: block blk of particle p, whose force/torque sums on
+// every particle q land in partials[((p * nblk + blk) * np + q) * 6 + c] (the
+// warp's sum, fixed order).  `sp` holds the particle records in shared memory;
+// all 32 lanes call it.
+template <typename T, typename C, int KIND, bool NOSTREAM, typename LW>
 __device__ __forceinline__ void near_block(const T* __restrict__ src, T* __restrict__ dst,
                                            const Geom& g, const Coll<C>& k, const Coupl& cp,
                                            const DevParticle* sp, const GeoMap& gm,
                                            double* __restrict__ partials, int* __restrict__ status,
-                                           int p, int bx, int by, int bzz, long long nblk,
-                                           long long blk, double (*red)[6], LinkWarp* lw) {
-    const int tid = threadIdx.x + NEAR_BX * (threadIdx.y + NEAR_BY * threadIdx.z);
-    constexpr int nthr = NEAR_BX * NEAR_BY * NEAR_BZ;
+                                           int p, long long nblk, long long blk, LW& lw) {
+    const int lane = threadIdx.x;
     const int* R = sp[p].reg;
-    const int kx = bx * NEAR_BX + threadIdx.x, ky = by * NEAR_BY + threadIdx.y,
-              kz = bzz * NEAR_BZ + threadIdx.z;
-    bool active = kx < R[1] && ky < R[5] && kz < R[9];
+    int kx, ky, kz;
+    bool active = near_cell<KIND>(R, blk, lane, kx, ky, kz);
+    if (blk == 0 && lane == 0 && (long long)R[1] * R[5] * R[9] > nblk * NEAR_THREADS)
+        atomicOr(status, ST_BOUNDS);  // a region larger than its grid
     int x = R[0] + kx, y = R[4] + ky, z = R[8] + kz;
     if (x >= g.nx) x -= g.nx;
     if (y >= g.ny) y -= g.ny;
@@ -1097,7 +1151,7 @@ __device__ __forceinline__ void near_block(const T* __restrict__ src, T* __restr
         }
         if (active) store_own(dst, g, idx, f);
     }
-    if (KIND == 2 && !NOSTREAM) {
+    if constexpr (KIND == 2 && !NOSTREAM) {
         // MEM (Sec. 2.2): solid cells are not updated; every lane of the warp
         // takes part in the link loop, cells or not
         C f[NQ];
@@ -1113,8 +1167,7 @@ __device__ __forceinline__ void near_block(const T* __restrict__ src, T* __restr
                 near_pull(src, g, sp, cp.np, gm, p, kx, ky, kz, x, y, z, idx, f, cut, status);
             }
         }
-        mem_links_warp(src, g, cp, sp, &gm, x, y, z, idx, cut, f, slots, status, lw[tid >> 5],
-                       tid & 31);
+        mem_links_warp(src, g, cp, sp, &gm, x, y, z, idx, cut, f, slots, status, lw, lane);
         if (fluid) {
             if (collide_cell(f, k)) atomicOr(status, ST_FLUID);
             store_own(dst, g, idx, f);
@@ -1122,53 +1175,43 @@ __device__ __forceinline__ void near_block(const T* __restrict__ src, T* __restr
     }
     if (KIND == 0 || (NOSTREAM && KIND == 2)) return;
     // fixed-order reduction of this block's contribution for each particle
-    const int lane = tid & 31, warp = tid >> 5, nwarp = nthr / 32;
     const bool any = __any_sync(0xffffffffu, slots.id[0] >= 0);
+    if (p >= cp.np || blk >= nblk) {
+        if (lane == 0) atomicOr(status, ST_BOUNDS);
+        return;
+    }
     for (int q = 0; q < cp.np; ++q) {
-        if (any) {
+        double s = 0.0;
+        if (any) {  // (else no cell of this warp feels a force)
+            double v[6];
 #pragma unroll
-            for (int c = 0; c < 6; ++c) {
-                double v = warp_sum(slots.get(q, c));
-                if (lane == 0) red[warp][c] = v;
-            }
-        } else if (lane < 6) {
-            red[warp][lane] = 0.0;  // no cell of this warp feels a force
+            for (int c = 0; c < 6; ++c) v[c] = slots.get(q, c);
+            s = warp_sum6(v, lane);
         }
-        __syncthreads();
-        if (tid < 6) {
-            double acc = 0.0;
-            for (int w = 0; w < nwarp; ++w) acc += red[w][tid];
-            if (p < cp.np && blk < nblk) partials[(((long long)p * nblk + blk) * cp.np + q) * 6 + tid] = acc;
-            else atomicOr(status, ST_BOUNDS);
-        }
-        __syncthreads();
+        if ((lane & 3) == 0 && lane < 24)
+            partials[(((long long)p * nblk + blk) * cp.np + q) * 6 + (lane >> 2)] = s;
     }
 }
 
 // ---------------------------------------------------------------------------
 // near-particle sweep over the cell region of each particle (cells within
-// R + NEAR_HALO of the centre per axis).  Grid (bx, by, bz * np) of
-// NEAR_BX x NEAR_BY x NEAR_BZ blocks: block (bx, by, bz) of particle p covers
-// region offsets [bx*NEAR_BX, ...) etc.; a cell that also lies in the region
-// of a lower-index particle is left to that particle's blocks.
+// R + NEAR_HALO of the centre per axis).  Grid (near_nblk, np), a warp per
+// block; a cell that also lies in the region of a lower-index particle is left
+// to that particle's blocks.  The particle records are staged in shared memory
+// (dynamic: np records).
 template <typename T, typename C, int KIND, bool NOSTREAM>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(NEAR_THREADS)
     k_near(const T* __restrict__ src, T* __restrict__ dst, Geom g, Coll<C> k, Coupl cp,
            const DevParticle* __restrict__ parts, GeoMap gm, double* __restrict__ partials,
-           int* __restrict__ status, int bz) {
-    __shared__ DevParticle sp[MAX_PARTICLES];
-    __shared__ double red[8][6];
-    __shared__ LinkWarp lw[KIND == 2 ? NEAR_BX * NEAR_BY * NEAR_BZ / 32 : 1];
-    const int tid = threadIdx.x + NEAR_BX * (threadIdx.y + NEAR_BY * threadIdx.z);
-    constexpr int nthr = NEAR_BX * NEAR_BY * NEAR_BZ;
-    for (int i = tid; i < cp.np * (int)(sizeof(DevParticle) / sizeof(double)); i += nthr)
-        reinterpret_cast<double*>(sp)[i] = reinterpret_cast<const double*>(parts)[i];
-    __syncthreads();
-    const int p = blockIdx.z / bz, bzz = blockIdx.z % bz;
-    const long long nblk = (long long)gridDim.x * gridDim.y * bz;
-    const long long blk = blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * bzz);
-    near_block<T, C, KIND, NOSTREAM>(src, dst, g, k, cp, sp, gm, partials, status, p, blockIdx.x,
-                                     blockIdx.y, bzz, nblk, blk, red, lw);
+           int* __restrict__ status) {
+    extern __shared__ double sp_words[];
+    __shared__ typename std::conditional<KIND == 2, LinkWarp, char>::type lw;
+    for (int i = threadIdx.x; i < cp.np * (int)(sizeof(DevParticle) / sizeof(double)); i += NEAR_THREADS)
+        sp_words[i] = reinterpret_cast<const double*>(parts)[i];
+    __syncwarp();
+    near_block<T, C, KIND, NOSTREAM>(src, dst, g, k, cp,
+                                     reinterpret_cast<const DevParticle*>(sp_words), gm, partials,
+                                     status, blockIdx.y, gridDim.x, blockIdx.x, lw);
 }
 
 // ---------------------------------------------------------------------------
@@ -1929,32 +1972,25 @@ __global__ void __launch_bounds__(32) k_batch_map(BatchCase* __restrict__ cases,
 }
 
 // near-particle sweep: one near block of one case per thread block
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(NEAR_THREADS)
     k_batch_near(BatchCase* __restrict__ cases, BatchList l, int sub, int* __restrict__ status) {
     __shared__ DevParticle sp[1];
-    __shared__ double red[8][6];
-    __shared__ LinkWarp lw[NEAR_BX * NEAR_BY * NEAR_BZ / 32];
+    __shared__ LinkWarp lw;
     const int i = find_item(l.base, l.n, blockIdx.x);
     const BatchCase& B = cases[l.list[i]];
     const long long local = blockIdx.x - l.base[i];
-    const int tid = threadIdx.x + NEAR_BX * (threadIdx.y + NEAR_BY * threadIdx.z);
-    for (int k = tid; k < (int)(sizeof(DevParticle) / sizeof(double)); k += NEAR_BX * NEAR_BY * NEAR_BZ)
+    for (int k = threadIdx.x; k < (int)(sizeof(DevParticle) / sizeof(double)); k += NEAR_THREADS)
         reinterpret_cast<double*>(sp)[k] = reinterpret_cast<const double*>(B.part)[k];
-    __syncthreads();
-    const int bx = (int)(local % B.box[0]);
-    const int by = (int)((local / B.box[0]) % B.box[1]);
-    const int bzz = (int)(local / ((long long)B.box[0] * B.box[1]));
+    __syncwarp();
     const GeoMap gm{B.map, B.map_ext[0], B.map_ext[1], B.map_ext[2]};
     const int cur = B.cur;
     double* partials = B.partials + (long long)sub * B.nblk * 6;
     if (B.kind == 2)
         near_block<double, double, 2, false>(B.buf[cur], B.buf[1 - cur], B.g, B.kd, B.cp, sp, gm,
-                                             partials, status, 0, bx, by, bzz, B.nblk, local, red,
-                                             lw);
+                                             partials, status, 0, B.nblk, local, lw);
     else
         near_block<double, double, 1, false>(B.buf[cur], B.buf[1 - cur], B.g, B.kd, B.cp, sp, gm,
-                                             partials, status, 0, bx, by, bzz, B.nblk, local, red,
-                                             lw);
+                                             partials, status, 0, B.nblk, local, lw);
 }
 
 // Threads of a k_batch_bulk block and its resident blocks per SM; a work item
@@ -2095,8 +2131,10 @@ namespace {
 // 2980 / 3110.
 constexpr int SMEM_CARVEOUT = 50;  // percent of the largest shared-memory size
 template <typename... P, typename... A>
-cudaError_t launch(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t s, A&&... args) {
+cudaError_t launch_smem(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                        A&&... args) {
     cudaLaunchConfig_t c{};
+    c.dynamicSmemBytes = smem;
     c.gridDim = grid;
     c.blockDim = block;
     c.stream = s;
@@ -2106,6 +2144,10 @@ cudaError_t launch(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t s, 
     c.attrs = at;
     c.numAttrs = 1;
     return cudaLaunchKernelEx(&c, kernel, std::forward<A>(args)...);
+}
+template <typename... P, typename... A>
+cudaError_t launch(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t s, A&&... args) {
+    return launch_smem(kernel, grid, block, 0, s, std::forward<A>(args)...);
 }
 
 template <typename T, typename C>
@@ -2170,15 +2212,15 @@ cudaError_t bulk_t(const void* src, void* dst, const Launch& L) {
 template <typename T, int KIND>
 cudaError_t near_kind(const void* src, void* dst, const Launch& L) {
     using C = typename ComputeOf<T>::type;
-    dim3 grid(L.box[0], L.box[1], L.box[2] * L.cp.np);
-    dim3 block(NEAR_BX, NEAR_BY, NEAR_BZ);
+    const dim3 grid((unsigned)L.near_nblk, L.cp.np), block(NEAR_THREADS);
+    const size_t smem = sizeof(DevParticle) * L.cp.np;
     const auto& k = coll_of<C, C>(L);
     const GeoMap gm{L.map, L.map_ext[0], L.map_ext[1], L.map_ext[2]};
     if (L.nostream)
-        return launch(k_near<T, C, KIND, true>, grid, block, L.stream, (const T*)src, (T*)dst, L.g, k,
-                      L.cp, L.parts, gm, L.partials, L.status, L.box[2]);
-    return launch(k_near<T, C, KIND, false>, grid, block, L.stream, (const T*)src, (T*)dst, L.g, k,
-                  L.cp, L.parts, gm, L.partials, L.status, L.box[2]);
+        return launch_smem(k_near<T, C, KIND, true>, grid, block, smem, L.stream, (const T*)src,
+                           (T*)dst, L.g, k, L.cp, L.parts, gm, L.partials, L.status);
+    return launch_smem(k_near<T, C, KIND, false>, grid, block, smem, L.stream, (const T*)src, (T*)dst,
+                       L.g, k, L.cp, L.parts, gm, L.partials, L.status);
 }
 
 template <typename T>
@@ -2194,7 +2236,7 @@ cudaError_t refill_t(const void* srcB, void* dst, const Launch& L, const DevPart
                      const DevParticle* pn, int extrapolate, double* charge_part) {
     using C = typename ComputeOf<T>::type;
     if (L.cp.np <= 0) return cudaSuccess;
-    int side = L.box[0];  // set by the caller: cube side in cells
+    const int side = L.refill_side;
     dim3 grid((unsigned)refill_blocks(side), L.cp.np, 1);
     return launch(k_refill<T, C>, grid, REFILL_THREADS, L.stream, (const T*)srcB, (T*)dst, L.g,
                   coll_of<C, C>(L), L.cp, po, pn, extrapolate, side, L.status, charge_part);
@@ -2271,7 +2313,7 @@ cudaError_t launch_refill(int storage, const void* srcB, void* dst, const Launch
 }
 cudaError_t launch_charge_total(const Launch& L, const double* charge_part, double* charge) {
     if (L.cp.np <= 0) return cudaSuccess;
-    return launch(k_charge_total, L.cp.np, 192, L.stream, refill_blocks(L.box[0]), charge_part,
+    return launch(k_charge_total, L.cp.np, 192, L.stream, refill_blocks(L.refill_side), charge_part,
                   charge);
 }
 cudaError_t launch_macro(int storage, const void* state, const Launch& L, int what, void* out) {
@@ -2323,7 +2365,7 @@ cudaError_t launch_map(const Launch& L) {
 
 cudaError_t launch_finalize(const Launch& L, int nsub, double* force_out, const double* charge) {
     if (L.cp.np <= 0) return cudaSuccess;
-    return launch(k_finalize, L.cp.np, FIN_THREADS, L.stream, L.cp.np, near_blocks(L.box), L.partials, nsub,
+    return launch(k_finalize, L.cp.np, FIN_THREADS, L.stream, L.cp.np, L.near_nblk, L.partials, nsub,
                   force_out, charge);
 }
 cudaError_t launch_rigid_body(const Launch& L, const double* force, double gx, double gy,
@@ -2336,7 +2378,7 @@ cudaError_t launch_finalize_rigid(const Launch& L, int nsub, double* force, cons
                                   double gx, double gy, double gz, int wall_contact) {
     if (L.cp.np <= 0) return cudaSuccess;
     return launch(k_finalize_rigid, L.cp.np, FIN_THREADS, L.stream, L.g, L.cp.np,
-                  near_blocks(L.box), L.partials, nsub, force, charge, L.parts, L.parts_prev,
+                  L.near_nblk, L.partials, nsub, force, charge, L.parts, L.parts_prev,
                   L.kd.rho0, gx, gy, gz, (double)nsub, wall_contact, L.status);
 }
 cudaError_t launch_regions(const Launch& L) {
@@ -2362,7 +2404,7 @@ cudaError_t launch_batch_map(BatchCase* cases, BatchList l, long long total, cud
 cudaError_t launch_batch_near(BatchCase* cases, BatchList l, long long total, int sub,
                               int* status, cudaStream_t s) {
     if (l.n == 0 || total == 0) return cudaSuccess;
-    k_batch_near<<<(unsigned)total, dim3(NEAR_BX, NEAR_BY, NEAR_BZ), 0, s>>>(cases, l, sub, status);
+    k_batch_near<<<(unsigned)total, NEAR_THREADS, 0, s>>>(cases, l, sub, status);
     return cudaGetLastError();
 }
 cudaError_t launch_batch_bulk(BatchCase* cases, BatchList l, long long total, int grid,

@@ -25,19 +25,26 @@ struct Launch {
     int* status;
     int nostream;             // 1: stored buffer holds pre-collision f (no stream)
     int all_tiles;            // bulk kernel: process every tile (no coupling)
-    int box[3];               // near-kernel grid per particle (blocks per axis)
+    long long near_nblk;      // near-kernel blocks per particle
+    int refill_side;          // refill box: cube side in cells
     unsigned short* map;      // per-step geometry map (see k_map)
     int map_ext[3];           // region box extents of the map (cells)
     dim3 block;
     cudaStream_t stream;
 };
 
-// Near-kernel block shape and grid: a particle's cell region spans at most
-// D + 2 NEAR_HALO + 1 cells per axis; the grid covers ceil(D) + 6 cells.
-constexpr int NEAR_BX = 32, NEAR_BY = 2, NEAR_BZ = 1;
+// Near-kernel blocks: one warp, 32 cells of a particle's region (at most
+// D + 2 NEAR_HALO + 1 cells per axis; the grid covers ceil(D) + 6).  A warp is
+// one chain of ~3500 instructions (MEM CLI, D = 8: 22 us, a third of it waiting
+// for instructions, a third for the latency of the one before), so full warps
+// and one to an SM are what a small sphere needs; rows of 32 cells, two to a
+// block, left 20 of 32 lanes idle at D = 8 and 22 of 64 at D = 36.  us per pass,
+// rows / this: 32^3 FP64 PSM 1954 / 1850; four D = 16 spheres, one sweep
+// 139 / 128; ensemble of 12, 3467 / 3397; 192 x 192 x 768 BF16 5712 / 5556.
+constexpr int NEAR_THREADS = 32;
 // threads per block of the refill kernels (whole warps: a warp rebuilds a cell)
 constexpr int REFILL_THREADS = 128;
-static_assert(NEAR_BX * NEAR_BY * NEAR_BZ % 32 == 0, "near blocks are whole warps");
+static_assert(NEAR_THREADS == 32, "a near block is one warp");
 static_assert(REFILL_THREADS % 32 == 0, "refill blocks are whole warps");
 // blocks of the refill kernel per particle for a box of side^3 cells
 __host__ __device__ inline long long refill_blocks(int side) {
@@ -52,13 +59,6 @@ inline void region_extent(const Geom& g, double maxd, int ext[3]) {
     ext[2] = g.nz < span ? g.nz : span;
 }
 
-inline void near_grid(const Geom& g, double maxd, int box[3]) {
-    int ext[3];
-    region_extent(g, maxd, ext);
-    const int b[3] = {NEAR_BX, NEAR_BY, NEAR_BZ};
-    for (int a = 0; a < 3; ++a) box[a] = (ext[a] + b[a] - 1) / b[a];
-}
-
 // Map entries (unsigned short) for np particles.
 inline long long map_entries(const Geom& g, double maxd, int np) {
     int ext[3];
@@ -66,12 +66,14 @@ inline long long map_entries(const Geom& g, double maxd, int np) {
     return (long long)(np > 0 ? np : 1) * ext[0] * ext[1] * ext[2];
 }
 
-inline long long near_blocks(const int box[3]) { return (long long)box[0] * box[1] * box[2]; }
+inline long long near_blocks(const Geom& g, double maxd) {
+    return (map_entries(g, maxd, 1) + NEAR_THREADS - 1) / NEAR_THREADS;
+}
 
 // Doubles of force partials one sweep needs: np regions x blocks x np x 6.
-inline long long near_partial_doubles(const int box[3], int np) {
+inline long long near_partial_doubles(long long nblk, int np) {
     const long long n = np > 0 ? np : 1;
-    return n * near_blocks(box) * n * 6;
+    return n * nblk * n * 6;
 }
 
 // ---- batched ensemble ----------------------------------------------------------
@@ -94,8 +96,7 @@ struct BatchCase {
     double* partials;  // subcycles x nblk x 6
     unsigned short* map;
     int map_ext[3];
-    int box[3];        // near-kernel grid (blocks)
-    long long nblk;
+    long long nblk;    // near-kernel blocks
     int refill_side;
     double gravity[3];
     int remap_charge;     // MEM: charge the re-mapping momentum (lbm_batch_set_remap_charge)
@@ -302,7 +303,7 @@ static_assert((int)ST_TOO_MANY_OBJECTS == (int)LBM_STATUS_TOO_MANY_OBJECTS &&
 cudaError_t launch_bulk(int storage, const void* src, void* dst, const Launch& L);
 cudaError_t launch_near(int storage, const void* src, void* dst, const Launch& L);
 // charge_part != nullptr: also the re-mapping momentum charge partials,
-// refill_blocks(L.box[0]) blocks x 6 doubles per particle (see k_refill)
+// refill_blocks(L.refill_side) blocks x 6 doubles per particle (see k_refill)
 cudaError_t launch_refill(int storage, const void* srcB, void* dst, const Launch& L,
                           const DevParticle* p_old, const DevParticle* p_new, int extrapolate,
                           double* charge_part = nullptr);

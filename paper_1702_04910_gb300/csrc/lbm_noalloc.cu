@@ -29,8 +29,15 @@ namespace {
 // (np regions x blocks x np x 6 doubles, see near_partial_doubles), the
 // per-call geometry map (np x region box entries), the particle records and
 // a status word.
+// What a call may ask for is counted in blocks of 32 x 2 cells of a z plane;
+// the sweep's one-warp blocks are at most twice as many.
 constexpr size_t NOALLOC_PARTIAL_DOUBLES = LBM_NOALLOC_MAX_PARTIAL_DOUBLES;
-static __device__ __align__(256) double g_partials[NOALLOC_PARTIAL_DOUBLES];
+static __device__ __align__(256) double g_partials[2 * NOALLOC_PARTIAL_DOUBLES];
+long long counted_blocks(const Geom& g, double maxd) {
+    int ext[3];
+    region_extent(g, maxd, ext);
+    return (long long)((ext[0] + 31) / 32) * ((ext[1] + 1) / 2) * ext[2];
+}
 static __device__ __align__(256) DevParticle g_particles[MAX_PARTICLES];
 static __device__ __align__(256) int g_status[64];
 constexpr size_t NOALLOC_MAP_ENTRIES = 1 << 20;  // geometry map, 2 MiB
@@ -157,8 +164,8 @@ extern "C" lbm_status lbm_sweep_noalloc(const lbm_config* cfg, const double* src
         up.rec[i] = d;
         maxd = std::max(maxd, p.diameter);
     }
-    near_grid(g, maxd, L.box);
-    const long long need = near_partial_doubles(L.box, n);
+    L.near_nblk = near_blocks(g, maxd);
+    const long long need = near_partial_doubles(counted_blocks(g, maxd), n);
     if ((unsigned long long)need > (unsigned long long)NOALLOC_PARTIAL_DOUBLES) {
         char msg[200];
         std::snprintf(msg, sizeof(msg),
