@@ -571,9 +571,19 @@ __device__ __forceinline__ void moments_j(const C (&f)[NQ], C& rho, C& jx, C& jy
 // f_q + l+ (f_q^+ - f^eq,+) + l- (f_q^- - f^eq,-) + F_q exactly.
 // C is the arithmetic type, KT the type of the constants (C itself, or float
 // for the packed f2: C(k.x) broadcasts a constant to both lanes).
-template <typename C, int Q, int K, bool FORCE, typename KT>
+// FUSE: P +- M without force as one FMA each, as the compiler contracts them in
+// the scalar form (the packed f2 operations are never contracted).
+template <typename C, int Q, int K, bool FORCE, bool FUSE, typename KT>
 __device__ __forceinline__ void trt_pair(C (&f)[NQ], C cu, const C (&bw)[3], const Coll<KT>& k) {
     constexpr int QB = Q + 1;
+    if constexpr (FUSE && !FORCE) {
+        const C P = fma(C(k.k1w[K]), cu * cu, bw[K]);
+        const C up = fma(C(k.k2w[K]), cu, P), dn = fma(C(-k.k2w[K]), cu, P);
+        const C a = f[Q], b = f[QB];
+        f[Q] = fma(C(k.alpha), a, fma(C(k.beta), b, -up));
+        f[QB] = fma(C(k.alpha), b, fma(C(k.beta), a, -dn));
+        return;
+    }
     C P = FORCE ? fma(C(k.k1w[K]), cu * cu, fma(C(-k.gq[(Q - 1) / 2]), cu, bw[K]))
                 : fma(C(k.k1w[K]), cu * cu, bw[K]);
     C M = FORCE ? fma(C(k.k2w[K]), cu, C(-k.fq[(Q - 1) / 2])) : C(k.k2w[K]) * cu;
@@ -621,6 +631,8 @@ __device__ __forceinline__ unsigned density_bad(f2 r) {
 // a bool, or a lane mask for the packed f2.
 template <typename C, bool FORCE, bool SHIFTED, typename KT>
 __device__ __forceinline__ auto collide_fluid_t(C (&f)[NQ], const Coll<KT>& k) {
+    // packed form of the unshifted populations: the scalar form's bits
+    constexpr bool FUSE = std::is_same<C, f2>::value && !SHIFTED;
     C rho, ux, uy, uz;
     moments_j(f, rho, ux, uy, uz);
     const auto bad = SHIFTED ? density_bad(rho + C(1)) : density_bad(rho);
@@ -636,15 +648,15 @@ __device__ __forceinline__ auto collide_fluid_t(C (&f)[NQ], const Coll<KT>& k) {
         for (int c = 0; c < 3; ++c) bw[c] = C(k.lpw[c]) * base;
     }
     f[0] = fma(C(k.c0), f[0], -bw[0]);
-    trt_pair<C, 1, 1, FORCE>(f, ux, bw, k);
-    trt_pair<C, 3, 1, FORCE>(f, uy, bw, k);
-    trt_pair<C, 5, 1, FORCE>(f, uz, bw, k);
-    trt_pair<C, 7, 2, FORCE>(f, ux + uy, bw, k);
-    trt_pair<C, 9, 2, FORCE>(f, ux - uy, bw, k);
-    trt_pair<C, 11, 2, FORCE>(f, ux + uz, bw, k);
-    trt_pair<C, 13, 2, FORCE>(f, ux - uz, bw, k);
-    trt_pair<C, 15, 2, FORCE>(f, uy + uz, bw, k);
-    trt_pair<C, 17, 2, FORCE>(f, uy - uz, bw, k);
+    trt_pair<C, 1, 1, FORCE, FUSE>(f, ux, bw, k);
+    trt_pair<C, 3, 1, FORCE, FUSE>(f, uy, bw, k);
+    trt_pair<C, 5, 1, FORCE, FUSE>(f, uz, bw, k);
+    trt_pair<C, 7, 2, FORCE, FUSE>(f, ux + uy, bw, k);
+    trt_pair<C, 9, 2, FORCE, FUSE>(f, ux - uy, bw, k);
+    trt_pair<C, 11, 2, FORCE, FUSE>(f, ux + uz, bw, k);
+    trt_pair<C, 13, 2, FORCE, FUSE>(f, ux - uz, bw, k);
+    trt_pair<C, 15, 2, FORCE, FUSE>(f, uy + uz, bw, k);
+    trt_pair<C, 17, 2, FORCE, FUSE>(f, uy - uz, bw, k);
     return bad;
 }
 

@@ -870,8 +870,9 @@ __global__ void __launch_bounds__(W, 768 / W)
 // 16-bit shifted storage where rows cannot be taken as aligned words (odd nx)
 // or the boundary planes have their own rules (open boundaries): each thread
 // takes the cells z and z + 1 of one column, with 2-byte accesses, and collides
-// them in the two lanes of the packed arithmetic on the shifted values, as
-// k_bulk_pair does.  One cell per thread in scalar FP32 was bound by issue
+// them in the two lanes of the packed arithmetic.  The weights are added to the
+// populations before and taken off after it, operation for operation as the
+// scalar FP32 form does, so every lane's result has its bits.  One cell per thread in scalar FP32 was bound by issue
 // (565 instructions per cell, 0.34 of HBM); this form halves the arithmetic
 // and the addresses: 101 x 101 x 304 cells FP16 85 us -> 73 us (k_near beside
 // it), 440 instructions per 64 cells, issue 57 %.
@@ -901,20 +902,6 @@ struct PullRaw<T, NQ> {
     __device__ __forceinline__ static void run(const T* __restrict__, const Geom&, const NbrOff&,
                                                long long, float (&)[NQ]) {}
 };
-// Shifted values pulled to cell (x, y, z).  The open boundaries work on f:
-// the cells of those planes take the plain pull and are shifted after it.
-template <typename T>
-__device__ __forceinline__ void pull_raw(const T* __restrict__ src, const Geom& g, int x, int y,
-                                         int z, long long idx, float (&f)[NQ]) {
-    const NbrOff o = make_off(g, x, y, z);
-    if (g.bc_z == 2 && (o.zlo || o.zhi)) {
-        pull_plain(src, g, x, y, z, idx, f);
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) f[q] -= (float)wq(q);
-    } else {
-        PullRaw<T, 0>::run(src, g, o, idx, f);
-    }
-}
 
 // Blocks are runs of 128 cells of a plane, x fastest (row tiles of 64 left a
 // fifth of the lanes of a 101-cell row idle).
@@ -936,13 +923,23 @@ __global__ void __launch_bounds__(ZPAIR_THREADS, ZPAIR_BLOCKS)
     if (!act0 && !act1) return;
     const long long idx = lin(g, x, y, z), plane = (long long)g.nx * g.ny;
     float a[NQ], b[NQ];
-    if (act0) pull_raw(src, g, x, y, z, idx, a);
-    if (act1) pull_raw(src, g, x, y, z + 1, idx + plane, b);
     f2 f[NQ];
+    if (g.bc_z == 2 && (z == 0 || z + 2 >= g.nz)) {  // a boundary plane (block-uniform)
+        if (act0) pull_plain(src, g, x, y, z, idx, a);
+        if (act1) pull_plain(src, g, x, y, z + 1, idx + plane, b);
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) f[q] = f2(make_float2(act0 ? a[q] : 0.0f, act1 ? b[q] : 0.0f));
-    const unsigned bad = collide_fluid<f2, true>(f, k);
+        for (int q = 0; q < NQ; ++q) f[q] = f2(make_float2(act0 ? a[q] : 0.0f, act1 ? b[q] : 0.0f));
+    } else {
+        if (act0) PullRaw<T, 0>::run(src, g, make_off(g, x, y, z), idx, a);
+        if (act1) PullRaw<T, 0>::run(src, g, make_off(g, x, y, z + 1), idx + plane, b);
+#pragma unroll
+        for (int q = 0; q < NQ; ++q)
+            f[q] = f2(make_float2(act0 ? a[q] : 0.0f, act1 ? b[q] : 0.0f)) + f2((float)wq(q));
+    }
+    const unsigned bad = collide_fluid<f2>(f, k);
     if (((bad & 1u) && act0) || ((bad & 2u) && act1)) atomicOr(status, ST_FLUID);
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) f[q] = f[q] - f2((float)wq(q));
     if (act0)
 #pragma unroll
         for (int q = 0; q < NQ; ++q) dst[(long long)q * g.n + idx] = Pair16<T>::one(f[q].v.x);
