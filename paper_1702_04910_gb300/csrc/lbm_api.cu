@@ -156,6 +156,7 @@ Launch base_launch(lbm_handle* h) {
     L.status = h->d_status;
     L.nostream = 0;
     L.all_tiles = 0;
+    L.beside = 0;
     L.block = dim3(h->g.tx, h->g.ty, 1);
     L.stream = h->stream;
     L.near_nblk = near_blocks(h->g, h->maxd);
@@ -271,6 +272,12 @@ lbm_status sweep(lbm_handle* h, int sub, bool with_map) {
     L.partials = h->d_partials + (size_t)sub * (size_t)near_partial_doubles(L.near_nblk, h->np);
     const void* src = h->buf[h->cur];
     void* dst = h->buf[1 - h->cur];
+    if (!h->profiling && sweep_fused(L, h->bulk_mode)) {
+        if (with_map) CK(h, launch_map(L), "geometry map launch");
+        CK(h, launch_sweep(h->storage, src, dst, L), "sweep launch");
+        h->cur = 1 - h->cur;
+        return LBM_OK;
+    }
     // The near-particle cells and the bulk cells are disjoint: the (small,
     // latency-bound) near sweep runs on a private stream beside k_bulk.
     if (h->np > 0) {

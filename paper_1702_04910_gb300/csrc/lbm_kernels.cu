@@ -30,6 +30,26 @@
 namespace lbmgpu {
 
 // ---------------------------------------------------------------------------
+// Programmatic dependent launch.  The kernels of a step are short and follow one
+// another on a stream, so each is launched while its predecessor still runs
+// (launch_after below): its blocks take their places and wait here until the
+// predecessor has completed and its writes are visible, then let the successor
+// be launched in turn.  Every kernel launched that way calls this before it
+// touches memory, so a kernel's completion implies that of all before it.
+__device__ __forceinline__ void step_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void step_enter() {
+    step_wait();
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+// A pointer whose loads cannot be moved ahead of step_enter (they may be
+// declared invariant).
+template <typename P>
+__device__ __forceinline__ P* entered(P* p) {
+    asm volatile("" : "+l"(p));
+    return p;
+}
+
+// ---------------------------------------------------------------------------
 // per-cell force/torque slots (a cell may touch up to CELL_SLOTS particles)
 struct Slots {
     int id[CELL_SLOTS];
@@ -711,9 +731,15 @@ __device__ __forceinline__ void bulk_tile(const T* __restrict__ src, T* __restri
 template <typename T, typename C, bool NOSTREAM, int CPT>
 __global__ void __launch_bounds__(BulkShape<T, C>::threads, BulkShape<T, C>::blocks)
     k_bulk(const T* __restrict__ src, T* __restrict__ dst, Geom g, Coll<C> k,
-           const DevParticle* __restrict__ parts, int np, int all_tiles, int* __restrict__ status) {
+           const DevParticle* __restrict__ parts, int np, int all_tiles, int* __restrict__ status,
+           int beside) {
     bulk_tile<T, C, NOSTREAM, CPT>(src, dst, g, k, parts, np, all_tiles, blockIdx.x, blockIdx.y,
                                    blockIdx.z, threadIdx.x, threadIdx.y, status);
+    // launched beside k_near (which has waited for everything before the two):
+    // the grid completes only after k_near, for the kernels that follow both
+    if (beside && threadIdx.x == 0 && threadIdx.y == 0 && blockIdx.x == gridDim.x - 1 &&
+        blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1)
+        step_wait();
 }
 
 // ---------------------------------------------------------------------------
@@ -1203,12 +1229,54 @@ __global__ void __launch_bounds__(NEAR_THREADS)
            int* __restrict__ status) {
     extern __shared__ double sp_words[];
     __shared__ typename std::conditional<KIND == 2, LinkWarp, char>::type lw;
+    step_enter();
+    parts = entered(parts);
+    src = entered(src);
+    gm.map = entered(gm.map);
     for (int i = threadIdx.x; i < cp.np * (int)(sizeof(DevParticle) / sizeof(double)); i += NEAR_THREADS)
         sp_words[i] = reinterpret_cast<const double*>(parts)[i];
     __syncwarp();
     near_block<T, C, KIND, NOSTREAM>(src, dst, g, k, cp,
                                      reinterpret_cast<const DevParticle*>(sp_words), gm, partials,
                                      status, blockIdx.y, gridDim.x, blockIdx.x, lw);
+}
+
+// One sweep of a small lattice (FP64 or FP32 PDFs, MEM or PSM) in one launch:
+// blocks 0 .. nblk * np - 1 are k_near's, the others take 32 consecutive cells of
+// the lattice each, as k_bulk collides them, and skip k_near's cells.  Where the
+// bulk cells are done before the chain of a near block is (SWEEP_FUSED_CELLS),
+// a second stream beside it only adds its fork and join to the step.
+template <typename T, typename C, int KIND>
+__global__ void __launch_bounds__(NEAR_THREADS)
+    k_sweep(const T* __restrict__ src, T* __restrict__ dst, Geom g, Coll<C> k, Coupl cp,
+            const DevParticle* __restrict__ parts, GeoMap gm, double* __restrict__ partials,
+            int* __restrict__ status, unsigned nblk) {
+    extern __shared__ double sp_words[];
+    __shared__ typename std::conditional<KIND == 2, LinkWarp, char>::type lw;
+    step_enter();
+    parts = entered(parts);
+    src = entered(src);
+    gm.map = entered(gm.map);
+    for (int i = threadIdx.x; i < cp.np * (int)(sizeof(DevParticle) / sizeof(double)); i += NEAR_THREADS)
+        sp_words[i] = reinterpret_cast<const double*>(parts)[i];
+    __syncwarp();
+    const DevParticle* sp = reinterpret_cast<const DevParticle*>(sp_words);
+    const unsigned nnear = nblk * cp.np;
+    if (blockIdx.x < nnear) {
+        near_block<T, C, KIND, false>(src, dst, g, k, cp, sp, gm, partials, status,
+                                      blockIdx.x / nblk, nblk, blockIdx.x % nblk, lw);
+        return;
+    }
+    const unsigned idx = (blockIdx.x - nnear) * NEAR_THREADS + threadIdx.x;
+    if (idx >= (unsigned)g.n) return;
+    const unsigned row = idx / g.nx;
+    const int x = (int)(idx - row * g.nx), z = (int)(row / g.ny), y = (int)(row - z * g.ny);
+    for (int s = 0; s < cp.np; ++s)
+        if (cell_in_reg(g, sp[s].reg, x, y, z)) return;
+    C f[NQ];
+    pull_plain(src, g, x, y, z, (long long)idx, f);
+    if (collide_cell(f, k)) atomicOr(status, ST_FLUID);
+    store_own(dst, g, (long long)idx, f);
 }
 
 // ---------------------------------------------------------------------------
@@ -1260,6 +1328,8 @@ __global__ void __launch_bounds__(32)
     k_map(Geom g, Coupl cp, const DevParticle* __restrict__ parts, unsigned short* __restrict__ map,
           int ex, int ey, int ez) {
     __shared__ DevParticle sp[MAX_PARTICLES];
+    step_enter();
+    parts = entered(parts);
     const int nd = cp.np * (int)(sizeof(DevParticle) / sizeof(double));
     for (int i = threadIdx.x; i < nd; i += blockDim.x)
         reinterpret_cast<double*>(sp)[i] = reinterpret_cast<const double*>(parts)[i];
@@ -1306,7 +1376,9 @@ __global__ void __launch_bounds__(FIN_THREADS)
     k_finalize(int np, long long nblk, const double* __restrict__ partials, int nsub,
                double* __restrict__ out, const double* __restrict__ charge) {
     __shared__ double red[FIN_THREADS];
-    finalize_block(np, nblk, partials, nsub, out, blockIdx.x, red, charge);
+    step_enter();
+    finalize_block(np, nblk, entered(partials), nsub, out, blockIdx.x, red,
+                   charge ? entered(charge) : nullptr);
 }
 
 // ---------------------------------------------------------------------------
@@ -1378,6 +1450,9 @@ __global__ void __launch_bounds__(32)
     k_rigid(Geom g, DevParticle* __restrict__ parts, DevParticle* __restrict__ prev,
             const double* __restrict__ force, double rho0, double gx, double gy, double gz,
             double dt, int wall_contact, int* __restrict__ status) {
+    step_enter();
+    parts = entered(parts);
+    force = entered(force);
     const int p = blockIdx.x;
     rigid_one(g, parts + p, prev + p, force + 6 * p, rho0, gx, gy, gz, dt, wall_contact, status);
 }
@@ -1390,14 +1465,19 @@ __global__ void __launch_bounds__(FIN_THREADS)
                      DevParticle* prev, double rho0, double gx, double gy, double gz, double dt,
                      int wall_contact, int* status) {
     __shared__ double red[FIN_THREADS];
+    step_enter();
+    parts = entered(parts);
     const int p = blockIdx.x;
-    finalize_block(np, nblk, partials, nsub, force, p, red, charge);
+    finalize_block(np, nblk, entered(partials), nsub, force, p, red,
+                   charge ? entered(charge) : nullptr);
     __syncthreads();
     if (threadIdx.x < 32)
         rigid_one(g, parts + p, prev + p, force + 6 * p, rho0, gx, gy, gz, dt, wall_contact, status);
 }
 
 __global__ void k_regions(Geom g, DevParticle* parts, int np) {
+    step_enter();
+    parts = entered(parts);
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p < np) store_region(g, parts[p]);
 }
@@ -1754,6 +1834,10 @@ __global__ void __launch_bounds__(REFILL_THREADS)
              double* __restrict__ charge_part) {
     __shared__ DevParticle so[MAX_PARTICLES], sn[MAX_PARTICLES];
     const int tid = threadIdx.x;
+    step_enter();
+    p_old = entered(p_old);
+    p_new = entered(p_new);
+    srcB = entered(srcB);
     const int nd = cp.np * (int)(sizeof(DevParticle) / sizeof(double));
     for (int i = tid; i < nd; i += blockDim.x) {
         reinterpret_cast<double*>(so)[i] = reinterpret_cast<const double*>(p_old)[i];
@@ -1788,7 +1872,8 @@ __device__ __forceinline__ void charge_total(long long nblk, const double* __res
 // one block of six warps per particle
 __global__ void __launch_bounds__(192)
     k_charge_total(long long nblk, const double* __restrict__ part, double* __restrict__ out) {
-    charge_total(nblk, part + (long long)blockIdx.x * nblk * 6, out + blockIdx.x * 6);
+    step_enter();
+    charge_total(nblk, entered(part) + (long long)blockIdx.x * nblk * 6, out + blockIdx.x * 6);
 }
 
 // ---------------------------------------------------------------------------
@@ -2128,23 +2213,30 @@ namespace {
 // 2980 / 3110.
 constexpr int SMEM_CARVEOUT = 50;  // percent of the largest shared-memory size
 template <typename... P, typename... A>
-cudaError_t launch_smem(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                        A&&... args) {
+cudaError_t launch_with(bool early, size_t smem, void (*kernel)(P...), dim3 grid, dim3 block,
+                        cudaStream_t s, A&&... args) {
     cudaLaunchConfig_t c{};
     c.dynamicSmemBytes = smem;
     c.gridDim = grid;
     c.blockDim = block;
     c.stream = s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
     at[0].val.sharedMemCarveout = SMEM_CARVEOUT;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     c.attrs = at;
-    c.numAttrs = 1;
+    c.numAttrs = early ? 2 : 1;
     return cudaLaunchKernelEx(&c, kernel, std::forward<A>(args)...);
 }
 template <typename... P, typename... A>
 cudaError_t launch(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t s, A&&... args) {
-    return launch_smem(kernel, grid, block, 0, s, std::forward<A>(args)...);
+    return launch_with(false, 0, kernel, grid, block, s, std::forward<A>(args)...);
+}
+// for kernels that begin with step_enter
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t s, A&&... args) {
+    return launch_with(true, 0, kernel, grid, block, s, std::forward<A>(args)...);
 }
 
 template <typename T, typename C>
@@ -2166,11 +2258,12 @@ template <typename T, typename C, int CPT>
 cudaError_t bulk_cpt(const void* src, void* dst, const Launch& L) {
     dim3 grid(L.g.ntx, L.g.nty, L.g.ntz);
     const auto& k = coll_of<typename std::conditional<(sizeof(T) < 4), C, T>::type, C>(L);
+    const bool beside = L.beside != 0;
     if (L.nostream)
-        return launch(k_bulk<T, C, true, CPT>, grid, L.block, L.stream, (const T*)src, (T*)dst, L.g,
-                      k, L.parts, L.cp.np, L.all_tiles, L.status);
-    return launch(k_bulk<T, C, false, CPT>, grid, L.block, L.stream, (const T*)src, (T*)dst, L.g, k,
-                  L.parts, L.cp.np, L.all_tiles, L.status);
+        return launch_with(beside, 0, k_bulk<T, C, true, CPT>, grid, L.block, L.stream, (const T*)src,
+                           (T*)dst, L.g, k, L.parts, L.cp.np, L.all_tiles, L.status, L.beside);
+    return launch_with(beside, 0, k_bulk<T, C, false, CPT>, grid, L.block, L.stream, (const T*)src,
+                       (T*)dst, L.g, k, L.parts, L.cp.np, L.all_tiles, L.status, L.beside);
 }
 
 // FP64-state sweeps are arithmetic bound and use one cell per thread; the
@@ -2213,11 +2306,24 @@ cudaError_t near_kind(const void* src, void* dst, const Launch& L) {
     const size_t smem = sizeof(DevParticle) * L.cp.np;
     const auto& k = coll_of<C, C>(L);
     const GeoMap gm{L.map, L.map_ext[0], L.map_ext[1], L.map_ext[2]};
+    // 16 bits: not launched ahead of the map's end, where its registers would be
+    // held back from the bulk sweep for longer
+    constexpr bool early = sizeof(T) > 2;
     if (L.nostream)
-        return launch_smem(k_near<T, C, KIND, true>, grid, block, smem, L.stream, (const T*)src,
+        return launch_with(early, smem, k_near<T, C, KIND, true>, grid, block, L.stream, (const T*)src,
                            (T*)dst, L.g, k, L.cp, L.parts, gm, L.partials, L.status);
-    return launch_smem(k_near<T, C, KIND, false>, grid, block, smem, L.stream, (const T*)src, (T*)dst,
-                       L.g, k, L.cp, L.parts, gm, L.partials, L.status);
+    return launch_with(early, smem, k_near<T, C, KIND, false>, grid, block, L.stream, (const T*)src,
+                       (T*)dst, L.g, k, L.cp, L.parts, gm, L.partials, L.status);
+}
+
+template <typename T, int KIND>
+cudaError_t sweep_kind(const void* src, void* dst, const Launch& L) {
+    const unsigned nblk = (unsigned)L.near_nblk;
+    const dim3 grid(nblk * L.cp.np + (unsigned)((L.g.n + NEAR_THREADS - 1) / NEAR_THREADS));
+    const GeoMap gm{L.map, L.map_ext[0], L.map_ext[1], L.map_ext[2]};
+    return launch_with(true, sizeof(DevParticle) * L.cp.np, k_sweep<T, T, KIND>, grid,
+                       dim3(NEAR_THREADS), L.stream, (const T*)src, (T*)dst, L.g, coll_of<T, T>(L),
+                       L.cp, L.parts, gm, L.partials, L.status, nblk);
 }
 
 template <typename T>
@@ -2235,7 +2341,7 @@ cudaError_t refill_t(const void* srcB, void* dst, const Launch& L, const DevPart
     if (L.cp.np <= 0) return cudaSuccess;
     const int side = L.refill_side;
     dim3 grid((unsigned)refill_blocks(side), L.cp.np, 1);
-    return launch(k_refill<T, C>, grid, REFILL_THREADS, L.stream, (const T*)srcB, (T*)dst, L.g,
+    return launch_after(k_refill<T, C>, grid, REFILL_THREADS, L.stream, (const T*)srcB, (T*)dst, L.g,
                   coll_of<C, C>(L), L.cp, po, pn, extrapolate, side, L.status, charge_part);
 }
 
@@ -2297,6 +2403,15 @@ cudaError_t launch_near(int storage, const void* src, void* dst, const Launch& L
         default: return near_t<double>(src, dst, L);
     }
 }
+bool sweep_fused(const Launch& L, int bulk_mode) {
+    return L.cp.np > 0 && (L.cp.kind == 1 || L.cp.kind == 2) && !L.nostream &&
+           (bulk_mode == 0 || bulk_mode == 1 || bulk_mode == 3) && L.g.n <= SWEEP_FUSED_CELLS;
+}
+cudaError_t launch_sweep(int storage, const void* src, void* dst, const Launch& L) {
+    if (storage == 1)
+        return L.cp.kind == 1 ? sweep_kind<float, 1>(src, dst, L) : sweep_kind<float, 2>(src, dst, L);
+    return L.cp.kind == 1 ? sweep_kind<double, 1>(src, dst, L) : sweep_kind<double, 2>(src, dst, L);
+}
 cudaError_t launch_refill(int storage, const void* srcB, void* dst, const Launch& L,
                           const DevParticle* p_old, const DevParticle* p_new, int extrapolate,
                           double* charge_part) {
@@ -2310,7 +2425,7 @@ cudaError_t launch_refill(int storage, const void* srcB, void* dst, const Launch
 }
 cudaError_t launch_charge_total(const Launch& L, const double* charge_part, double* charge) {
     if (L.cp.np <= 0) return cudaSuccess;
-    return launch(k_charge_total, L.cp.np, 192, L.stream, refill_blocks(L.refill_side), charge_part,
+    return launch_after(k_charge_total, L.cp.np, 192, L.stream, refill_blocks(L.refill_side), charge_part,
                   charge);
 }
 cudaError_t launch_macro(int storage, const void* state, const Launch& L, int what, void* out) {
@@ -2354,33 +2469,33 @@ cudaError_t launch_map(const Launch& L) {
     if (L.cp.np <= 0 || L.cp.kind == 0) return cudaSuccess;
     dim3 grid((L.map_ext[0] + 31) / 32, L.map_ext[1], L.map_ext[2] * L.cp.np);
     if (L.cp.kind == 2)
-        return launch(k_map<2>, grid, 32, L.stream, L.g, L.cp, L.parts, L.map, L.map_ext[0],
+        return launch_after(k_map<2>, grid, 32, L.stream, L.g, L.cp, L.parts, L.map, L.map_ext[0],
                       L.map_ext[1], L.map_ext[2]);
-    return launch(k_map<1>, grid, 32, L.stream, L.g, L.cp, L.parts, L.map, L.map_ext[0], L.map_ext[1],
+    return launch_after(k_map<1>, grid, 32, L.stream, L.g, L.cp, L.parts, L.map, L.map_ext[0], L.map_ext[1],
                   L.map_ext[2]);
 }
 
 cudaError_t launch_finalize(const Launch& L, int nsub, double* force_out, const double* charge) {
     if (L.cp.np <= 0) return cudaSuccess;
-    return launch(k_finalize, L.cp.np, FIN_THREADS, L.stream, L.cp.np, L.near_nblk, L.partials, nsub,
+    return launch_after(k_finalize, L.cp.np, FIN_THREADS, L.stream, L.cp.np, L.near_nblk, L.partials, nsub,
                   force_out, charge);
 }
 cudaError_t launch_rigid_body(const Launch& L, const double* force, double gx, double gy,
                               double gz, double dt, int wall_contact) {
     if (L.cp.np <= 0) return cudaSuccess;
-    return launch(k_rigid, L.cp.np, 32, L.stream, L.g, L.parts, L.parts_prev, force, L.kd.rho0, gx,
+    return launch_after(k_rigid, L.cp.np, 32, L.stream, L.g, L.parts, L.parts_prev, force, L.kd.rho0, gx,
                   gy, gz, dt, wall_contact, L.status);
 }
 cudaError_t launch_finalize_rigid(const Launch& L, int nsub, double* force, const double* charge,
                                   double gx, double gy, double gz, int wall_contact) {
     if (L.cp.np <= 0) return cudaSuccess;
-    return launch(k_finalize_rigid, L.cp.np, FIN_THREADS, L.stream, L.g, L.cp.np,
+    return launch_after(k_finalize_rigid, L.cp.np, FIN_THREADS, L.stream, L.g, L.cp.np,
                   L.near_nblk, L.partials, nsub, force, charge, L.parts, L.parts_prev,
                   L.kd.rho0, gx, gy, gz, (double)nsub, wall_contact, L.status);
 }
 cudaError_t launch_regions(const Launch& L) {
     if (L.cp.np <= 0) return cudaSuccess;
-    return launch(k_regions, 1, 32, L.stream, L.g, L.parts, L.cp.np);
+    return launch_after(k_regions, 1, 32, L.stream, L.g, L.parts, L.cp.np);
 }
 
 

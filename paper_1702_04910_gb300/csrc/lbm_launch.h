@@ -25,6 +25,7 @@ struct Launch {
     int* status;
     int nostream;             // 1: stored buffer holds pre-collision f (no stream)
     int all_tiles;            // bulk kernel: process every tile (no coupling)
+    int beside;               // FP64 bulk sweep right after launch_near on the same stream: runs beside it
     long long near_nblk;      // near-kernel blocks per particle
     int refill_side;          // refill box: cube side in cells
     unsigned short* map;      // per-step geometry map (see k_map)
@@ -302,6 +303,14 @@ static_assert((int)ST_TOO_MANY_OBJECTS == (int)LBM_STATUS_TOO_MANY_OBJECTS &&
 // storage with 64-bit fixed-point collision
 cudaError_t launch_bulk(int storage, const void* src, void* dst, const Launch& L);
 cudaError_t launch_near(int storage, const void* src, void* dst, const Launch& L);
+// Whether a sweep runs as one launch (launch_sweep: near and bulk cells), and the
+// largest lattice that does.  us for 20 steps, near sweep on a second stream /
+// one launch: FP64 PSM 32^3 756 / 643, 64^3 964 / 872, 80^3 1400 / 1469; FP64 MEM
+// (two sweeps a step) 32^3 1221 / 1050, 64^3 1777 / 1571, 80^3 2511 / 2476; FP32
+// PSM 64^3 684 / 637, 80^3 793 / 936; FP32 MEM 64^3 1512 / 1257, 80^3 1745 / 1491.
+constexpr long long SWEEP_FUSED_CELLS = 1 << 18;
+bool sweep_fused(const Launch& L, int bulk_mode);
+cudaError_t launch_sweep(int storage, const void* src, void* dst, const Launch& L);
 // charge_part != nullptr: also the re-mapping momentum charge partials,
 // refill_blocks(L.refill_side) blocks x 6 doubles per particle (see k_refill)
 cudaError_t launch_refill(int storage, const void* srcB, void* dst, const Launch& L,

@@ -232,8 +232,15 @@ extern "C" lbm_status lbm_sweep_noalloc(const lbm_config* cfg, const double* src
         if (e == cudaSuccess) e = launch_regions(L);
         if (e == cudaSuccess) e = launch_map(L);
     }
-    if (e == cudaSuccess) e = launch_bulk(0, src_pdf_dev, dst_pdf_dev, L);
-    if (e == cudaSuccess && n > 0) e = launch_near(0, src_pdf_dev, dst_pdf_dev, L);
+    if (sweep_fused(L, 0)) {
+        if (e == cudaSuccess) e = launch_sweep(0, src_pdf_dev, dst_pdf_dev, L);
+    } else {
+        // near sweep first: its blocks are placed, then the bulk sweep runs
+        // beside it
+        if (e == cudaSuccess && n > 0) e = launch_near(0, src_pdf_dev, dst_pdf_dev, L);
+        L.beside = n > 0;
+        if (e == cudaSuccess) e = launch_bulk(0, src_pdf_dev, dst_pdf_dev, L);
+    }
     if (e == cudaSuccess && n > 0) e = launch_finalize(L, 1, force_torque_dev);
     if (e != cudaSuccess) {
         set_err(err, err_len, cudaGetErrorString(e));
