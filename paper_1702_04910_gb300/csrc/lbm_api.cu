@@ -66,7 +66,7 @@ struct lbm_handle {
     size_t partial_cap;  // doubles allocated in d_partials
     unsigned short* d_map;  // per-step geometry map [np][region box]
     size_t map_cap;         // entries allocated in d_map
-    int* d_status;
+    int* d_status;       // in front of d_force, so that both are read in one copy
     double* h_stage;     // pinned: status word + np*6 forces
     size_t dev_bytes;
     Coll<double> kd;
@@ -170,13 +170,12 @@ lbm_status free_particles(lbm_handle* h) {
     cudaFree(h->d_parts);
     cudaFree(h->d_prev);
     cudaFree(h->d_tmp);
-    cudaFree(h->d_force);
     cudaFree(h->d_partials);
     cudaFree(h->d_map);
     cudaFree(h->d_charge);
     cudaFree(h->d_charge_part);
     h->d_parts = h->d_prev = h->d_tmp = nullptr;
-    h->d_force = h->d_partials = nullptr;
+    h->d_partials = nullptr;
     h->d_map = nullptr;
     h->map_cap = 0;
     h->d_charge = h->d_charge_part = nullptr;
@@ -193,7 +192,6 @@ lbm_status alloc_particles(lbm_handle* h, int n) {
     CK(h, cudaMalloc(&h->d_parts, part_bytes), "cudaMalloc particles");
     CK(h, cudaMalloc(&h->d_prev, part_bytes), "cudaMalloc particles");
     CK(h, cudaMalloc(&h->d_tmp, part_bytes), "cudaMalloc particles");
-    CK(h, cudaMalloc(&h->d_force, sizeof(double) * 6 * np), "cudaMalloc forces");
     CK(h, cudaMemsetAsync(h->d_force, 0, sizeof(double) * 6 * np, h->stream), "memset");
     CK(h, cudaMalloc(&h->d_charge, sizeof(double) * 6 * np), "cudaMalloc charge");
     CK(h, cudaMemsetAsync(h->d_charge, 0, sizeof(double) * 6 * np, h->stream), "memset");
@@ -361,10 +359,12 @@ lbm_status step_once(lbm_handle* h) {
     return LBM_OK;
 }
 
-lbm_status read_status(lbm_handle* h) {
+// forces: how many doubles of d_force come with the status word (h_stage + 1).
+lbm_status read_status(lbm_handle* h, int forces = 0) {
     int st = 0;
-    CK(h, cudaMemcpyAsync(&h->h_stage[0], h->d_status, sizeof(int), cudaMemcpyDeviceToHost,
-                          h->stream),
+    CK(h, cudaMemcpyAsync(&h->h_stage[0], h->d_status,
+                          forces ? sizeof(double) * (1 + forces) : sizeof(int),
+                          cudaMemcpyDeviceToHost, h->stream),
        "status copy");
     CK(h, cudaStreamSynchronize(h->stream), "stream synchronize");
     std::memcpy(&st, &h->h_stage[0], sizeof(int));
@@ -406,7 +406,7 @@ const char* lbm_last_error(const lbm_handle* h) {
 size_t lbm_device_bytes(const lbm_handle* h) {
     if (!h) return 0;
     const size_t np = (size_t)std::max(h->np, 1);
-    return h->dev_bytes + 3 * sizeof(DevParticle) * np + sizeof(double) * 6 * np +
+    return h->dev_bytes + 3 * sizeof(DevParticle) * np +
            sizeof(double) * h->partial_cap + sizeof(unsigned short) * h->map_cap +
            sizeof(double) * 6 * np + sizeof(double) * h->charge_part_cap;
 }
@@ -474,13 +474,14 @@ lbm_status lbm_create(const lbm_config* cfg, void* stream, lbm_handle** out) {
     size_t bytes = (size_t)NQ * (size_t)n * h->esize;
     cudaError_t e = cudaMalloc(&h->buf[0], bytes);
     if (e == cudaSuccess) e = cudaMalloc(&h->buf[1], bytes);
-    if (e == cudaSuccess) e = cudaMalloc(&h->d_status, sizeof(int));
+    if (e == cudaSuccess) e = cudaMalloc(&h->d_status, sizeof(double) * (1 + 6 * MAX_PARTICLES));
     if (e != cudaSuccess) {
         lbm_status st = cuda_fail(h, e, "cudaMalloc PDF buffers");
         lbm_destroy(h);
         return st;
     }
-    h->dev_bytes = 2 * bytes + sizeof(int);
+    h->d_force = reinterpret_cast<double*>(h->d_status) + 1;
+    h->dev_bytes = 2 * bytes + sizeof(double) * (1 + 6 * MAX_PARTICLES);
     cudaMemsetAsync(h->d_status, 0, sizeof(int), h->stream);
     lbm_status st = alloc_particles(h, 0);
     if (st == LBM_OK) st = ensure_partials(h);
@@ -545,7 +546,7 @@ lbm_status lbm_set_particles(lbm_handle* h, int n, const lbm_particle* host_in) 
     const bool remap = h->have_particles && h->kind == 2 && n == h->np && n > 0;
     if (h->have_particles && h->kind == 2 && n != h->np && h->np > 0)
         return fail(h, LBM_ERR_ARG, "the particle count cannot change once MEM particles are mapped");
-    std::vector<DevParticle> recs((size_t)std::max(n, 1));
+    ParticleUpload up{};
     for (int i = 0; i < n; ++i) {
         const lbm_particle& p = host_in[i];
         DevParticle d{};
@@ -564,40 +565,27 @@ lbm_status lbm_set_particles(lbm_handle* h, int n, const lbm_particle* host_in) 
         d.r = 0.5 * p.diameter;
         d.rho = p.density;
         d.fixed = p.fixed ? 1.0 : 0.0;
-        recs[i] = d;
+        up.rec[i] = d;
     }
     if (n != h->np || !h->d_parts) {
         h->np = n;
         lbm_status st = alloc_particles(h, n);
         if (st != LBM_OK) return st;
     }
-    // a replacement from the host clears the pending re-mapping charge
-    CK(h, cudaMemsetAsync(h->d_charge, 0, sizeof(double) * 6 * (size_t)std::max(n, 1), h->stream),
-       "charge reset");
+    // a replacement from the host clears the pending re-mapping charge (kept only while it is on)
+    if (h->remap_charge)
+        CK(h, cudaMemsetAsync(h->d_charge, 0, sizeof(double) * 6 * (size_t)std::max(n, 1), h->stream),
+           "charge reset");
     h->maxd = std::max(h->maxd, maxd);
     {
         lbm_status st = ensure_partials(h);
         if (st != LBM_OK) return st;
     }
-    if (remap)
-        CK(h, cudaMemcpyAsync(h->d_tmp, h->d_parts, sizeof(DevParticle) * n,
-                              cudaMemcpyDeviceToDevice, h->stream),
-           "particle copy");
-    if (n > 0) {
-        CK(h, cudaMemcpyAsync(h->d_parts, recs.data(), sizeof(DevParticle) * n,
-                              cudaMemcpyHostToDevice, h->stream),
-           "particle upload");
-        CK(h, cudaMemcpyAsync(h->d_prev, recs.data(), sizeof(DevParticle) * n,
-                              cudaMemcpyHostToDevice, h->stream),
-           "particle upload");
-    }
-    CK(h, cudaStreamSynchronize(h->stream), "particle upload sync");  // recs is pageable
     Launch L = base_launch(h);
-    CK(h, launch_regions(L), "region launch");
-    L.parts = h->d_prev;
-    CK(h, launch_regions(L), "region launch");
+    if (n > 0)
+        CK(h, launch_set_particles(L, up, n, h->d_parts, h->d_prev, remap ? h->d_tmp : nullptr),
+           "particle upload");
     if (remap) {
-        L = base_launch(h);
         CK(h, launch_refill(h->storage, h->buf[1 - h->cur], h->buf[h->cur], L, h->d_tmp, h->d_parts, 0),
            "refill launch");
     }
@@ -650,10 +638,7 @@ lbm_status lbm_get_forces(lbm_handle* h, double* F, double* T) {
     if (!h) return LBM_ERR_ARG;
     if (h->np == 0) return read_status(h);
     if (!F || !T) return fail(h, LBM_ERR_ARG, "null output");
-    CK(h, cudaMemcpyAsync(h->h_stage + 1, h->d_force, sizeof(double) * 6 * h->np,
-                          cudaMemcpyDeviceToHost, h->stream),
-       "force download");
-    lbm_status st = read_status(h);
+    lbm_status st = read_status(h, 6 * h->np);
     for (int i = 0; i < h->np; ++i)
         for (int a = 0; a < 3; ++a) {
             F[3 * i + a] = h->h_stage[1 + 6 * i + a];

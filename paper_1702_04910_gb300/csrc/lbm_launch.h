@@ -332,7 +332,15 @@ cudaError_t launch_finalize(const Launch& L, int nsub, double* force_out,
 // the force total and the rigid-body update (dt = nsub) in one launch
 cudaError_t launch_finalize_rigid(const Launch& L, int nsub, double* force, const double* charge,
                                   double gx, double gy, double gz, int wall_contact);
-cudaError_t launch_regions(const Launch& L);
+// Stores n particle records with their regions in parts (and prev), the records
+// that parts held before in old (prev, old: may be null).  The records travel as
+// a kernel argument, copied at launch: nothing waits for the host array.
+struct ParticleUpload {
+    DevParticle rec[MAX_PARTICLES];
+};
+static_assert(sizeof(ParticleUpload) <= 16000, "kernel argument too large");
+cudaError_t launch_set_particles(const Launch& L, const ParticleUpload& up, int n, DevParticle* parts,
+                                 DevParticle* prev, DevParticle* old);
 // batched ensemble (all cases on one stream; see lbm_batch.cu)
 cudaError_t launch_batch_regions(BatchCase* cases, int n, cudaStream_t s);
 cudaError_t launch_batch_map(BatchCase* cases, BatchList l, long long total, cudaStream_t s);

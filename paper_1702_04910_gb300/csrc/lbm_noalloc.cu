@@ -43,18 +43,6 @@ static __device__ __align__(256) int g_status[64];
 constexpr size_t NOALLOC_MAP_ENTRIES = 1 << 20;  // geometry map, 2 MiB
 static __device__ __align__(256) unsigned short g_map[NOALLOC_MAP_ENTRIES];
 
-// Particle records passed by value to the kernel that stores them in
-// g_particles (32 x 160 B: within the 32 KiB kernel-argument limit).
-struct ParticleUpload {
-    DevParticle rec[MAX_PARTICLES];
-};
-static_assert(sizeof(ParticleUpload) <= 32000, "kernel argument too large");
-
-__global__ void k_upload_particles(ParticleUpload up, int n) {
-    const int i = threadIdx.x;
-    if (i < n && i < MAX_PARTICLES) g_particles[i] = up.rec[i];
-}
-
 constexpr int MAX_DEVICES = 64;
 struct Addresses {
     bool ready;
@@ -225,11 +213,7 @@ extern "C" lbm_status lbm_sweep_noalloc(const lbm_config* cfg, const double* src
         return LBM_ERR_CUDA;
     }
     if (n > 0) {
-        // the records travel as a kernel argument, copied at launch: nothing
-        // waits for the host array
-        k_upload_particles<<<1, MAX_PARTICLES, 0, s>>>(up, n);
-        e = cudaGetLastError();
-        if (e == cudaSuccess) e = launch_regions(L);
+        e = launch_set_particles(L, up, n, a.particles, nullptr, nullptr);
         if (e == cudaSuccess) e = launch_map(L);
     }
     if (sweep_fused(L, 0)) {
