@@ -276,8 +276,19 @@ lbm_status sweep(lbm_handle* h, int sub, bool with_map) {
         h->cur = 1 - h->cur;
         return LBM_OK;
     }
-    // The near-particle cells and the bulk cells are disjoint: the (small,
-    // latency-bound) near sweep runs on a private stream beside k_bulk.
+    // The near-particle cells and the bulk cells are disjoint, so the two sweeps run
+    // at the same time.
+    if (!h->profiling && h->np > 0 && h->bulk_mode < 4 &&
+        L.near_nblk * h->np <= NEAR_BESIDE_BLOCKS) {
+        if (with_map) CK(h, launch_map(L), "geometry map launch");
+        CK(h, launch_near(h->storage, src, dst, L), "near sweep launch");
+        L.beside = 1;
+        CK(h, launch_bulk(h->bulk_mode, src, dst, L), "bulk sweep launch");
+        h->cur = 1 - h->cur;
+        h->pending_pre = 0;
+        return LBM_OK;
+    }
+    // a large near sweep, or one that is timed: on a private stream beside k_bulk
     if (h->np > 0) {
         CK(h, cudaEventRecord(h->ev_fork, h->stream), "fork record");
         CK(h, cudaStreamWaitEvent(h->side, h->ev_fork, 0), "fork wait");

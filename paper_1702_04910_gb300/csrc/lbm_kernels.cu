@@ -41,6 +41,18 @@ __device__ __forceinline__ void step_enter() {
     step_wait();
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+// A bulk sweep launched beside k_near on one stream (launch_bulk with L.beside):
+// k_near has waited for everything before the two, so the bulk blocks need not,
+// and the grid's last block waits for k_near, so that whatever follows the bulk
+// sweep follows both.
+__device__ __forceinline__ void beside_enter(int beside) {
+    if (beside) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void beside_leave(int beside) {
+    if (beside && threadIdx.x == 0 && threadIdx.y == 0 && blockIdx.x == gridDim.x - 1 &&
+        blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1)
+        step_wait();
+}
 // A pointer whose loads cannot be moved ahead of step_enter (they may be
 // declared invariant).
 template <typename P>
@@ -733,13 +745,10 @@ __global__ void __launch_bounds__(BulkShape<T, C>::threads, BulkShape<T, C>::blo
     k_bulk(const T* __restrict__ src, T* __restrict__ dst, Geom g, Coll<C> k,
            const DevParticle* __restrict__ parts, int np, int all_tiles, int* __restrict__ status,
            int beside) {
+    beside_enter(beside);
     bulk_tile<T, C, NOSTREAM, CPT>(src, dst, g, k, parts, np, all_tiles, blockIdx.x, blockIdx.y,
                                    blockIdx.z, threadIdx.x, threadIdx.y, status);
-    // launched beside k_near (which has waited for everything before the two):
-    // the grid completes only after k_near, for the kernels that follow both
-    if (beside && threadIdx.x == 0 && threadIdx.y == 0 && blockIdx.x == gridDim.x - 1 &&
-        blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1)
-        step_wait();
+    beside_leave(beside);
 }
 
 // ---------------------------------------------------------------------------

@@ -25,7 +25,7 @@ struct Launch {
     int* status;
     int nostream;             // 1: stored buffer holds pre-collision f (no stream)
     int all_tiles;            // bulk kernel: process every tile (no coupling)
-    int beside;               // FP64 bulk sweep right after launch_near on the same stream: runs beside it
+    int beside;               // bulk sweep right after launch_near on the same stream: runs beside it
     long long near_nblk;      // near-kernel blocks per particle
     int refill_side;          // refill box: cube side in cells
     unsigned short* map;      // per-step geometry map (see k_map)
@@ -310,6 +310,13 @@ cudaError_t launch_near(int storage, const void* src, void* dst, const Launch& L
 // PSM 64^3 684 / 637, 80^3 793 / 936; FP32 MEM 64^3 1512 / 1257, 80^3 1745 / 1491.
 constexpr long long SWEEP_FUSED_CELLS = 1 << 18;
 bool sweep_fused(const Launch& L, int bulk_mode);
+// FP64 and FP32 near sweeps of up to this many blocks (8 to an SM) go ahead of the
+// bulk sweep on its stream (L.beside); larger ones would hold it up and keep a
+// stream of their own.  us per pass, two streams / one: coarse FP32 features, 10
+// steps 1065 / 1020; 96 x 96 x 288 frame 4009 / 3938; 128 x 128 x 512 FP32 3859 /
+// 3820.  16 bits: no gain, and the flag alone cost k_bulk_pair 4 % (5559 / 5825 us
+// for 192 x 192 x 768 BF16).
+constexpr long long NEAR_BESIDE_BLOCKS = 152 * 8;
 cudaError_t launch_sweep(int storage, const void* src, void* dst, const Launch& L);
 // charge_part != nullptr: also the re-mapping momentum charge partials,
 // refill_blocks(L.refill_side) blocks x 6 doubles per particle (see k_refill)
