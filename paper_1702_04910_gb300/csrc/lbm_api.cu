@@ -262,8 +262,7 @@ lbm_status after_pre_state(lbm_handle* h) {
 }
 
 // with_map: first sweep of a coupled step; the geometry map of the step's
-// particle state is built on the side stream ahead of the near sweep (k_bulk
-// does not read it, so it hides under the bulk sweep).
+// particle state is built ahead of the near sweep (the bulk cells do not read it).
 lbm_status sweep(lbm_handle* h, int sub, bool with_map) {
     Launch L = base_launch(h);
     L.nostream = h->pending_pre;
@@ -318,7 +317,7 @@ lbm_status step_once(lbm_handle* h) {
     const int coupled = h->np > 0 && h->kind != 0;
     const int nsub = h->kind != 0 ? h->subcycles : 1;
     // the geometry of the current particle state, shared by the step's
-    // sweeps, is built by the first sweep (side stream)
+    // sweeps, is built by the first sweep
     for (int s = 0; s < nsub; ++s)
         if ((st = sweep(h, s, coupled && s == 0)) != LBM_OK) return st;
     if (!coupled) return LBM_OK;

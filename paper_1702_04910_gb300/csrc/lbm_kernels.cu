@@ -22,6 +22,7 @@
 // the global timer around a launch for device-side timing.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <type_traits>
 #include <utility>
 
@@ -846,7 +847,7 @@ struct PullPair<T, NQ> {
 // cells per row are 96 threads; as two blocks of 64, a quarter of them idle,
 // the BF16 sweep of 192 x 192 x 768 cells took 473 us, 0.67 of HBM, and takes
 // 376 us, 0.85).  One row of 128 cells per 64-thread block: the near-particle sweep runs
-// beside this kernel and each of its blocks holds 7.7k (MEM) to 11.5k (PSM)
+// beside this kernel and each of its one-warp blocks holds 3.4k (MEM) to 6.2k (PSM)
 // registers; with small bulk blocks an SM that hosts near blocks gives up
 // only as many bulk warps as their registers need (measured in the 128 x 128
 // x 512 step, FP16: 0.70 of HBM with 64 x 4, 0.745 with 64 x 2, 0.76 with
@@ -2097,6 +2098,11 @@ __global__ void __launch_bounds__(NEAR_THREADS)
 // Threads of a k_batch_bulk block and its resident blocks per SM; a work item
 // is 256 cells, so each thread takes BATCH_ITEM / BATCH_THREADS of them.
 constexpr int BATCH_ITEM = 256, BATCH_THREADS = 128, BATCH_BLOCKS = 5;
+// A block takes up to 4 items in a row: finding the item's case and staging its
+// record is a chain of dependent loads ahead of its PDFs (12 cases of D = 8..16, 3
+// steps: 3375 us with one item per block, 3327 with four).  One per block while
+// there are fewer than six waves of 760 blocks.
+constexpr long long BATCH_CHUNK_ITEMS = 4560;
 
 // Cell (x, y, z) of an item's thread slot t: false beyond the lattice.  Plane
 // segments (layout 1) are 256 consecutive cells of an xy plane, so domains
@@ -2128,29 +2134,36 @@ __device__ __forceinline__ bool batch_cell(const Geom& g, int layout, long long 
 // constants from global memory, 256 threads, 1 KB of spills 4.10 ms; staged,
 // 128 threads, 3.87 ms; the FP64 form 10.08 ms).
 __global__ void __launch_bounds__(BATCH_THREADS, BATCH_BLOCKS)
-    k_batch_bulk(BatchCase* __restrict__ cases, BatchList l, long long total,
+    k_batch_bulk(BatchCase* __restrict__ cases, BatchList l, long long total, int chunk,
                  int* __restrict__ status) {
     __shared__ BatchCase B;
     __shared__ int reg[12];
-    int held = -1;
-    for (long long t = blockIdx.x; t < total; t += gridDim.x) {
-        const int i = find_item(l.base, l.n, t);
-        const int c = l.list[i];
-        if (c != held) {
+    long long lo = 0, hi = 0;  // items of the staged case
+    long long t = (long long)blockIdx.x * chunk;
+    for (int left = chunk; t < total; ++t) {
+        if (left == 0) {  // the next chunk of a persistent block
+            t += ((long long)gridDim.x - 1) * chunk;
+            if (t >= total) break;
+            left = chunk;
+        }
+        --left;
+        if (t < lo || t >= hi) {
+            const int i = find_item(l.base, l.n, t);
+            lo = l.base[i];
+            hi = l.base[i + 1];
             __syncthreads();
-            const BatchCase* G = cases + c;
+            const BatchCase* G = cases + l.list[i];
             for (int k = threadIdx.x; k < (int)(sizeof(BatchCase) / 8); k += BATCH_THREADS)
                 reinterpret_cast<long long*>(&B)[k] = reinterpret_cast<const long long*>(G)[k];
             if (threadIdx.x < 12) reg[threadIdx.x] = G->part->reg[threadIdx.x];
             __syncthreads();
-            held = c;
         }
         const double* src = B.buf[B.cur];
         double* dst = B.buf[1 - B.cur];
         bool bad = false;
         for (int s = threadIdx.x; s < BATCH_ITEM; s += BATCH_THREADS) {
             int x, y, z;
-            if (!batch_cell(B.g, B.layout, t - l.base[i], s, x, y, z)) continue;
+            if (!batch_cell(B.g, B.layout, t - lo, s, x, y, z)) continue;
             if (cell_in_reg(B.g, reg, x, y, z)) continue;  // k_batch_near's cell
             const long long idx = lin(B.g, x, y, z);
             double f[NQ];
@@ -2222,8 +2235,8 @@ __global__ void __launch_bounds__(192) k_batch_charge_total(BatchCase* __restric
 // launchers
 namespace {
 // Launch with one common split of the SM's 256 KB between L1 and shared memory.
-// The near sweep needs up to 24 KB of shared memory per block and runs beside
-// the bulk sweep, which needs none.  Left to the default, a bulk block puts its
+// The near sweep needs 9 KB of shared memory per warp (MEM) and runs beside the
+// bulk sweep, which needs none.  Left to the default, a bulk block puts its
 // SM in the all-L1 split, and near blocks cannot start there until the SM has
 // drained.  Measured (us per pass, default / 25 / 50 / 100 % of the largest
 // shared-memory size): 24 x 24 x 40 cells FP64, 20 steps 3210 / 2340 / 2330 /
@@ -2541,8 +2554,10 @@ cudaError_t launch_batch_near(BatchCase* cases, BatchList l, long long total, in
 cudaError_t launch_batch_bulk(BatchCase* cases, BatchList l, long long total, int grid,
                               int* status, cudaStream_t s) {
     if (l.n == 0 || total == 0) return cudaSuccess;
-    const unsigned gsz = (unsigned)(grid <= 0 || total < grid ? total : grid);
-    k_batch_bulk<<<gsz, BATCH_THREADS, 0, s>>>(cases, l, total, status);
+    const int chunk = (int)std::min<long long>(4, std::max<long long>(1, total / BATCH_CHUNK_ITEMS));
+    const long long chunks = (total + chunk - 1) / chunk;
+    const unsigned gsz = (unsigned)(grid <= 0 || chunks < grid ? chunks : grid);
+    k_batch_bulk<<<gsz, BATCH_THREADS, 0, s>>>(cases, l, total, chunk, status);
     return cudaGetLastError();
 }
 cudaError_t launch_batch_swap(BatchCase* cases, BatchList l, cudaStream_t s) {
