@@ -32,19 +32,12 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 METRIC = "MLUPS and % of HBM roofline, coupled D3Q19 step; force/velocity error vs FP64"
-# k_bulk with FP64 arithmetic is bound by the FP64 pipe (2 FP64 lane-operations
-# per SM per cycle on GB300, ncu peak_sustained): its roofline counts FP64
-# thread-instructions per cell update, measured by ncu on the 128x128x256
-# settling case (DADD + DFMA + DMUL per cell the kernel updates), and the DRAM
-# bytes per cell update of the same capture (set to None whenever the kernel
-# changes).
-K_BULK_F64_DP_INST_PER_CELL = 124.0
-K_BULK_F64_DRAM_BYTES_PER_CELL = 292.6
-# FP64 operations per cell update as written in the collision (hand count:
-# moments 39 -- 18 for rho, 21 for j --, equilibrium base 8, nine pair
-# updates 87); the compiler contracts some of them into fused multiply-adds
-# (124 issued, above)
-K_BULK_F64_DP_OPS_WRITTEN = 134
+# k_bulk on FP64 PDFs collides in 64-bit fixed point on the integer pipes and is
+# bound by HBM; the FP64 pipe (2 lane-operations per SM per cycle on GB300) only
+# converts the 19 results back.  DRAM bytes per cell update of an ncu capture:
+# None whenever the kernel has changed since.
+K_BULK_F64_DP_INST_PER_CELL = 19.0
+K_BULK_F64_DRAM_BYTES_PER_CELL = None
 FP64_LANE_OPS_PER_SM_CLK = 2
 COUPLINGS = ("PSM_M1B1", "PSM_M2B2", "MEM_BB", "MEM_CLI", "MEM_MR")
 FRAME_COUPLINGS = ("MEM_BB", "MEM_CLI", "MEM_MR", "PSM_M1B1", "PSM_M2B2", "PSM_M3B2")
@@ -653,8 +646,8 @@ def run_ours(args):
         variants[f"learned_{args.learned}"] = run_learned(args, stream)
 
     # dominant kernel's roofline against the metric's own bound, HBM bytes per
-    # cell update; the kernel's actual limiter, the FP64 pipe, beside it with
-    # the DFMA rate measured on this device
+    # cell update; the FP64 pipe's share beside it, with the DFMA rate measured
+    # on this device
     from paper_1702_04910_gb300.binding import lbm_measure_fp64_rate
     props = torch.cuda.get_device_properties(local)
     sm_max_mhz = clocks.get("sm_max_mhz") or 2070.0
@@ -673,15 +666,13 @@ def run_ours(args):
         "peak_source": peak_kind, "traffic": traffic,
         "per_unit": f"{bytes_per_cell} B per cell update (19 FP64 values read, 19 written)",
         "cells_per_launch": bulk_cells, "avg_launch_ms": bulk_ms / bulk_n,
-        "limiter": "FP64 pipe (see alu): the kernel issues FP64 instructions at "
-                   f"{fp64_achieved / fp64_peak:.2f} of the measured DFMA rate",
+        "limiter": "HBM; the FP64 pipe (see alu) converts the results of the fixed-point collision",
         "alu": {"achieved": fp64_achieved, "peak": fp64_peak, "unit": "T FP64 inst/s",
                 "frac": fp64_achieved / fp64_peak, "peak_source": fp64_src,
                 "peak_nominal": fp64_nominal,
                 "peak_nominal_source": f"{FP64_LANE_OPS_PER_SM_CLK} FP64 lane-ops/SM/cycle x "
                                        f"{props.multi_processor_count} SMs x {sm_max_mhz:.0f} MHz",
-                "per_unit": f"{K_BULK_F64_DP_INST_PER_CELL} FP64 instructions per cell update "
-                            f"issued (ncu); {K_BULK_F64_DP_OPS_WRITTEN} written in the source"},
+                "per_unit": f"{K_BULK_F64_DP_INST_PER_CELL} FP64-pipe conversions per cell update"},
     }
 
     cpu = None
@@ -701,7 +692,9 @@ def run_ours(args):
                        # MEM's two sweeps counted once): value x couplings / sweeps
                        "mlups_per_global_step": value * len(args.couplings) / sweeps_per_step,
                        "collision": "TRT (Lambda=3/16)",
-                       "precision": "FP64 PDFs and collision; FP64 forces and rigid-body update",
+                       "precision": "FP64 PDFs; 64-bit fixed-point collision of cells away from "
+                                    "particles (closer to exact than FP64), FP64 elsewhere; FP64 forces "
+                                    "and rigid-body update",
                        "l2": "inputs larger than L2 (2.55 GB of PDFs per simulation)",
                        "replicas_per_rank": 1},
             "roofline": roofline,

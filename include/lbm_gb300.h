@@ -277,8 +277,9 @@ enum {
     LBM_STATUS_FLUID = 32            /* a fluid cell's density became non-finite or <= 0 */
 };
 
-/* Capacity, in doubles, of the fixed force-partial scratch that
- * lbm_sweep_noalloc uses: 524288 doubles = 4 MiB per GPU. */
+/* Largest request, in doubles of force partials counted as below, that
+ * lbm_sweep_noalloc's fixed scratch takes (it holds twice as many, 8 MiB per
+ * GPU: the sweep's own blocks are half the size of the ones counted). */
 #define LBM_NOALLOC_MAX_PARTIAL_DOUBLES 524288
 
 /* One coupled LBM sweep that allocates no memory.  The paper has no
@@ -315,7 +316,7 @@ enum {
  *                    argument.
  *   err, err_len     optional buffer for a message on failure.
  * Scratch: the force partials of the near-particle blocks live in a fixed
- * device array of LBM_NOALLOC_MAX_PARTIAL_DOUBLES doubles, next to a
+ * device array for LBM_NOALLOC_MAX_PARTIAL_DOUBLES doubles, next to a
  * geometry map of 1,048,576 16-bit entries (2 MiB), 32 particle records and
  * a status word; every GPU using the library holds them until exit.  A call
  * needs max(n,1)^2 * B * 6 doubles of partials, where B = ceil(E_x/32) *
