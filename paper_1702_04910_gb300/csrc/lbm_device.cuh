@@ -157,18 +157,21 @@ __device__ __forceinline__ bool point_inside(const Geom& g, const DevParticle& P
 // r^2 by more than 4e-6 (r^2 + r + 1) is decided in FP32, the few others by
 // the FP64 form: the same decisions everywhere.
 
-// Minimum-image offset along axis a of the point i + add from P's centre.
-// (A wrapped offset that the FP64 form would leave, or the reverse, has a
-// length of half the domain, beyond any sphere.)
+// Minimum-image offset along axis a of the point i + add from P's centre.  The
+// image is chosen on the integers, before FP32: i - xi is exact at any length of
+// the domain, where an FP32 offset of a domain's length keeps only 2^-24 of it
+// (3e-5 at 768 cells, beyond the margin of a small sphere).  An image that
+// the FP64 form would not choose has a length of half the domain but a cell,
+// which is beyond R + 3/2 of any sphere (an axis holds at least D + 6 cells).
 __device__ __forceinline__ float offset_f(const DevParticle& P, int a, int i, float add, int n,
                                           bool periodic) {
-    float d = (float)(i - P.xi[a]) + (add - P.xf[a]);
+    int d = i - P.xi[a];
     if (periodic) {
-        const float L = (float)n, h = 0.5f * L;
-        if (d > h) d -= L;
-        else if (d < -h) d += L;
+        const int h = n >> 1;
+        if (d > h) d -= n;
+        else if (d < -h) d += n;
     }
-    return d;
+    return (float)d + (add - P.xf[a]);
 }
 __device__ __forceinline__ float margin_f(float r) { return 4e-6f * (r * r + r + 1.0f); }
 // 1: inside or on the sphere of radius r, 0: outside, -1: too close to tell
