@@ -45,6 +45,7 @@ struct lbm_handle {
     cudaStream_t side;           // private stream: near-particle sweep runs beside k_bulk
     cudaEvent_t ev_fork, ev_join;
     int device;
+    int sms;             // multiprocessors of the device
     Geom g;
     int storage;       // 0 FP64, 1 FP32 (PDF storage / arithmetic of every kernel but k_bulk)
     int bulk_mode;     // k_bulk arithmetic: 0 FP64, 1 FP32, 2 float-float, 3 fixed point (FP64 PDFs)
@@ -66,7 +67,7 @@ struct lbm_handle {
     size_t partial_cap;  // doubles allocated in d_partials
     unsigned short* d_map;  // per-step geometry map [np][region box]
     size_t map_cap;         // entries allocated in d_map
-    int* d_status;       // in front of d_force, so that both are read in one copy
+    int* d_status;       // status, gate (see gate_open), then d_force: read in one copy
     double* h_stage;     // pinned: status word + np*6 forces
     size_t dev_bytes;
     Coll<double> kd;
@@ -137,6 +138,8 @@ void prof_end(lbm_handle* h, int i, cudaStream_t s = nullptr) {
     if (i >= 0) cudaEventRecord(h->events[i].b, s ? s : h->stream);
 }
 
+int* gate_of(lbm_handle* h) { return h->d_status + 1; }
+
 Launch base_launch(lbm_handle* h) {
     Launch L{};
     L.g = h->g;
@@ -156,7 +159,8 @@ Launch base_launch(lbm_handle* h) {
     L.status = h->d_status;
     L.nostream = 0;
     L.all_tiles = 0;
-    L.beside = 0;
+    L.gate = nullptr;
+    L.gate_key = 0;
     L.block = dim3(h->g.tx, h->g.ty, 1);
     L.stream = h->stream;
     L.near_nblk = near_blocks(h->g, h->maxd);
@@ -277,17 +281,17 @@ lbm_status sweep(lbm_handle* h, int sub, bool with_map) {
     }
     // The near-particle cells and the bulk cells are disjoint, so the two sweeps run
     // at the same time.
-    if (!h->profiling && h->np > 0 && h->bulk_mode < 4 &&
-        L.near_nblk * h->np <= NEAR_BESIDE_BLOCKS) {
+    if (!h->profiling && sweep_beside(L, h->bulk_mode, h->sms)) {
         if (with_map) CK(h, launch_map(L), "geometry map launch");
+        L.gate = gate_of(h);
+        L.gate_key = sub + 1;
         CK(h, launch_near(h->storage, src, dst, L), "near sweep launch");
-        L.beside = 1;
         CK(h, launch_bulk(h->bulk_mode, src, dst, L), "bulk sweep launch");
         h->cur = 1 - h->cur;
         h->pending_pre = 0;
         return LBM_OK;
     }
-    // a large near sweep, or one that is timed: on a private stream beside k_bulk
+    // the (small, latency-bound) near sweep on a private stream beside k_bulk
     if (h->np > 0) {
         CK(h, cudaEventRecord(h->ev_fork, h->stream), "fork record");
         CK(h, cudaStreamWaitEvent(h->side, h->ev_fork, 0), "fork wait");
@@ -322,6 +326,7 @@ lbm_status step_once(lbm_handle* h) {
         if ((st = sweep(h, s, coupled && s == 0)) != LBM_OK) return st;
     if (!coupled) return LBM_OK;
     Launch L = base_launch(h);
+    L.gate = gate_of(h);  // closed by the force total
     const double* charge = h->remap_charge ? h->d_charge : nullptr;
     const double* gr = h->cfg.gravity;
     int pi;
@@ -436,6 +441,8 @@ lbm_status lbm_create(const lbm_config* cfg, void* stream, lbm_handle** out) {
     if (h->cfg.subsample == 0) h->cfg.subsample = 4;
     h->stream = (cudaStream_t)stream;
     cudaGetDevice(&h->device);
+    h->sms = 0;
+    cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
     {
         // the near sweep's stream has the highest priority: its few long-lived
         // blocks are placed as soon as k_bulk blocks retire, instead of
@@ -492,7 +499,7 @@ lbm_status lbm_create(const lbm_config* cfg, void* stream, lbm_handle** out) {
     }
     h->d_force = reinterpret_cast<double*>(h->d_status) + 1;
     h->dev_bytes = 2 * bytes + sizeof(double) * (1 + 6 * MAX_PARTICLES);
-    cudaMemsetAsync(h->d_status, 0, sizeof(int), h->stream);
+    cudaMemsetAsync(h->d_status, 0, 2 * sizeof(int), h->stream);
     lbm_status st = alloc_particles(h, 0);
     if (st == LBM_OK) st = ensure_partials(h);
     if (st == LBM_OK) {

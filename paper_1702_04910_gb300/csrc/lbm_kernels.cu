@@ -38,21 +38,47 @@ namespace lbmgpu {
 // be launched in turn.  Every kernel launched that way calls this before it
 // touches memory, so a kernel's completion implies that of all before it.
 __device__ __forceinline__ void step_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void step_enter() {
-    step_wait();
+__device__ __forceinline__ void step_trigger() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
-// A bulk sweep launched beside k_near on one stream (launch_bulk with L.beside):
-// k_near has waited for everything before the two, so the bulk blocks need not,
-// and the grid's last block waits for k_near, so that whatever follows the bulk
-// sweep follows both.
-__device__ __forceinline__ void beside_enter(int beside) {
-    if (beside) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+__device__ __forceinline__ void step_enter() {
+    step_wait();
+    step_trigger();
 }
-__device__ __forceinline__ void beside_leave(int beside) {
-    if (beside && threadIdx.x == 0 && threadIdx.y == 0 && blockIdx.x == gridDim.x - 1 &&
+// A bulk sweep beside k_near on one stream (launch_near, then launch_bulk, with
+// L.gate).  k_bulk is launched once every block of k_near has begun, and has to
+// see what the kernels before k_near wrote.  k_near's wait gives that view to
+// k_near alone, so it is handed on by memory order: block 0 of k_near stores the
+// key to the gate with release after its wait, and a block of k_bulk loads it with
+// acquire before anything else.  That store precedes the trigger that lets k_bulk
+// start, so the load finds it at once; a block that does not after GATE_TRIES
+// loads reports ST_BOUNDS and leaves its cells.  The grid's last block waits for
+// k_near, so that whatever follows the bulk sweep follows both; the force total
+// closes the gate again.
+constexpr int GATE_TRIES = 1 << 16;
+__device__ __forceinline__ void gate_open(int* gate, int key) {
+    if (gate && threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0)
+        asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(gate), "r"(key) : "memory");
+}
+__device__ __forceinline__ bool gate_pass(const int* gate, int key) {
+    if (!gate) return true;
+    step_trigger();
+    int seen = 1;
+    if (threadIdx.x == 0 && threadIdx.y == 0) {
+        int v = 0;
+        for (int i = 0; i < GATE_TRIES && v != key; ++i)
+            asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(gate) : "memory");
+        seen = v == key;
+    }
+    return __syncthreads_and(seen);
+}
+__device__ __forceinline__ void gate_leave(const int* gate) {
+    if (gate && threadIdx.x == 0 && threadIdx.y == 0 && blockIdx.x == gridDim.x - 1 &&
         blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1)
         step_wait();
+}
+__device__ __forceinline__ void gate_close(int* gate) {
+    if (gate && blockIdx.x == 0 && threadIdx.x == 0) *gate = 0;
 }
 // A pointer whose loads cannot be moved ahead of step_enter (they may be
 // declared invariant).
@@ -741,15 +767,28 @@ __device__ __forceinline__ void bulk_tile(const T* __restrict__ src, T* __restri
     if (bad) atomicOr(status, ST_FLUID);
 }
 
-template <typename T, typename C, bool NOSTREAM, int CPT>
+// GATE: the form that runs beside k_near (gate_pass); the others are launched
+// plainly and carry none of its code but, in FP32, gate_leave (null gate, no
+// effect): ptxas makes a faster kernel with a branch at its end (128 x 128 x 512 MEM
+// with charge, 8 steps 4082 us without, 3890 with; FP64 MEM MR, 4 steps 4265 without,
+// 4331 with).
+template <typename T, typename C, bool NOSTREAM, int CPT, bool GATE>
 __global__ void __launch_bounds__(BulkShape<T, C>::threads, BulkShape<T, C>::blocks)
     k_bulk(const T* __restrict__ src, T* __restrict__ dst, Geom g, Coll<C> k,
            const DevParticle* __restrict__ parts, int np, int all_tiles, int* __restrict__ status,
-           int beside) {
-    beside_enter(beside);
+           const int* gate, int key) {
+    if constexpr (GATE) {
+        if (!gate_pass(gate, key)) {
+            if (threadIdx.x == 0 && threadIdx.y == 0) atomicOr(status, ST_BOUNDS);
+            gate_leave(gate);
+            return;
+        }
+        src = entered(src);
+        parts = entered(parts);
+    }
     bulk_tile<T, C, NOSTREAM, CPT>(src, dst, g, k, parts, np, all_tiles, blockIdx.x, blockIdx.y,
                                    blockIdx.z, threadIdx.x, threadIdx.y, status);
-    beside_leave(beside);
+    if constexpr (GATE || sizeof(T) == 4) gate_leave(gate);
 }
 
 // ---------------------------------------------------------------------------
@@ -1236,10 +1275,12 @@ template <typename T, typename C, int KIND, bool NOSTREAM>
 __global__ void __launch_bounds__(NEAR_THREADS)
     k_near(const T* __restrict__ src, T* __restrict__ dst, Geom g, Coll<C> k, Coupl cp,
            const DevParticle* __restrict__ parts, GeoMap gm, double* __restrict__ partials,
-           int* __restrict__ status) {
+           int* __restrict__ status, int* gate, int key) {
     extern __shared__ double sp_words[];
     __shared__ typename std::conditional<KIND == 2, LinkWarp, char>::type lw;
-    step_enter();
+    step_wait();
+    gate_open(gate, key);
+    step_trigger();
     parts = entered(parts);
     src = entered(src);
     gm.map = entered(gm.map);
@@ -1384,9 +1425,10 @@ __device__ __forceinline__ void finalize_block(int np, long long nblk,
 
 __global__ void __launch_bounds__(FIN_THREADS)
     k_finalize(int np, long long nblk, const double* __restrict__ partials, int nsub,
-               double* __restrict__ out, const double* __restrict__ charge) {
+               double* __restrict__ out, const double* __restrict__ charge, int* gate) {
     __shared__ double red[FIN_THREADS];
     step_enter();
+    gate_close(gate);
     finalize_block(np, nblk, entered(partials), nsub, out, blockIdx.x, red,
                    charge ? entered(charge) : nullptr);
 }
@@ -1473,9 +1515,10 @@ __global__ void __launch_bounds__(FIN_THREADS)
     k_finalize_rigid(Geom g, int np, long long nblk, const double* __restrict__ partials, int nsub,
                      double* force, const double* __restrict__ charge, DevParticle* parts,
                      DevParticle* prev, double rho0, double gx, double gy, double gz, double dt,
-                     int wall_contact, int* status) {
+                     int wall_contact, int* status, int* gate) {
     __shared__ double red[FIN_THREADS];
     step_enter();
+    gate_close(gate);
     parts = entered(parts);
     const int p = blockIdx.x;
     finalize_block(np, nblk, entered(partials), nsub, force, p, red,
@@ -2290,12 +2333,15 @@ template <typename T, typename C, int CPT>
 cudaError_t bulk_cpt(const void* src, void* dst, const Launch& L) {
     dim3 grid(L.g.ntx, L.g.nty, L.g.ntz);
     const auto& k = coll_of<typename std::conditional<(sizeof(T) < 4), C, T>::type, C>(L);
-    const bool beside = L.beside != 0;
-    if (L.nostream)
-        return launch_with(beside, 0, k_bulk<T, C, true, CPT>, grid, L.block, L.stream, (const T*)src,
-                           (T*)dst, L.g, k, L.parts, L.cp.np, L.all_tiles, L.status, L.beside);
-    return launch_with(beside, 0, k_bulk<T, C, false, CPT>, grid, L.block, L.stream, (const T*)src,
-                       (T*)dst, L.g, k, L.parts, L.cp.np, L.all_tiles, L.status, L.beside);
+    const auto go = [&](auto kernel) {
+        return launch_with(L.gate != nullptr, 0, kernel, grid, L.block, L.stream, (const T*)src, (T*)dst,
+                           L.g, k, L.parts, L.cp.np, L.all_tiles, L.status, (const int*)L.gate,
+                           L.gate_key);
+    };
+    if constexpr (sizeof(T) >= 4 && !std::is_same<C, dfloat>::value)
+        if (L.gate)
+            return L.nostream ? go(k_bulk<T, C, true, CPT, true>) : go(k_bulk<T, C, false, CPT, true>);
+    return L.nostream ? go(k_bulk<T, C, true, CPT, false>) : go(k_bulk<T, C, false, CPT, false>);
 }
 
 // FP64-state sweeps are arithmetic bound and use one cell per thread; the
@@ -2343,9 +2389,9 @@ cudaError_t near_kind(const void* src, void* dst, const Launch& L) {
     constexpr bool early = sizeof(T) > 2;
     if (L.nostream)
         return launch_with(early, smem, k_near<T, C, KIND, true>, grid, block, L.stream, (const T*)src,
-                           (T*)dst, L.g, k, L.cp, L.parts, gm, L.partials, L.status);
+                           (T*)dst, L.g, k, L.cp, L.parts, gm, L.partials, L.status, L.gate, L.gate_key);
     return launch_with(early, smem, k_near<T, C, KIND, false>, grid, block, L.stream, (const T*)src,
-                       (T*)dst, L.g, k, L.cp, L.parts, gm, L.partials, L.status);
+                       (T*)dst, L.g, k, L.cp, L.parts, gm, L.partials, L.status, L.gate, L.gate_key);
 }
 
 template <typename T, int KIND>
@@ -2439,6 +2485,12 @@ bool sweep_fused(const Launch& L, int bulk_mode) {
     return L.cp.np > 0 && (L.cp.kind == 1 || L.cp.kind == 2) && !L.nostream &&
            (bulk_mode == 0 || bulk_mode == 1 || bulk_mode == 3) && L.g.n <= SWEEP_FUSED_CELLS;
 }
+bool sweep_beside(const Launch& L, int bulk_mode, int sms) {
+    const long long blocks = (long long)L.g.ntx * L.g.nty * L.g.ntz;
+    const int waves = L.cp.kind == 2 ? 6 : 4;
+    return L.cp.np > 0 && L.cp.kind != 0 && bulk_mode == 1 && L.near_nblk * L.cp.np <= 8LL * sms &&
+           blocks <= (long long)waves * BulkShape<float, float>::blocks * sms;
+}
 cudaError_t launch_sweep(int storage, const void* src, void* dst, const Launch& L) {
     if (storage == 1)
         return L.cp.kind == 1 ? sweep_kind<float, 1>(src, dst, L) : sweep_kind<float, 2>(src, dst, L);
@@ -2510,7 +2562,7 @@ cudaError_t launch_map(const Launch& L) {
 cudaError_t launch_finalize(const Launch& L, int nsub, double* force_out, const double* charge) {
     if (L.cp.np <= 0) return cudaSuccess;
     return launch_after(k_finalize, L.cp.np, FIN_THREADS, L.stream, L.cp.np, L.near_nblk, L.partials, nsub,
-                  force_out, charge);
+                  force_out, charge, L.gate);
 }
 cudaError_t launch_rigid_body(const Launch& L, const double* force, double gx, double gy,
                               double gz, double dt, int wall_contact) {
@@ -2523,7 +2575,7 @@ cudaError_t launch_finalize_rigid(const Launch& L, int nsub, double* force, cons
     if (L.cp.np <= 0) return cudaSuccess;
     return launch_after(k_finalize_rigid, L.cp.np, FIN_THREADS, L.stream, L.g, L.cp.np,
                   L.near_nblk, L.partials, nsub, force, charge, L.parts, L.parts_prev,
-                  L.kd.rho0, gx, gy, gz, (double)nsub, wall_contact, L.status);
+                  L.kd.rho0, gx, gy, gz, (double)nsub, wall_contact, L.status, L.gate);
 }
 cudaError_t launch_set_particles(const Launch& L, const ParticleUpload& up, int n, DevParticle* parts,
                                  DevParticle* prev, DevParticle* old) {

@@ -25,7 +25,8 @@ struct Launch {
     int* status;
     int nostream;             // 1: stored buffer holds pre-collision f (no stream)
     int all_tiles;            // bulk kernel: process every tile (no coupling)
-    int beside;               // bulk sweep right after launch_near on the same stream: runs beside it
+    int* gate;                // not null: launch_near and, right after it on the same stream,
+    int gate_key;             //   launch_bulk run beside one another (see gate_open)
     long long near_nblk;      // near-kernel blocks per particle
     int refill_side;          // refill box: cube side in cells
     unsigned short* map;      // per-step geometry map (see k_map)
@@ -310,13 +311,16 @@ cudaError_t launch_near(int storage, const void* src, void* dst, const Launch& L
 // PSM 64^3 684 / 637, 80^3 793 / 936; FP32 MEM 64^3 1512 / 1257, 80^3 1745 / 1491.
 constexpr long long SWEEP_FUSED_CELLS = 1 << 18;
 bool sweep_fused(const Launch& L, int bulk_mode);
-// FP64 and FP32 near sweeps of up to this many blocks (8 to an SM) go ahead of the
-// bulk sweep on its stream (L.beside); larger ones would hold it up and keep a
-// stream of their own.  us per pass, two streams / one: coarse FP32 features, 10
-// steps 1065 / 1020; 96 x 96 x 288 frame 4009 / 3938; 128 x 128 x 512 FP32 3859 /
-// 3820.  16 bits: no gain, and the flag alone cost k_bulk_pair 4 % (5559 / 5825 us
-// for 192 x 192 x 768 BF16).
-constexpr long long NEAR_BESIDE_BLOCKS = 152 * 8;
+// Whether a handle's near and bulk sweeps run beside one another on one stream
+// (L.gate), in place of a second stream with its fork and join: FP32 lattices whose
+// bulk sweep is up to 4 (PSM) or 6 (MEM, the longer near sweep) waves of blocks, each
+// of which pays for the gate's load.  us for 20 steps, second stream / gate, by
+// waves: PSM 66^3 (2.5) 690 / 634, 80^3 (3.5) 713 / 697, 88^3 (4.2) 771 / 801,
+// 96^3 (5.1) 841 / 921; MEM (two sweeps a step) 66^3 1367 / 1219, 88^3 1600 / 1534, 96^3
+// 1768 / 1676; 64 x 64 x 192 PSM with features (3.4), 10 steps 1077 / 1049.  FP64:
+// 72^3 1156 / 1173, 96^3 1646 / 1755, 128 x 128 x 512 4264 / 4497, so never.
+// Near sweeps of more than 8 blocks to an SM would hold the bulk blocks up.
+bool sweep_beside(const Launch& L, int bulk_mode, int sms);
 cudaError_t launch_sweep(int storage, const void* src, void* dst, const Launch& L);
 // charge_part != nullptr: also the re-mapping momentum charge partials,
 // refill_blocks(L.refill_side) blocks x 6 doubles per particle (see k_refill)

@@ -39,9 +39,17 @@ long long counted_blocks(const Geom& g, double maxd) {
     return (long long)((ext[0] + 31) / 32) * ((ext[1] + 1) / 2) * ext[2];
 }
 static __device__ __align__(256) DevParticle g_particles[MAX_PARTICLES];
-static __device__ __align__(256) int g_status[64];
+static __device__ __align__(256) int g_status[64];  // [0] status, [1] gate (see gate_open)
 constexpr size_t NOALLOC_MAP_ENTRIES = 1 << 20;  // geometry map, 2 MiB
 static __device__ __align__(256) unsigned short g_map[NOALLOC_MAP_ENTRIES];
+
+// Largest lattice whose bulk sweep runs beside the near sweep: there is no second
+// stream here, and beyond this size the gate's load at the head of every bulk
+// block costs more than the overlap gives.  us for one sweep, one after the other
+// / beside: 72^3, one D = 16 sphere 90 / 70; 96^3, four D = 16 117 / 103; 128^3,
+// one D = 24 188 / 173; 128^3, eight D = 24 360 / 358; 128 x 128 x 256 310 / 308;
+// 192^3, four D = 24 601 / 636.
+constexpr long long NOALLOC_BESIDE_CELLS = 1 << 22;
 
 constexpr int MAX_DEVICES = 64;
 struct Addresses {
@@ -220,9 +228,12 @@ extern "C" lbm_status lbm_sweep_noalloc(const lbm_config* cfg, const double* src
         if (e == cudaSuccess) e = launch_sweep(0, src_pdf_dev, dst_pdf_dev, L);
     } else {
         // near sweep first: its blocks are placed, then the bulk sweep runs
-        // beside it
+        // beside it (NOALLOC_BESIDE_CELLS) or follows it
+        if (n > 0 && g.n <= NOALLOC_BESIDE_CELLS) {
+            L.gate = a.status + 1;
+            L.gate_key = 1;
+        }
         if (e == cudaSuccess && n > 0) e = launch_near(0, src_pdf_dev, dst_pdf_dev, L);
-        L.beside = n > 0;
         if (e == cudaSuccess) e = launch_bulk(0, src_pdf_dev, dst_pdf_dev, L);
     }
     if (e == cudaSuccess && n > 0) e = launch_finalize(L, 1, force_torque_dev);
