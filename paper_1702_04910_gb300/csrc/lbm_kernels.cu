@@ -1093,15 +1093,15 @@ struct NearPull<T, C, NQ> {
                                                long long, unsigned, unsigned, C (&)[NQ]) {}
 };
 template <typename T, typename C>
-__device__ __forceinline__ void near_pull(const T* __restrict__ src, const Geom& g,
+__device__ __forceinline__ bool near_pull(const T* __restrict__ src, const Geom& g,
                                           const DevParticle* sp, int np, const GeoMap& gm, int p,
                                           int kx, int ky, int kz, int x, int y, int z,
                                           long long idx, C (&f)[NQ], unsigned& cut, int* status) {
-    f[0] = PdfStore<T>::template load<C>(src + idx, 0);
     if (kx >= gm.ex || ky >= gm.ey || kz >= gm.ez) {  // a box larger than its map: report, no access
         atomicOr(status, ST_BOUNDS);
-        return;
+        return false;  // (the caller stores no cell that was not pulled)
     }
+    f[0] = PdfStore<T>::template load<C>(src + idx, 0);
     const int* R = sp[p].reg;
     const unsigned in = (kx > 0 ? 1u : 0u) | (kx + 1 < min(R[1], gm.ex) ? 2u : 0u) |
                         (ky > 0 ? 4u : 0u) | (ky + 1 < min(R[5], gm.ey) ? 8u : 0u) |
@@ -1116,6 +1116,7 @@ __device__ __forceinline__ void near_pull(const T* __restrict__ src, const Geom&
     for (int q = 1; q < NQ; ++q) solid |= e[q] ? 1u << q : 0u;
     NearPull<T, C, 1>::run(src, g, o, idx, solid, wall, f);
     cut = solid;
+    return true;
 }
 
 // Cell of a lane of near block blk, as offsets in the region R; false beyond it.
@@ -1236,7 +1237,7 @@ __device__ __forceinline__ void near_block(const T* __restrict__ src, T* __restr
             if (clear_of_particles(g, sp, cp.np, x, y, z)) {
                 pull_plain(src, g, x, y, z, idx, f);  // no solid neighbour, no link
             } else {
-                near_pull(src, g, sp, cp.np, gm, p, kx, ky, kz, x, y, z, idx, f, cut, status);
+                fluid = near_pull(src, g, sp, cp.np, gm, p, kx, ky, kz, x, y, z, idx, f, cut, status);
             }
         }
         mem_links_warp(src, g, cp, sp, &gm, x, y, z, idx, cut, f, slots, status, lw, lane);
