@@ -106,14 +106,18 @@ typedef enum { LBM_BGK = 0, LBM_TRT = 1 } lbm_collision;
  *                     for the fixed-point collision by name).
  *   LBM_STORE_F16S    PDFs stored as FP16 shifted populations f_q - w_q, FP32
  *                     collision arithmetic (76 B per cell update).
- *   LBM_STORE_BF16S   the same with BF16 storage. */
+ *   LBM_STORE_BF16S   the same with BF16 storage.
+ *   LBM_STORE_F64_DP  FP64 PDFs, FP64 arithmetic in every cell: the yardstick of
+ *                     the other modes.  About a quarter of LBM_STORE_F64's
+ *                     speed.  Same state layout as LBM_STORE_F64. */
 typedef enum {
     LBM_STORE_F64 = 0,
     LBM_STORE_F32 = 1,
     LBM_STORE_F64_FF = 2,
     LBM_STORE_F64_FX = 3,
     LBM_STORE_F16S = 4,
-    LBM_STORE_BF16S = 5
+    LBM_STORE_BF16S = 5,
+    LBM_STORE_F64_DP = 6
 } lbm_storage;
 
 typedef struct {
@@ -294,7 +298,8 @@ enum {
  * fixed-order force/torque total of that sweep -- but no subcycle average,
  * rigid-body update or MEM refilling, and no handle.
  *   cfg              configuration as for lbm_create; storage must be
- *                    LBM_STORE_F64 (LBM_ERR_UNSUPPORTED otherwise); LBM_MEM_MR
+ *                    LBM_STORE_F64 or LBM_STORE_F64_DP
+ *                    (LBM_ERR_UNSUPPORTED otherwise); LBM_MEM_MR
  *                    is refused as in lbm_create (|Lambda_- - 1/2| < 0.01).
  *   src_pdf_dev      device, 19*N doubles: post-collision PDFs (the layout
  *                    of lbm_get_fields(LBM_FIELD_PDF)); read only.
@@ -368,8 +373,8 @@ enum {
 /* Creates a batch of n_cases (1..4096) cases.
  *   cfgs[c]       configuration of case c (as for lbm_create); coupling must
  *                 be a PSM or MEM variant (LBM_MEM_MR as for lbm_create);
- *                 bc_z 0 or 1; storage must be LBM_STORE_F64 or
- *                 LBM_STORE_F64_FX and the same for every case.
+ *                 bc_z 0 or 1; storage must be LBM_STORE_F64, LBM_STORE_F64_FX
+ *                 or LBM_STORE_F64_DP and the same for every case.
  *   particles[c]  the one sphere of case c (copied).
  *   stream        cudaStream_t or NULL: stream of every batch call.
  * All device memory of the batch is one allocation (PDF buffers, particle

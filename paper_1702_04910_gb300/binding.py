@@ -32,7 +32,7 @@ STATUS_BITS = {"LBM_STATUS_TOO_MANY_OBJECTS": 1, "LBM_STATUS_DOMAIN": 2, "LBM_ST
 COUPLING = {"PSM_M1B1": 0, "PSM_M2B2": 1, "PSM_M3B2": 2, "MEM_BB": 3, "MEM_CLI": 4,
             "MEM_MR": 5, "NONE": 6}
 COLLISION = {"BGK": 0, "TRT": 1}
-STORAGE = {"f64": 0, "f32": 1, "f64ff": 2, "f64fx": 3, "f16s": 4, "bf16s": 5}
+STORAGE = {"f64": 0, "f32": 1, "f64ff": 2, "f64fx": 3, "f16s": 4, "bf16s": 5, "f64dp": 6}
 (FIELD_PDF, FIELD_PDF_PRE, FIELD_RHO, FIELD_U, FIELD_EPS, FIELD_FLAG, FIELD_PDF_F64,
  FIELD_REMAP_CHARGE) = range(8)
 PROFILE_CLASSES = ("bulk", "near", "force_total", "rigid_body", "refill", "other")

@@ -48,7 +48,7 @@ struct lbm_handle {
     int sms;             // multiprocessors of the device
     Geom g;
     int storage;       // 0 FP64, 1 FP32 (PDF storage / arithmetic of every kernel but k_bulk)
-    int bulk_mode;     // k_bulk arithmetic: 0 FP64, 1 FP32, 2 float-float, 3 fixed point (FP64 PDFs)
+    int bulk_mode;     // k_bulk arithmetic: 0 FP64, 1 FP32, 2 float-float (FP64 PDFs), 4 / 5 FP16 / BF16
     size_t esize;      // bytes per stored PDF value
     void* buf[2];
     int cur;           // buffer holding the stored state
@@ -464,7 +464,8 @@ lbm_status lbm_create(const lbm_config* cfg, void* stream, lbm_handle** out) {
                  : cfg->storage == LBM_STORE_BF16S ? 5
                                                    : 0;
     h->esize = h->storage == 0 ? sizeof(double) : (h->storage == 1 ? sizeof(float) : 2);
-    h->bulk_mode = cfg->storage;  // bulk arithmetic: the storage code, or 2 / 3 on FP64 state
+    // bulk arithmetic: the storage code, or 2 (float-float) on FP64 state
+    h->bulk_mode = h->storage == 0 && cfg->storage != LBM_STORE_F64_FF ? 0 : cfg->storage;
     h->kind = is_psm(cfg->coupling) ? 1 : (is_mem(cfg->coupling) ? 2 : 0);
     h->variant = h->kind == 1 ? cfg->coupling - LBM_PSM_M1B1
                               : (h->kind == 2 ? cfg->coupling - LBM_MEM_BB : 0);
@@ -484,7 +485,7 @@ lbm_status lbm_create(const lbm_config* cfg, void* stream, lbm_handle** out) {
 
     const double lp = -1.0 / cfg->tau;
     const double lm = cfg->collision == LBM_TRT ? 1.0 / (cfg->magic / (0.5 + 1.0 / lp) - 0.5) : lp;
-    h->kd = make_coll<double>(lp, lm, cfg->rho0, cfg->force_density);
+    h->kd = make_coll_f64(cfg->storage, lp, lm, cfg->rho0, cfg->force_density);
     h->kf = make_coll<float>(lp, lm, cfg->rho0, cfg->force_density);
     h->kff = make_coll<dfloat>(lp, lm, cfg->rho0, cfg->force_density);
 

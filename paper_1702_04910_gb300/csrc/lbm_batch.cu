@@ -344,7 +344,7 @@ lbm_status make_case(lbm_batch* b, int c, const lbm_config& cfg, const lbm_parti
     k.cp.tau = cfg.tau;
     k.cp.rho0 = cfg.rho0;
     k.cp.mr_cpc = cfg.coupling == LBM_MEM_MR ? mr_correction_scale(cfg) : 0.0;
-    k.kd = make_coll<double>(lp, lm, cfg.rho0, cfg.force_density);
+    k.kd = make_coll_f64(cfg.storage, lp, lm, cfg.rho0, cfg.force_density);
     region_extent(g, p.diameter, k.map_ext);
     k.nblk = near_blocks(g, p.diameter);
     k.refill_side = (int)std::ceil(p.diameter) + 4;
@@ -419,9 +419,9 @@ lbm_status lbm_batch_create(int n_cases, const lbm_config* cfgs, const lbm_parti
         return LBM_ERR_ARG;
     }
     const int storage = cfgs[0].storage;
-    if (storage != LBM_STORE_F64 && storage != LBM_STORE_F64_FX) {
+    if (storage != LBM_STORE_F64 && storage != LBM_STORE_F64_FX && storage != LBM_STORE_F64_DP) {
         std::snprintf(g_create_err, sizeof(g_create_err),
-                      "storage must be LBM_STORE_F64 or LBM_STORE_F64_FX");
+                      "storage must be LBM_STORE_F64, LBM_STORE_F64_FX or LBM_STORE_F64_DP");
         return LBM_ERR_UNSUPPORTED;
     }
     lbm_batch* b = new (std::nothrow) lbm_batch();

@@ -2484,7 +2484,7 @@ cudaError_t launch_near(int storage, const void* src, void* dst, const Launch& L
 }
 bool sweep_fused(const Launch& L, int bulk_mode) {
     return L.cp.np > 0 && (L.cp.kind == 1 || L.cp.kind == 2) && !L.nostream &&
-           (bulk_mode == 0 || bulk_mode == 1 || bulk_mode == 3) && L.g.n <= SWEEP_FUSED_CELLS;
+           (bulk_mode == 0 || bulk_mode == 1) && L.g.n <= SWEEP_FUSED_CELLS;
 }
 bool sweep_beside(const Launch& L, int bulk_mode, int sms) {
     const long long blocks = (long long)L.g.ntx * L.g.nty * L.g.ntz;

@@ -229,6 +229,14 @@ inline Coll<C> make_coll(double lp, double lm, double rho0, const double fe[3]) 
     return k;
 }
 
+// FP64 collision constants of a storage mode: LBM_STORE_F64_DP has no
+// fixed-point form, so every cell takes the FP64 one.
+inline Coll<double> make_coll_f64(int storage, double lp, double lm, double rho0, const double fe[3]) {
+    Coll<double> k = make_coll<double>(lp, lm, rho0, fe);
+    if (storage == LBM_STORE_F64_DP) k.fix.on = 0;
+    return k;
+}
+
 // Checks of a configuration shared by every entry point that takes one
 // (lbm_create, lbm_sweep_noalloc): LBM_ERR_ARG for a value outside its
 // range, LBM_ERR_UNSUPPORTED for MEM MR within 0.01 of Lambda_- = 1/2.
@@ -240,7 +248,7 @@ inline lbm_status check_config(const lbm_config& c) {
         return LBM_ERR_ARG;
     if (c.coupling < 0 || c.coupling > LBM_NONE) return LBM_ERR_ARG;
     if (c.collision != LBM_BGK && c.collision != LBM_TRT) return LBM_ERR_ARG;
-    if (c.storage < LBM_STORE_F64 || c.storage > LBM_STORE_BF16S) return LBM_ERR_ARG;
+    if (c.storage < LBM_STORE_F64 || c.storage > LBM_STORE_F64_DP) return LBM_ERR_ARG;
     if (c.bc_z < 0 || c.bc_z > 2 || (c.bc_z == 2 && c.nz < 3)) return LBM_ERR_ARG;
     if (c.bc_z == 2 && !(std::isfinite(c.inflow[0]) && std::isfinite(c.inflow[1]) &&
                          std::isfinite(c.inflow[2]) && c.rho_out > 0.0 && std::isfinite(c.rho_out)))
@@ -300,8 +308,7 @@ static_assert((int)ST_TOO_MANY_OBJECTS == (int)LBM_STATUS_TOO_MANY_OBJECTS &&
 
 // storage: 0 = FP64, 1 = FP32 (arithmetic in the same precision), 4 = FP16
 // and 5 = BF16 shifted populations f - w_q (FP32 arithmetic); launch_bulk
-// also takes 2 = FP64 storage with float-float collision and 3 = FP64
-// storage with 64-bit fixed-point collision
+// also takes 2 = FP64 storage with float-float collision
 cudaError_t launch_bulk(int storage, const void* src, void* dst, const Launch& L);
 cudaError_t launch_near(int storage, const void* src, void* dst, const Launch& L);
 // Whether a sweep runs as one launch (launch_sweep: near and bulk cells), and the

@@ -104,7 +104,7 @@ extern "C" lbm_status lbm_sweep_noalloc(const lbm_config* cfg, const double* src
             return st;
         }
     }
-    if (cfg->storage != LBM_STORE_F64) {
+    if (cfg->storage != LBM_STORE_F64 && cfg->storage != LBM_STORE_F64_DP) {
         set_err(err, err_len, "lbm_sweep_noalloc takes FP64 PDF buffers only");
         return LBM_ERR_UNSUPPORTED;
     }
@@ -198,7 +198,7 @@ extern "C" lbm_status lbm_sweep_noalloc(const lbm_config* cfg, const double* src
     const double lp = -1.0 / cfg->tau;
     const double lm =
         cfg->collision == LBM_TRT ? 1.0 / (cfg->magic / (0.5 + 1.0 / lp) - 0.5) : lp;
-    L.kd = make_coll<double>(lp, lm, cfg->rho0, cfg->force_density);
+    L.kd = make_coll_f64(cfg->storage, lp, lm, cfg->rho0, cfg->force_density);
     const bool psm = cfg->coupling <= LBM_PSM_M3B2;
     L.cp.kind = !coupled ? 0 : (psm ? 1 : 2);
     L.cp.variant = psm ? cfg->coupling - LBM_PSM_M1B1 : cfg->coupling - LBM_MEM_BB;
