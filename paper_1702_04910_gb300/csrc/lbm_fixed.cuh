@@ -11,16 +11,20 @@
 //            their 53-bit significands fit above the unit;
 //   + and -  exact;
 //   *        high half of the 128-bit product from 32-bit limbs, rounded to
-//            nearest, the low x low limb product replaced by its mean: within
-//            0.8 units, unbiased (below);
+//            nearest, the low x low limb product replaced by its mean:
+//            unbiased, within 1 unit of the product by the stored constant,
+//            within 3/4 of a unit of that of two variables (below);
 //   FP64 out the hardware conversion (round to nearest even), exponent moved.
 // A population of a diagonal direction at rest, 1/36, has its last FP64 bit
 // at 2^-58 too; every FP64 operation on rho or j (~1) rounds at 2^-53.  The
-// result is therefore closer to exact arithmetic than the FP64 form's:
-// collided populations against 113-bit arithmetic, relative 2-norm, 5.1e-17
-// (FP64 form 1.9e-16; the correctly rounded result has 4.6e-17), largest
-// error 9.7e-17 of max f (6.9e-16), mean mass error per cell 1e-19 (3e-17),
-// and likewise with a force, BGK, rho0 1.37 and 1000.  A cell with any population outside the
+// result is therefore closer to exact arithmetic than the FP64 form's over the
+// cells of a flow: collided populations against 113-bit arithmetic, tau = 0.6,
+// relative 2-norm, 5.2e-17 (FP64 form 1.9e-16; the correctly rounded result has
+// 4.6e-17), largest error 1.0e-16 of max f (6.8e-16), mean mass error per cell
+// 1e-19 (3e-17), and likewise with a force, BGK, rho0 1.37 and 1000.  The FP64
+// form's error falls as tau grows, to this one's near tau = 6 (FIX_TAU_MAX), and
+// single cells may have the larger error here (0.1 % at tau = 0.6, 14 % at tau = 1
+// with BGK).  A cell with any population outside the
 // range (negative, below 2^-6, more than ~2 to 4 times its rest value,
 // non-finite) or |j| >= rho0/4 is left to the FP64 form (collide_cell), which
 // also reports bad densities.

@@ -42,3 +42,53 @@ def test_filtered_predicates_decide_as_fp64(predicates, n, D):
     out = (ct.c_longlong * 2)()
     predicates.filter_mismatches(n, ct.c_double(D), 100000 if n < 1000 else 40000, 7, out)
     assert list(out) == [0, 0]
+
+
+# ---- the fixed-point collision of FP64 populations against exact arithmetic -----------
+@pytest.fixture(scope="module")
+def collision(tmp_path_factory):
+    lib = build(tmp_path_factory, "collision")
+    lib.constant_product_error.restype = ct.c_double
+    lib.variable_product_error.restype = ct.c_double
+    return lib
+
+
+def lambda_minus(tau, kind):
+    return -1.0 / tau if kind == "BGK" else 1.0 / ((3.0 / 16.0) / (0.5 - tau) - 0.5)
+
+
+@pytest.mark.parametrize("tau", [0.5001, 0.53, 0.6, 0.8, 1.0, 1.5, 4.0])
+@pytest.mark.parametrize("kind", ["BGK", "TRT"])
+def test_fixed_point_products(collision, tau, kind):
+    """By a constant: half a unit of rounding and a low x low limb product below one
+    unit, taken at its mean: one unit.  Of two variables: half a unit and signed low
+    limbs, 2^62 / 2^64: three quarters."""
+    lp, lm = -1.0 / tau, lambda_minus(tau, kind)
+    for c in (-lp / 12, -lp / 36, -lp / 72, -lm / 6, -lm / 12):
+        assert collision.constant_product_error(ct.c_double(c), 100000, 3) <= 1.0
+    assert collision.variable_product_error(100000, 3) <= 0.75
+
+
+@pytest.mark.parametrize("tau", [0.5001, 0.53, 0.8, 1.0, 4.0])
+@pytest.mark.parametrize("kind", ["BGK", "TRT"])
+def test_fixed_point_error_over_a_flow(collision, tau, kind):
+    """Root mean square error over the cells of a flow: below the FP64 form's, and
+    refused cells come back bit for bit."""
+    out = (ct.c_double * 7)()
+    for rho0, fext in ((1.0, (0.0, 0.0, 0.0)), (1.0, (3e-4, -1e-6, 2e-9)),
+                       (1.37, (1e-5, 2e-5, -3e-5)), (0.75, (0.0, 0.0, 0.0))):
+        for noise, drift in ((0.0, 0.1), (0.02, 0.05), (0.1, 0.1), (0.3, 0.1), (1e-4, 1e-3)):
+            collision.collision_errors(ct.c_double(tau), ct.c_double(lambda_minus(tau, kind)),
+                                       ct.c_double(rho0), (ct.c_double * 3)(*fext),
+                                       ct.c_double(noise), ct.c_double(drift), 10000, 11, out)
+            cells, fixed, fp64 = out[0], out[1], out[2]
+            assert cells >= 100 and fixed < fp64, (rho0, fext, noise, drift, list(out))
+
+
+def test_which_modes_collide_in_fixed_point(collision):
+    from paper_1702_04910_gb300.binding import STORAGE
+    for tau in (0.5001, 0.8, 4.0, 4.01, 100.0):
+        t = ct.c_double(tau)
+        assert collision.fixed_point_on(STORAGE["f64"], t) == (tau <= 4.0)
+        assert collision.fixed_point_on(STORAGE["f64fx"], t) == 1
+        assert collision.fixed_point_on(STORAGE["f64dp"], t) == 0
