@@ -87,7 +87,7 @@ typedef enum { LBM_BGK = 0, LBM_TRT = 1 } lbm_collision;
 
 /* PDF storage and collision arithmetic.  Forces, solid fractions and the
  * rigid-body update are FP64 in every mode.
- *   LBM_STORE_F64     FP64 PDFs.  For tau <= 4 the plain fluid collision runs in
+ *   LBM_STORE_F64     FP64 PDFs.  For tau <= 2 the plain fluid collision runs in
  *                     64-bit fixed point on the integer pipes (unit 2^-58 of
  *                     the power of two nearest to rho0; exact sums, products
  *                     within one unit) where the cell's populations and
@@ -95,10 +95,10 @@ typedef enum { LBM_BGK = 0, LBM_TRT = 1 } lbm_collision;
  *                     (populations that are negative, tiny or several times
  *                     their rest value, non-finite values, |j| >= rho0/4).
  *                     Over the cells of a flow its root mean square error
- *                     against exact arithmetic is 0.2 to 0.93 of FP64's (tau
- *                     0.5001 to 4, BGK and TRT, with and without a force); in a
- *                     single cell it can be the larger one (0.1 % of them at
- *                     tau = 0.6, a quarter at tau = 4 with BGK).  Coupling terms
+ *                     against exact arithmetic is 0.1 to 0.66 of FP64's (tau
+ *                     0.5001 to 2, BGK and TRT, with and without a force); in a
+ *                     single cell it can be the larger one (up to 2 % of them
+ *                     at tau <= 0.8, a third at tau = 1.5).  Coupling terms
  *                     (solid fractions, links) and cells that they change use
  *                     FP64; other cells near particles collide as the rest.
  *   LBM_STORE_F32     FP32 PDFs, FP32 collision arithmetic.
@@ -108,7 +108,7 @@ typedef enum { LBM_BGK = 0, LBM_TRT = 1 } lbm_collision;
  *                     FP64 with integer operations); cells near particles
  *                     as with LBM_STORE_F64.  Same state layout.
  *   LBM_STORE_F64_FX  as LBM_STORE_F64, with the fixed-point collision at any tau
- *                     (above 4 its error is up to 1.06 of FP64's).
+ *                     (above 2 its error is up to 1.06 of FP64's).
  *   LBM_STORE_F16S    PDFs stored as FP16 shifted populations f_q - w_q, FP32
  *                     collision arithmetic (76 B per cell update).
  *   LBM_STORE_BF16S   the same with BF16 storage.

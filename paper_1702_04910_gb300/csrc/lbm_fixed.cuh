@@ -22,9 +22,9 @@
 // relative 2-norm, 5.2e-17 (FP64 form 1.9e-16; the correctly rounded result has
 // 4.6e-17), largest error 1.0e-16 of max f (6.8e-16), mean mass error per cell
 // 1e-19 (3e-17), and likewise with a force, BGK, rho0 1.37 and 1000.  The FP64
-// form's error falls as tau grows, to this one's near tau = 6 (FIX_TAU_MAX), and
-// single cells may have the larger error here (0.1 % at tau = 0.6, 14 % at tau = 1
-// with BGK).  A cell with any population outside the
+// form's error falls as tau grows, to this one's near tau = 6 (FIX_TAU_MAX stays
+// below that), and single cells may have the larger error here (0.1 % at tau =
+// 0.6, 14 % at tau = 1 with BGK).  A cell with any population outside the
 // range (negative, below 2^-6, more than ~2 to 4 times its rest value,
 // non-finite) or |j| >= rho0/4 is left to the FP64 form (collide_cell), which
 // also reports bad densities.

@@ -230,10 +230,10 @@ inline Coll<C> make_coll(double lp, double lm, double rho0, const double fe[3]) 
 }
 
 // FP64 collision constants of a storage mode.  The fixed-point form is left out in
-// LBM_STORE_F64_DP, and above tau = 4 unless LBM_STORE_F64_FX asks for it: root mean
-// square error over that of the FP64 form, largest of 20 flows, BGK: tau = 3 0.91,
-// 4 0.93, 6 1.05, 8 1.06 (TRT stays below 1).
-constexpr double FIX_TAU_MAX = 4.0;
+// LBM_STORE_F64_DP, and above tau = 2 unless LBM_STORE_F64_FX asks for it: root mean
+// square error over that of the FP64 form, largest of 20 flows, BGK: tau = 2 0.66, 3
+// 0.91, 4 0.93, 6 1.05, 8 1.06 (TRT stays below 1).
+constexpr double FIX_TAU_MAX = 2.0;
 inline Coll<double> make_coll_f64(int storage, double lp, double lm, double rho0, const double fe[3]) {
     Coll<double> k = make_coll<double>(lp, lm, rho0, fe);
     if (storage == LBM_STORE_F64_DP || (storage != LBM_STORE_F64_FX && lp > -1.0 / FIX_TAU_MAX))

@@ -57,7 +57,7 @@ def lambda_minus(tau, kind):
     return -1.0 / tau if kind == "BGK" else 1.0 / ((3.0 / 16.0) / (0.5 - tau) - 0.5)
 
 
-@pytest.mark.parametrize("tau", [0.5001, 0.53, 0.6, 0.8, 1.0, 1.5, 4.0])
+@pytest.mark.parametrize("tau", [0.5001, 0.53, 0.6, 0.8, 1.0, 1.5, 2.0])
 @pytest.mark.parametrize("kind", ["BGK", "TRT"])
 def test_fixed_point_products(collision, tau, kind):
     """By a constant: half a unit of rounding and a low x low limb product below one
@@ -69,7 +69,7 @@ def test_fixed_point_products(collision, tau, kind):
     assert collision.variable_product_error(100000, 3) <= 0.75
 
 
-@pytest.mark.parametrize("tau", [0.5001, 0.53, 0.8, 1.0, 4.0])
+@pytest.mark.parametrize("tau", [0.5001, 0.53, 0.8, 1.0, 2.0])
 @pytest.mark.parametrize("kind", ["BGK", "TRT"])
 def test_fixed_point_error_over_a_flow(collision, tau, kind):
     """Root mean square error over the cells of a flow: below the FP64 form's, and
@@ -87,8 +87,8 @@ def test_fixed_point_error_over_a_flow(collision, tau, kind):
 
 def test_which_modes_collide_in_fixed_point(collision):
     from paper_1702_04910_gb300.binding import STORAGE
-    for tau in (0.5001, 0.8, 4.0, 4.01, 100.0):
+    for tau in (0.5001, 0.8, 2.0, 2.01, 100.0):
         t = ct.c_double(tau)
-        assert collision.fixed_point_on(STORAGE["f64"], t) == (tau <= 4.0)
+        assert collision.fixed_point_on(STORAGE["f64"], t) == (tau <= 2.0)
         assert collision.fixed_point_on(STORAGE["f64fx"], t) == 1
         assert collision.fixed_point_on(STORAGE["f64dp"], t) == 0
