@@ -5,7 +5,7 @@ workload (D = 24, density ratio 1.5, Galileo number 144, closed top and bottom).
 One benchmark step is one global time step of each coupling variant that
 stays stable for a freely settling sphere (PSM M1B1, M2B2: one LBM sweep each;
 MEM BB, CLI, MR: two LBM sweeps each, with refilling), each in its own simulation,
-FP64 PDFs and arithmetic.  MLUPS counts every lattice cell of every sweep.
+FP64 PDFs (storage f64).  MLUPS counts every lattice cell of every sweep.
 (PSM M3B2 runs the same kernel; as printed, with an explicit rigid-body
 update, it diverges for a free sphere, so it is not part of the timed step.)
 
@@ -138,6 +138,20 @@ def job_mlups(world: int, cells: int, sweeps_per_step: int, steps: int, seconds:
     return world * cells * sweeps_per_step * steps / seconds / 1e6
 
 
+FUSED_CELLS = 1 << 18  # FP64 sweeps up to here are one launch (SWEEP_FUSED_CELLS)
+
+
+def unprofiled_launches(profs, cells: int) -> int:
+    """Kernel launches of unprofiled steps, from the counts of as many profiled ones:
+    the force total takes the rigid-body update with it, and up to FUSED_CELLS cells
+    the near and the bulk sweep are one launch."""
+    total = sum(v[1] for p in profs for v in p.values())
+    total -= sum(p["rigid_body"][1] for p in profs)
+    if cells <= FUSED_CELLS:
+        total -= sum(p["near"][1] for p in profs)
+    return total
+
+
 def workload(coupling: str, scale: float):
     from paper_1702_04910_gb300 import workloads as W
     if scale == 1.0:
@@ -162,7 +176,7 @@ def near_cells(particle, shape, halo=2.0):
     return int(count)
 
 
-def run_ensemble(args, stream, world, dist, barrier, peak, storages=("f64", "f64fx")):
+def run_ensemble(args, stream, world, dist, barrier, peak, storages=("f64", "f64dp")):
     """The batched ensemble: 64 independent settling cases of uneven size and
     Galileo number advanced by one captured step graph per global step."""
     import numpy as np
@@ -408,8 +422,8 @@ def trajectory(case, storage, steps, stream, every=50, profile=False):
     """Release the sphere of `case` and advance it `steps` global steps in
     `storage`; sample the particle's vertical velocity and the vertical
     hydrodynamic force every `every` steps.  Returns (t, u_z, F_z, ms, bulk)
-    with ms the CUDA-event time of the run and bulk the mean bulk-sweep
-    launch time when profiling."""
+    with ms the CUDA-event time of the run and, with `profile`, bulk the mean
+    bulk-sweep launch time of 20 further steps."""
     import numpy as np
     import torch
 
@@ -419,7 +433,6 @@ def trajectory(case, storage, steps, stream, every=50, profile=False):
     s = Simulation(case["shape"], stream=stream, storage=storage, **W.sim_kwargs(case))
     s.set_particles(case["particles"])
     s.init_equilibrium()
-    lbm_profile_enable(s.h, profile)
     t, uz, fz = [], [], []
     torch.cuda.synchronize()
     ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -444,6 +457,8 @@ def trajectory(case, storage, steps, stream, every=50, profile=False):
     ms = ev0.elapsed_time(ev1)
     bulk = None
     if profile and failed is None:
+        lbm_profile_enable(s.h, True)
+        s.step(20)
         prof = lbm_profile_read(s.h)
         bulk = prof["bulk"][0] / max(prof["bulk"][1], 1)
     s.close()
@@ -454,7 +469,8 @@ def trajectory(case, storage, steps, stream, every=50, profile=False):
 
 def settling_errors(make_case, couplings, modes, duration, stream, speed=False, peak=None):
     """Per storage mode: relative error of the settling velocity and of the
-    hydrodynamic force against the FP64 run of the same released sphere,
+    hydrodynamic force against the run of the same released sphere in FP64
+    arithmetic throughout (storage f64dp),
     as means over the last third of `duration` lattice time units after
     release (MEM: duration/2 global steps of two sweeps), plus the largest
     sampled velocity deviation in that window."""
@@ -463,20 +479,20 @@ def settling_errors(make_case, couplings, modes, duration, stream, speed=False, 
                "settling_velocity_rel_err_vs_f64": {}, "settling_velocity_max_rel_dev_vs_f64": {},
                "force_rel_err_vs_f64": {}} for m in modes}
     info = {}
-    esize = {"f64": 8, "f64fx": 8, "f64ff": 8, "f32": 4, "f16s": 2, "bf16s": 2}
+    esize = {"f64": 8, "f64ff": 8, "f32": 4, "f16s": 2, "bf16s": 2}
     for cp in couplings:
         case = make_case(cp)
         nc = int(np.prod(case["shape"]))
         steps = duration // sweeps_of(cp)
-        runs = {m: trajectory(case, m, steps, stream, profile=speed) for m in ["f64"] + list(modes)}
-        t, u64, f64_, ms64, _, fail64 = runs["f64"]
+        runs = {m: trajectory(case, m, steps, stream, profile=speed) for m in ["f64dp"] + list(modes)}
+        t, u64, f64_, ms64, _, fail64 = runs["f64dp"]
         if fail64:
-            info[cp] = {"f64_failed": fail64}
+            info[cp] = {"f64dp_failed": fail64}
             continue
         win = t > steps - steps // 3
         ubar, fbar = u64[win].mean(), f64_[win].mean()
-        info[cp] = {"f64_settling_velocity": float(ubar), "f64_force_z": float(fbar),
-                    "f64_MLUPS": nc * sweeps_of(cp) * steps / (ms64 * 1e-3) / 1e6}
+        info[cp] = {"f64dp_settling_velocity": float(ubar), "f64dp_force_z": float(fbar),
+                    "f64dp_MLUPS": nc * sweeps_of(cp) * steps / (ms64 * 1e-3) / 1e6}
         for m in modes:
             _, um, fm, msm, bulk, failm = runs[m]
             o = out[m]
@@ -488,12 +504,12 @@ def settling_errors(make_case, couplings, modes, duration, stream, speed=False, 
             o["force_rel_err_vs_f64"][cp] = float(abs(fm[win].mean() - fbar) / abs(fbar))
             if speed:
                 o.setdefault("MLUPS", {})[cp] = nc * sweeps_of(cp) * steps / (msm * 1e-3) / 1e6
-                o.setdefault("speedup_vs_f64", {})[cp] = ms64 / msm
+                o.setdefault("speedup_vs_f64dp", {})[cp] = ms64 / msm
                 near = near_cells(case["particles"][0], case["shape"])
                 gbps = 2 * 19 * esize[m] * (nc - near) / (bulk * 1e-3) / 1e9
                 o.setdefault("bulk_GBps", {})[cp] = gbps
                 o.setdefault("frac", {})[cp] = gbps / peak
-    out["f64"] = info
+    out["f64dp"] = info
     if speed:
         shape = make_case(couplings[0])["shape"]
         out["workload"] = (f"settling sphere D=36, Ga=250 (nu=0.01), {shape[0]}x{shape[1]}x{shape[2]}, "
@@ -557,14 +573,16 @@ def run_ours(args):
         for s in sims:
             s.step(1)
     with ClockSampler(local) as clk:
-        ms, profs = timed(sims, args.steps, True)
+        ms, _ = timed(sims, args.steps, False)
     clocks = clk.summary()
+    # a second window for the kernels' times: profiling takes launches apart
+    _, profs = timed(sims, args.steps, True)
     value = job_mlups(world, ncell, sweeps_per_step, args.steps, ms * 1e-3)
 
     # dominant kernel: the bulk sweep (events recorded on the library's stream)
     bulk_ms = sum(p["bulk"][0] for p in profs)
     bulk_n = sum(p["bulk"][1] for p in profs)
-    launches = sum(sum(v[1] for v in p.values()) for p in profs)
+    launches = unprofiled_launches(profs, ncell)
     share = {k: sum(p[k][0] for p in profs) for k in PROFILE_CLASSES}
     tot = sum(share.values())
     parts_now = [s.get_particles()[0] for s in sims]
@@ -577,6 +595,8 @@ def run_ours(args):
     # end-to-end through the C ABI with host buffers: per step, the particle
     # state goes host -> device and forces + particle state come back
     e2e_sims = sims
+    for s in e2e_sims:
+        lbm_profile_enable(s.h, False)
     h2d = d2h = 0
     barrier()
     t0 = time.perf_counter()
@@ -592,26 +612,27 @@ def run_ours(args):
     e2e_s = max_over_ranks(time.perf_counter() - t0, dist, "cuda")
     e2e_value = job_mlups(world, ncell, sweeps_per_step, args.steps, e2e_s)
 
-    # FP64 storage with the collision of cells away from particles in
-    # float-float or 64-bit fixed-point arithmetic, FP32 and shifted 16-bit
+    # FP64 storage with FP64 arithmetic in every cell (the yardstick of the errors
+    # below) or float-float away from particles, FP32 and shifted 16-bit
     # storage: speed of the same timed step
     variants = {}
     for s in sims:
         s.close()
     sims = []
-    what = {"f64ff": (8, "float-float (2 x FP32) collision away from particles, FP64 elsewhere"),
-            "f64fx": (8, "64-bit fixed-point (2^-58) collision away from particles, FP64 elsewhere"),
+    what = {"f64ff": (8, "float-float (2 x FP32) collision away from particles"),
+            "f64dp": (8, "FP64 in every cell"),
             "f32": (4, "FP32 PDFs, FP32 collision"),
             "f16s": (2, "FP16 shifted populations f - w_q, FP32 collision"),
             "bf16s": (2, "BF16 shifted populations f - w_q, FP32 collision")}
-    modes = [] if args.no_fp32 else ["f64fx", "f64ff", "f32", "f16s", "bf16s"]
+    modes = [] if args.no_fp32 else ["f64dp", "f64ff", "f32", "f16s", "bf16s"]
     for mode in modes:
         esize, desc = what[mode]
         simsm = build(mode)
         for _ in range(args.warmup):
             for s in simsm:
                 s.step(1)
-        msm, profsm = timed(simsm, args.steps, True)
+        msm, _ = timed(simsm, args.steps, False)
+        _, profsm = timed(simsm, args.steps, True)
         vm = job_mlups(world, ncell, sweeps_per_step, args.steps, msm * 1e-3)
         bm = sum(p["bulk"][0] for p in profsm) / sum(p["bulk"][1] for p in profsm)
         achm = 2 * 19 * esize * bulk_cells / (bm * 1e-3) / 1e9
@@ -622,22 +643,22 @@ def run_ours(args):
                           "bulk_avg_launch_ms": bm, "algorithmic_bytes_per_cell": 2 * 19 * esize,
                           "arithmetic": desc}
 
-    # settling-velocity and force error of each mode against the FP64 run of
-    # the same case, as windowed means after release (the metric's "force /
+    # settling-velocity and force error of each mode against the run in FP64
+    # arithmetic of the same case, as windowed means after release (the metric's "force /
     # velocity error vs FP64"), on this workload and on the D = 36, Ga = 250
     # case in 192 x 192 x 768
     if args.acc_time > 0 and modes:
-        acc_modes = [m for m in modes if m != "f64ff"]
+        acc_modes = ["f64"] + [m for m in modes if m not in ("f64ff", "f64dp")]
         acc = settling_errors(lambda cp: workload(cp, args.scale), args.couplings, acc_modes,
                               args.acc_time, stream)
-        variants["settling_f64_reference"] = acc.pop("f64")
+        variants["settling_f64dp_reference"] = acc.pop("f64dp")
         for mode in acc_modes:
-            variants[mode].update(acc[mode])
+            variants.setdefault(mode, {}).update(acc[mode])
     if args.d36_time > 0 and not args.no_fp32:
         variants["settling_d36_ga250"] = settling_errors(
             lambda cp: W.settling_sphere(D=36.0, shape=(192, 192, 768), ga=250.0,
                                          drop_below_top=64.0, coupling=cp),
-            ("PSM_M2B2", "MEM_CLI"), ["f64fx", "f16s", "bf16s"], args.d36_time, stream,
+            ("PSM_M2B2", "MEM_CLI"), ["f64", "f16s", "bf16s"], args.d36_time, stream,
             speed=True, peak=peak)
 
     if not args.no_ensemble:
@@ -692,14 +713,14 @@ def run_ours(args):
                        # MEM's two sweeps counted once): value x couplings / sweeps
                        "mlups_per_global_step": value * len(args.couplings) / sweeps_per_step,
                        "collision": "TRT (Lambda=3/16)",
-                       "precision": "FP64 PDFs; 64-bit fixed-point collision of cells away from "
-                                    "particles (closer to exact than FP64), FP64 elsewhere; FP64 forces "
-                                    "and rigid-body update",
+                       "precision": "FP64 PDFs; 64-bit fixed-point collision (root mean square error "
+                                    "below FP64's), FP64 coupling, forces and rigid-body update",
                        "l2": "inputs larger than L2 (2.55 GB of PDFs per simulation)",
                        "replicas_per_rank": 1},
             "roofline": roofline,
             "kernel_time_share": {k: (v / tot if tot else 0.0) for k, v in share.items()},
-            "kernel_time_share_note": "CUDA-event time per class; the near sweep runs on its own "
+            "kernel_time_share_note": "CUDA-event time per class in a second window of as many steps "
+                                      "with profiling on; the near sweep runs on its own "
                                       "stream beside the bulk sweep, so its time includes the overlap",
             "e2e": {"value": e2e_value, "unit": "MLUPS", "h2d_bytes_per_step": h2d // args.steps,
                     "d2h_bytes_per_step": d2h // args.steps,
@@ -832,7 +853,7 @@ def main():
                          "runs (errors are windowed means over the last third; 0 skips them)")
     ap.add_argument("--d36-time", type=int, default=2000,
                     help="lattice time units of the D = 36, Ga = 250 settling case (192x192x768) "
-                         "run in FP64, F64_FX, FP16 and BF16 shifted storage (0 skips it)")
+                         "run in FP64 arithmetic, F64, FP16 and BF16 shifted storage (0 skips it)")
     ap.add_argument("--cpu-sample-steps", type=int, default=1)
     ap.add_argument("--no-fp32", action="store_true")
     ap.add_argument("--no-cpu-baseline", action="store_true")
@@ -840,7 +861,7 @@ def main():
     ap.add_argument("--ensemble-cases", type=int, default=64)
     ap.add_argument("--ensemble-only", action="store_true",
                     help="time only the batched ensemble (one JSON object of variants)")
-    ap.add_argument("--ensemble-storage", default="f64,f64fx")
+    ap.add_argument("--ensemble-storage", default="f64,f64dp")
     ap.add_argument("--learned", choices=("small", "full", "none"), default="small",
                     help="learned force correction study reported as a variant")
     ap.add_argument("--learned-only", action="store_true")
@@ -856,7 +877,7 @@ def main():
                     help="LBM sweeps per step of every coupling in the frame, forces averaged "
                          "(Sec. 4.1: 2)")
     ap.add_argument("--frame-storage", default="f64fx",
-                    choices=("f64", "f64fx", "f64ff", "f32", "f16s", "bf16s"))
+                    choices=("f64", "f64fx", "f64ff", "f64dp", "f32", "f16s", "bf16s"))
     ap.add_argument("--lab-drag", action="store_true",
                     help="drag of a fixed sphere in an inflow against a sphere translating "
                          "through fluid at rest at the same relative speed (D = 24)")
@@ -869,13 +890,13 @@ def main():
                          "and report wall contact and stability")
     ap.add_argument("--full-steps", type=int, default=20000)
     ap.add_argument("--full-storage", default="f64fx",
-                    choices=("f64", "f64fx", "f64ff", "f32", "f16s", "bf16s"))
+                    choices=("f64", "f64fx", "f64ff", "f64dp", "f32", "f16s", "bf16s"))
     ap.add_argument("--scale", type=float, default=1.0,
                     help="shrink the settling workload by this factor in every length (tests)")
     ap.add_argument("--case-shape", default=None,
                     help="run a single small profiling case of this shape (e.g. 128x128x256)")
     ap.add_argument("--case-storage", default="f64",
-                    choices=("f64", "f32", "f64ff", "f64fx", "f16s", "bf16s"))
+                    choices=("f64", "f32", "f64ff", "f64fx", "f64dp", "f16s", "bf16s"))
     args = ap.parse_args()
     args.frame_couplings = FRAME_COUPLINGS
     if args.couplings is None:

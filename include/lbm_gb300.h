@@ -248,7 +248,13 @@ lbm_status lbm_synchronize(lbm_handle *h);
  * (0 bulk sweep, 1 near-particle sweep, 2 force reduction, 3 rigid-body
  * update, 4 MEM refill, 5 other: per-step geometry map and set-up
  * collisions), the summed milliseconds and launches.
- * Reading synchronises the stream. */
+ * Reading synchronises the stream.
+ * A profiled handle takes launches apart that run merged or overlapped
+ * otherwise, with an event before and after each: the near-particle sweep runs
+ * on a second stream, never in one launch with the bulk sweep or beside it on
+ * one stream, and the force total and the rigid-body update are two launches.
+ * The classes' times are those of that form, and its steps take longer: time
+ * steps with profiling off. */
 lbm_status lbm_profile_enable(lbm_handle *h, int enable);
 lbm_status lbm_profile_read(lbm_handle *h, int n_classes, double *ms, long long *launches);
 

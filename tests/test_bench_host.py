@@ -43,3 +43,12 @@ def test_near_cells_of_the_settling_workload():
     centre)."""
     p = {"x": (64.0, 64.0, 448.0), "diameter": 24.0}
     assert bench.near_cells(p, (128, 128, 512)) == 28 ** 3 == _brute_force(p, (128, 128, 512))
+
+
+def test_launches_of_unprofiled_steps():
+    """Two steps of a MEM handle (two sweeps each): map, near and bulk twice, force
+    total with the rigid body, refill; near and bulk in one launch on a small lattice."""
+    prof = {"bulk": (1.0, 4), "near": (1.0, 4), "force_total": (1.0, 2), "rigid_body": (1.0, 2),
+            "refill": (1.0, 2), "other": (1.0, 2)}
+    assert bench.unprofiled_launches([prof, prof], 128 * 128 * 512) == 2 * 14
+    assert bench.unprofiled_launches([prof], 24 * 24 * 40) == 10
