@@ -206,9 +206,9 @@ __device__ __forceinline__ void shifted_rt(const Nbr& b, int x, int y, int z, in
 // bit Q of `cut`, filled by the link loop.
 template <typename T, typename C, int Q>
 __device__ __forceinline__ void mem_pull_one(const T* __restrict__ src, const Geom& g,
-                                             const DevParticle* parts, int np, const GeoMap* gm,
-                                             const Nbr& b, int x, int y, int z, long long idx,
-                                             C (&f)[NQ], unsigned& cut, int* status) {
+                                             const DevParticle* parts, int np, const Nbr& b, int x,
+                                             int y, int z, long long idx, C (&f)[NQ], unsigned& cut,
+                                             int* status) {
     constexpr int QP = opp(Q);
     int xs, ys, zs;
     shifted<Q>(b, x, y, z, -1, xs, ys, zs);
@@ -216,7 +216,7 @@ __device__ __forceinline__ void mem_pull_one(const T* __restrict__ src, const Ge
         f[Q] = PdfStore<T>::template load<C>(src + (long long)QP * g.n + idx, QP);
         return;
     }
-    const int owner = owner_of(g, parts, np, gm, xs, ys, zs);
+    const int owner = cell_owner(g, parts, np, xs, ys, zs);
     // index checks: a failure is reported (ST_BOUNDS) and the access skipped
     if (!owner) {
         if (xs < 0 || xs >= g.nx || ys < 0 || ys >= g.ny || zs < 0 || zs >= g.nz) {
@@ -238,19 +238,18 @@ __device__ __forceinline__ void mem_pull_one(const T* __restrict__ src, const Ge
 template <typename T, typename C, int Q>
 struct MemPull {
     __device__ __forceinline__ static void run(const T* __restrict__ src, const Geom& g,
-                                               const DevParticle* parts, int np, const GeoMap* gm,
-                                               const Nbr& b, int x, int y, int z, long long idx,
-                                               C (&f)[NQ], unsigned& cut, int* status) {
-        mem_pull_one<T, C, Q>(src, g, parts, np, gm, b, x, y, z, idx, f, cut, status);
-        MemPull<T, C, Q + 1>::run(src, g, parts, np, gm, b, x, y, z, idx, f, cut, status);
+                                               const DevParticle* parts, int np, const Nbr& b, int x,
+                                               int y, int z, long long idx, C (&f)[NQ],
+                                               unsigned& cut, int* status) {
+        mem_pull_one<T, C, Q>(src, g, parts, np, b, x, y, z, idx, f, cut, status);
+        MemPull<T, C, Q + 1>::run(src, g, parts, np, b, x, y, z, idx, f, cut, status);
     }
 };
 template <typename T, typename C>
 struct MemPull<T, C, NQ> {
     __device__ __forceinline__ static void run(const T* __restrict__, const Geom&,
-                                               const DevParticle*, int, const GeoMap*, const Nbr&,
-                                               int, int, int, long long, C (&)[NQ], unsigned&,
-                                               int*) {}
+                                               const DevParticle*, int, const Nbr&, int, int, int,
+                                               long long, C (&)[NQ], unsigned&, int*) {}
 };
 
 // Phase 2: the boundary value f_q(x, t+1) of one cut link (q filled at x,
@@ -377,27 +376,21 @@ struct MemMerge<C, NQ> {
 // loop over them (phase 2, one copy of the link code, links in increasing q).
 template <typename T, typename C>
 __device__ __forceinline__ void mem_pull(const T* __restrict__ src, const Geom& g, const Coupl& cp,
-                                         const DevParticle* parts, int np, const GeoMap* gm,
-                                         int x, int y, int z, long long idx, C (&f)[NQ],
-                                         Slots* slots, int* status) {
+                                         const DevParticle* parts, int np, int x, int y, int z,
+                                         long long idx, C (&f)[NQ], int* status) {
     Nbr b = make_nbr(g, x, y, z);
     f[0] = PdfStore<T>::template load<C>(src + idx, 0);
     unsigned cut = 0;
-    MemPull<T, C, 1>::run(src, g, parts, np, gm, b, x, y, z, idx, f, cut, status);
+    MemPull<T, C, 1>::run(src, g, parts, np, b, x, y, z, idx, f, cut, status);
     if (cut) {
         double lv[NQ];
         MrCell mc;
         mc.have = false;
         for (unsigned m = cut; m; m &= m - 1) {
             const int q = __ffs(m) - 1;
-            double ft[6];
             int owner = 0;
-            lv[q] = mem_link(src, g, cp, parts, np, gm, b, x, y, z, idx, q, slots ? ft : nullptr,
-                             &owner, status, mc);
-            if (slots && owner) {
-                const double F[3] = {ft[0], ft[1], ft[2]}, Tq[3] = {ft[3], ft[4], ft[5]};
-                if (!slots->add(owner - 1, F, Tq)) atomicOr(status, ST_TOO_MANY_OBJECTS);
-            }
+            lv[q] = mem_link(src, g, cp, parts, np, (const GeoMap*)nullptr, b, x, y, z, idx, q,
+                             (double*)nullptr, &owner, status, mc);
         }
         MemMerge<C, 1>::run(cut, lv, f);
     }
@@ -1168,16 +1161,6 @@ __device__ __forceinline__ void near_block(const T* __restrict__ src, T* __restr
         atomicOr(status, ST_BOUNDS);
         active = false;
     }
-    if (KIND == 2 && NOSTREAM && active) {
-        // MEM with no stream (first sweep after set-up): fluid cells collide
-        if (!map_at(gm, p, kx, ky, kz)) {
-            const long long idx = lin(g, x, y, z);
-            C f[NQ];
-            load_own(src, g, idx, f);
-            if (collide_cell(f, k)) atomicOr(status, ST_FLUID);
-            store_own(dst, g, idx, f);
-        }
-    }
     if (KIND != 2) {
         C f[NQ];
         int nobj = 0;
@@ -1224,7 +1207,7 @@ __device__ __forceinline__ void near_block(const T* __restrict__ src, T* __restr
         }
         if (active) store_own(dst, g, idx, f);
     }
-    if constexpr (KIND == 2 && !NOSTREAM) {
+    if constexpr (KIND == 2) {
         // MEM (Sec. 2.2): solid cells are not updated; every lane of the warp
         // takes part in the link loop, cells or not
         C f[NQ];
@@ -1246,7 +1229,7 @@ __device__ __forceinline__ void near_block(const T* __restrict__ src, T* __restr
             store_own(dst, g, idx, f);
         }
     }
-    if (KIND == 0 || (NOSTREAM && KIND == 2)) return;
+    if (KIND == 0) return;
     // fixed-order reduction of this block's contribution for each particle
     const bool any = __any_sync(0xffffffffu, slots.id[0] >= 0);
     if (p >= cp.np || blk >= nblk) {
@@ -1723,8 +1706,7 @@ __device__ __forceinline__ void refill_warp(const T* __restrict__ srcB, T* __res
                 double rho = 0.0;
                 if (ok) {
                     C fq[NQ];
-                    mem_pull(srcB, g, cp, so, cp.np, (const GeoMap*)nullptr, xx, yy, zz,
-                             lin(g, xx, yy, zz), fq, (Slots*)nullptr, status);
+                    mem_pull(srcB, g, cp, so, cp.np, xx, yy, zz, lin(g, xx, yy, zz), fq, status);
 #pragma unroll
                     for (int qq = 0; qq < NQ; ++qq) rho += (double)fq[qq];
                 }
@@ -2345,8 +2327,7 @@ cudaError_t bulk_cpt(const void* src, void* dst, const Launch& L) {
     return L.nostream ? go(k_bulk<T, C, true, CPT, false>) : go(k_bulk<T, C, false, CPT, false>);
 }
 
-// FP64-state sweeps are arithmetic bound and use one cell per thread; the
-// 16/32-bit sweeps are memory bound and take two z cells per thread.
+// k_bulk takes two z cells per thread in FP32, one elsewhere.
 template <typename T, typename C = T>
 cudaError_t bulk_t(const void* src, void* dst, const Launch& L) {
     if constexpr (sizeof(T) == 2) {
@@ -2372,10 +2353,7 @@ cudaError_t bulk_t(const void* src, void* dst, const Launch& L) {
                           ZPAIR_THREADS, L.stream, (const T*)src, (T*)dst, L.g, L.kf, L.parts, np,
                           L.status);
     }
-    if constexpr (sizeof(T) <= 4) {
-        if (L.g.tz == 2) return bulk_cpt<T, C, 2>(src, dst, L);
-    }
-    return bulk_cpt<T, C, 1>(src, dst, L);
+    return bulk_cpt<T, C, sizeof(T) == 4 ? 2 : 1>(src, dst, L);  // g.tz of set_tiles
 }
 
 template <typename T, int KIND>
@@ -2388,9 +2366,11 @@ cudaError_t near_kind(const void* src, void* dst, const Launch& L) {
     // 16 bits: not launched ahead of the map's end, where its registers would be
     // held back from the bulk sweep for longer
     constexpr bool early = sizeof(T) > 2;
-    if (L.nostream)
-        return launch_with(early, smem, k_near<T, C, KIND, true>, grid, block, L.stream, (const T*)src,
-                           (T*)dst, L.g, k, L.cp, L.parts, gm, L.partials, L.status, L.gate, L.gate_key);
+    if constexpr (KIND != 2)  // (MEM set-up collides in place: its sweeps always stream)
+        if (L.nostream)
+            return launch_with(early, smem, k_near<T, C, KIND, true>, grid, block, L.stream,
+                               (const T*)src, (T*)dst, L.g, k, L.cp, L.parts, gm, L.partials,
+                               L.status, L.gate, L.gate_key);
     return launch_with(early, smem, k_near<T, C, KIND, false>, grid, block, L.stream, (const T*)src,
                        (T*)dst, L.g, k, L.cp, L.parts, gm, L.partials, L.status, L.gate, L.gate_key);
 }
