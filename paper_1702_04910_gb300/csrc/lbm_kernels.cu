@@ -599,9 +599,10 @@ __device__ inline bool psm_collide(C (&f)[NQ], const Coll<C>& k, const Coupl& cp
 // are the even and odd parts of the change (the solid ones times B_s), and
 // sum_q C_q c_qbar of Eq. (28) is rho0 (U - v) for M1 and M2, twice that for
 // M3.  It is bound by the FP64 pipe: ~300 operations and no arrays over q
-// beside f, 123 registers, against ~700 and 254 of the general form (k_near
-// PSM M1B1 D = 8: 35.1 us -> 25.4 us).  FP32 keeps the general form: its time
-// hides under the bulk sweep, and its results stay the same bits.
+// beside f, 154 registers in k_near, against ~700 and 254 of the general form (k_near
+// PSM M1B1 D = 8: 35.1 us -> 25.4 us).  FP32 keeps the general form (195
+// registers): its time hides under the bulk sweep, though in 16 bits its
+// registers are what that sweep lacks beside it (k_bulk_pair).
 __device__ inline bool psm_collide64(double (&f)[NQ], const Coll<double>& k, const Coupl& cp,
                                      const Geom& g, const DevParticle* parts, int nobj,
                                      const int (&pid)[CELL_SLOTS], const double (&eps)[CELL_SLOTS],
@@ -706,8 +707,8 @@ __device__ inline bool psm_collide64(double (&f)[NQ], const Coll<double>& k, con
 // region touches skip the per-cell test (block-uniform branch).
 // Threads per block and resident blocks per SM of k_bulk by stored type and
 // arithmetic (the host's tiles, set_tiles in lbm_launch.h, follow).  FP64:
-// 5 x 128 threads leave the fixed-point collision its 96 registers without
-// spills and 20 warps per SM (128 x 128 x 512 cells, FP64 settling step of 2
+// 5 x 128 threads leave the fixed-point collision 96 registers (8 B of stack,
+// 4 B of them spills) and 20 warps per SM (128 x 128 x 512 cells, FP64 settling step of 2
 // sweeps: 256 x 3, 80 registers, 1.27 ms; 256 x 2, 128 registers, 1.38;
 // 128 x 4 1.29; 128 x 5 1.09; 128 x 6 1.21; 128 x 7 1.18).  16 bits, one
 // cell per thread: 128 threads balance the last wave better (101 x 101 x 304
@@ -879,7 +880,7 @@ struct PullPair<T, NQ> {
 // cells per row are 96 threads; as two blocks of 64, a quarter of them idle,
 // the BF16 sweep of 192 x 192 x 768 cells took 473 us, 0.67 of HBM, and takes
 // 376 us, 0.85).  One row of 128 cells per 64-thread block: the near-particle sweep runs
-// beside this kernel and each of its one-warp blocks holds 3.4k (MEM) to 6.2k (PSM)
+// beside this kernel and each of its one-warp blocks holds 3.1k (MEM) to 6.2k (PSM)
 // registers; with small bulk blocks an SM that hosts near blocks gives up
 // only as many bulk warps as their registers need (measured in the 128 x 128
 // x 512 step, FP16: 0.70 of HBM with 64 x 4, 0.745 with 64 x 2, 0.76 with
@@ -2154,11 +2155,13 @@ __device__ __forceinline__ bool batch_cell(const Geom& g, int layout, long long 
 // bulk sweep: persistent blocks striding over the 256-cell items of all
 // listed cases.  Each case has its own tiling (B.layout, chosen by the
 // autotuner): 0 box tiles of g.tx x g.ty cells; 1 plane segments.  The case
-// record is staged in shared memory once per item: its collision constants
+// record is staged in shared memory once per run of items of a case: its constants
 // are read ~60 times per cell, and as global loads they cost the registers
 // that the cell's 19 values need (12 cases of D = 8..16, 6.8 M cells, 3 steps:
 // constants from global memory, 256 threads, 1 KB of spills 4.10 ms; staged,
-// 128 threads, 3.87 ms; the FP64 form 10.08 ms).
+// 128 threads, 3.87 ms; the FP64 form 10.08 ms).  As shared-memory operands they
+// still leave 216 B of spills per thread (k_bulk, whose constants are kernel
+// parameters, 4 B): 0.65 to 0.70 of the measured HBM bandwidth.
 __global__ void __launch_bounds__(BATCH_THREADS, BATCH_BLOCKS)
     k_batch_bulk(BatchCase* __restrict__ cases, BatchList l, long long total, int chunk,
                  int* __restrict__ status) {

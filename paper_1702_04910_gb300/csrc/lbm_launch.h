@@ -301,7 +301,7 @@ enum : int {
     ST_DOMAIN = 2,            // a particle left the domain through a closed wall
     ST_REFILL_SOLID = 4,      // refill found no particle owning a cell (internal)
     ST_UNSTABLE = 8,          // a particle state became non-finite or too fast
-    ST_BOUNDS = 16,           // an index check in a coupling kernel failed (access skipped)
+    ST_BOUNDS = 16,           // an index check or a bounded wait failed (access skipped)
     ST_FLUID = 32,            // a fluid cell's density became non-finite or <= 0
 };
 static_assert((int)ST_TOO_MANY_OBJECTS == (int)LBM_STATUS_TOO_MANY_OBJECTS &&
@@ -319,7 +319,8 @@ cudaError_t launch_near(int storage, const void* src, void* dst, const Launch& L
 // largest lattice that does.  us for 20 steps, near sweep on a second stream /
 // one launch: FP64 PSM 32^3 756 / 643, 64^3 964 / 872, 80^3 1400 / 1469; FP64 MEM
 // (two sweeps a step) 32^3 1221 / 1050, 64^3 1777 / 1571, 80^3 2511 / 2476; FP32
-// PSM 64^3 684 / 637, 80^3 793 / 936; FP32 MEM 64^3 1512 / 1257, 80^3 1745 / 1491.
+// PSM 64^3 684 / 637, 80^3 793 / 936; FP32 MEM 64^3 1512 / 1257, 80^3 1745 / 1491
+// (and 1277 beside one another on one stream: sweep_beside).
 constexpr long long SWEEP_FUSED_CELLS = 1 << 18;
 bool sweep_fused(const Launch& L, int bulk_mode);
 // Whether a handle's near and bulk sweeps run beside one another on one stream

@@ -326,7 +326,7 @@ __global__ void __launch_bounds__(PASS_THREADS, 2)
 
 // Parameter gradient: dW[i][o] = sum_s a_s[i] d_s[o], db[o] = sum_s d_s[o],
 // samples in order (a long training run amplifies any other order).  One block
-// per 16 x 16 tile of a weight matrix, two outputs per thread; the tiles of a
+// per 16 x 16 tile of a weight matrix, 2 x 2 outputs per thread; the tiles of a
 // layer's first rows also add its bias.
 //
 // What bounds it: the chain of n dependent FMAs of every output, 4 cycles
